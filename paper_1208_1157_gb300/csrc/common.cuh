@@ -59,6 +59,35 @@ __device__ __forceinline__ double kmul(const F64k &k, double a, double b) { retu
 __device__ __forceinline__ double ksub(const F64k &k, double a, double b) { return fma(b, k.mone, a); }
 __device__ __forceinline__ double kadd(const F64k &k, double a, double b) { return fma(a, k.one, b); }
 
+// A pair of FP32 numbers (ff.cuh), and the coefficients of a Hermite step as pairs
+// (hermite_ff.cuh): in the kernel's parameters, so that they cost no registers.
+struct ff {
+  float h, l;
+};
+struct FCoef {
+  double h;
+  ff f, hh, h2_2, h3_6, h2_12;
+  float fl, hf;  // what f leaves of h; |h|
+};
+inline FCoef fcoef_host(double h) {
+  auto pair = [](double d) {
+    ff r;
+    r.h = (float)d;
+    r.l = (float)(d - (double)r.h);
+    return r;
+  };
+  FCoef C;
+  C.h = h;
+  C.f = pair(h);
+  C.fl = (float)(h - ((double)C.f.h + (double)C.f.l));
+  C.hh = pair(0.5 * h);
+  C.h2_2 = pair(0.5 * h * h);
+  C.h3_6 = pair(h * h * h * (1.0 / 6.0));
+  C.h2_12 = pair(h * h * (1.0 / 12.0));
+  C.hf = (float)(h < 0 ? -h : h);
+  return C;
+}
+
 struct StepParams {
   double t_end, dt;
   int n_corr;            // Hermite corrector passes
@@ -76,6 +105,7 @@ struct StepParams {
   const double *t_end_dev = nullptr;  // end time read from device memory (graph replays)
   double rk_eps = 1e-12;  // error tolerance of the adaptive Runge-Kutta Cash-Karp step
   F64k fk = {0.0, -1.0, 1.0};  // opaque constants (set on the host, never changed)
+  FCoef fc = {};               // coefficients of a step dt (set by the launchers that use them)
   int concurrent = 0;          // host-side hint: other bins' launches overlap this one
 };
 

@@ -669,10 +669,13 @@ static int run_persistent(swarm_ensemble *e, const StepParams &P0, int integrato
       const double span = std::max(std::fabs(P.t_end - e->t_lo), std::fabs(P.t_end - e->t_hi)) / std::fabs(P.dt);
       if (span >= 5000) bin_ctas[i] = 1;
     }
-    // adaptive system per lane: each lane integrates systems one after the other, so the
-    // call ends with lanes waiting for the last ones; one CTA per SM gives every lane
-    // more systems and makes that tail a smaller part of the call
-    if (integrator == SWARM_HERMITE4_ADAPTIVE && m == SWARM_MAP_SYSTEM_PER_LANE && !e->ctas_per_sm) bin_ctas[i] = 1;
+    // adaptive system per lane: the kernel's full residency (131072 x 3 systems over a
+    // quarter of an inner period: 17.1 ms at two CTAs per SM, 28.9 ms at one, whose single
+    // warp per sub-partition leaves both the FP64 and the FP32 pipe waiting); the printed
+    // corrector's steps are FP64, one warp fills that pipe, and one CTA per SM gives every
+    // lane more systems and the call a smaller tail
+    if (integrator == SWARM_HERMITE4_ADAPTIVE && m == SWARM_MAP_SYSTEM_PER_LANE && !e->ctas_per_sm)
+      bin_ctas[i] = P.corr_form ? 1 : 0;
   }
   int rc = build_work(e, maps);
   if (rc) return rc;
@@ -688,7 +691,7 @@ static int run_persistent(swarm_ensemble *e, const StepParams &P0, int integrato
   const int sms = sm_count();
   struct Uni {
     BinView view;
-    int nunits, grid, mapping, variant;
+    int nunits, grid, mapping;
   };
   // the single-bin kernel of one bin for this integrator (grid 0: only the resident
   // blocks per SM into *blocks)
@@ -698,7 +701,7 @@ static int run_persistent(swarm_ensemble *e, const StepParams &P0, int integrato
       if (hermite_family(integrator)) return launch_hermite_wide(u.view, Q, g, st, blocks);
       return launch_mvs_wide(u.view, Q, g, st, blocks);
     }
-    if (hermite_family(integrator)) return launch_hermite_uniform(u.mapping, u.view, u.nunits, Q, g, st, blocks, u.variant);
+    if (hermite_family(integrator)) return launch_hermite_uniform(u.mapping, u.view, u.nunits, Q, g, st, blocks);
     if (rkck_family(integrator)) return launch_rkck_uniform(u.view, u.nunits, Q, g, st, blocks);
     return launch_mvs_uniform(integrator == SWARM_MVS_JACOBI, u.view, u.nunits, Q, g, st, blocks);
   };
@@ -711,7 +714,6 @@ static int run_persistent(swarm_ensemble *e, const StepParams &P0, int integrato
       u.mapping = maps[i];
       u.nunits = units_of(u.view.n, u.view.S, u.mapping);
       int blocks = 0;
-      u.variant = bin_ctas[i] == 3 ? 1 : 0;
       CK(launch_uni(u, P, 0, e->stream, &blocks));
       if (blocks <= 0) return fail(SWARM_ECUDA, "single-bin kernel cannot be resident");
       int c = (bin_ctas[i] && bin_ctas[i] < blocks) ? bin_ctas[i] : blocks;
@@ -724,7 +726,6 @@ static int run_persistent(swarm_ensemble *e, const StepParams &P0, int integrato
       u.view = e->bins[i].view();
       u.mapping = kMapWide;
       u.nunits = u.view.S;
-      u.variant = 0;
       int blocks = 0;
       CK(launch_uni(u, P, 0, e->stream, &blocks));
       if (blocks <= 0) return fail(SWARM_ECUDA, "wide kernel cannot be resident");

@@ -3,6 +3,7 @@
 #pragma once
 #include "hermite.cuh"
 #include "hermite_block.cuh"
+#include "hermite_ff.cuh"
 #include "kernels.h"
 
 namespace swarm {
@@ -180,13 +181,41 @@ __device__ __forceinline__ void bpl_hermite_body(const BinView &B, const StepPar
 // inertial step moves by h v_cm, its accelerations summing to zero); it drops body 0's
 // predictor and corrector and the coordinate differences of body 0's pairs.  Inertial
 // coordinates are rebuilt at log points and at the end:
-//   x_0 = X_cm - sum_{k>=1} m_k X_k / M,  x_k = X_k + x_0   (likewise v).
-// The corrector bases of a step live in registers, or (sb != nullptr) in this lane's
-// column of shared memory (sb[k * 128], k < 6N), which frees registers for a build with
-// more resident warps.
+//   x_0 = X_cm - sum_{k>=1} m_k X_k / M,  x_k = X_k + x_0   (likewise v),
+// X_cm moved by its velocity times the time elapsed.
+//
+// The steps are those of hermite_ff.cuh.  Bound: the FP64 pipe and the issue slots about
+// evenly (57 and 58 % at n = 3, two warps per sub-partition at 255 registers; a 3-warp build
+// at 168 registers spills and misses the instruction cache: 9 % slower).  131072 x 3 systems
+// over 400 steps: 37.0 ms wholly in FP64 (413 FP64 slots per step, the pipe 97 % busy), 8.0 ms
+// with 50 FP64 and 3250 other instructions per step; 16384 x 4 over 400 steps 10.8 -> 4.1 ms;
+// steps of 0.003 and 0.02 orbits (levels 1 and 0), 100 of them: 9.5 -> 4.1 and 9.6 ms.
 template <int N>
-__device__ __forceinline__ void spl_hermite_body(const BinView &B, const StepParams &P, int unit,
-                                                 double *sb = nullptr) {
+__device__ __forceinline__ void spl_write(const BinView &B, int s, const double (&m)[N], const double (&x)[N][3],
+                                          const double (&v)[N][3], double Minv, const double (&Xc)[3],
+                                          const double (&Vc)[3], double elapsed, const StepParams *log, double t) {
+  const int SP = B.S_pad;
+  double xo[N][3], vo[N][3], Xe[3];
+#pragma unroll
+  for (int c = 0; c < 3; c++) Xe[c] = fma(elapsed, Vc[c], Xc[c]);
+  spl_from_rel<N>(m, x, v, Minv, Xe, Vc, xo, vo);
+  if (log) {
+    double e[4];
+    spl_energy<N>(xo, vo, m, e);
+    write_log(*log, B.gidx[s], t, e);
+    return;
+  }
+#pragma unroll
+  for (int i = 0; i < N; i++)
+#pragma unroll
+    for (int c = 0; c < 3; c++) {
+      B.x[(size_t)(c * N + i) * SP + s] = xo[i][c];
+      B.v[(size_t)(c * N + i) * SP + s] = vo[i][c];
+    }
+}
+
+template <int N>
+__device__ __forceinline__ void spl_hermite_body(const BinView &B, const StepParams &P, int unit) {
   const bool printed = P.corr_form != 0;  // warp-uniform
   const int s = unit * 32 + (threadIdx.x & 31);
   if (s >= B.S) return;
@@ -209,129 +238,52 @@ __device__ __forceinline__ void spl_hermite_body(const BinView &B, const StepPar
     B.status[s] = SWARM_SYS_DONE;
     return;
   }
-  double kc[N][N];
-#pragma unroll
-  for (int i = 1; i < N; i++)
-#pragma unroll
-    for (int k = i + 1; k < N; k++) kc[i][k] = hill_kc(P.ce_factor, m[i], m[k], m[0]);
-
-  // relative coordinates (index 0 unused) and the barycentre
+  const FLimits<N> L = flimits<N>(m, P.ce_factor, P.eject2);
   double Minv, Xc[3], Vc[3];
   spl_to_rel<N>(m, x, v, Minv, Xc, Vc);
-  auto inertial = [&](double (&xo)[N][3], double (&vo)[N][3]) { spl_from_rel<N>(m, x, v, Minv, Xc, Vc, xo, vo); };
-
-  double a0[N][3], j0[N][3], q2[N], d2[N][N];
-  spl_accjerk_rel<N>(P.fk, x, v, m, a0, j0, q2, d2);
-  // 1/|d| carried from evaluation to evaluation within a step (three bodies and fewer:
-  // the registers of four do not fit)
-  constexpr bool kCache = N <= 3;
-  RhoCache<N> rc;
-  const HCoef cdt = hcoef(P.dt);
-  const HCoef clast = hcoef(plan.h_last);
-  int steps_done = 0;
-  int code = 0;
-  const bool ej_on = P.eject2 > 0.0;
-  for (int k = 1; k <= Ns; k++) {
-    const HCoef C = (k == Ns && !plan.exact) ? clast : cdt;
-    double xk[N][3], vk[N][3], Xr[N][3], Vr[N][3];
-    auto XB = [&](int i, int c) -> double & { return sb ? sb[(i * 3 + c) * 128] : Xr[i][c]; };
-    auto VB = [&](int i, int c) -> double & { return sb ? sb[(3 * N + i * 3 + c) * 128] : Vr[i][c]; };
-#pragma unroll
-    for (int i = 1; i < N; i++)
-#pragma unroll
-      for (int c = 0; c < 3; c++) {
-        xk[i][c] = fma(j0[i][c], C.h3_6, fma(a0[i][c], C.h2_2, fma(v[i][c], C.h, x[i][c])));
-        vk[i][c] = fma(j0[i][c], C.h2_2, fma(a0[i][c], C.h, v[i][c]));
-        VB(i, c) = fma(j0[i][c], C.h2_12, fma(a0[i][c], C.hh, v[i][c]));
-      }
-    PCoef PC;
-    if (printed) {
-      PC = pcoef(C.h);
-#pragma unroll
-      for (int i = 1; i < N; i++)
-#pragma unroll
-        for (int c = 0; c < 3; c++) XB(i, c) = fma(j0[i][c], PC.pj, fma(a0[i][c], PC.pa, xk[i][c]));
+  FMass<N> F = fmass<N>(m);
+  F.ok = F.ok && fscale(P.dt, -60, 40) && !printed;
+  double a0[N][3];
+  ff j0[N][3], sa[3], sj[3];
+  float da[N][3], q2[N], d2[N][N];
+  int level = spl_ff_state_call<N, false>(P.fk, F, P.fc.hf, x, v, a0, da, j0, q2, d2, sa, sj);
+  int k = 0, code = 0;  // steps done
+  const int whole = plan.exact ? Ns : Ns - 1;
+  while (k < Ns) {
+    if (level == 2 && k < whole) {
+      k++;
+      level = spl_hermite_delta_step<N, false>(P.fk, F, P.fc, P.fc.hf, P.n_corr, x, v, a0, da, j0, q2, d2, sa, sj);
+      code = spl_ff_monitor<N>(P.fk, level, L, q2, d2, x, v, P.eject2);
+    } else if (level && k < whole) {
+      k++;
+      level = spl_hermite_ff_step_call<N, false>(P.fk, F, P.fc, P.fc.hf, P.n_corr, x, v, a0, da, j0, q2, d2, sa, sj);
+      code = spl_ff_monitor<N>(P.fk, level, L, q2, d2, x, v, P.eject2);
     } else {
-#pragma unroll
-      for (int i = 1; i < N; i++)
-#pragma unroll
-        for (int c = 0; c < 3; c++) XB(i, c) = fma(a0[i][c], C.h2_12, fma(v[i][c], C.hh, x[i][c]));
+      int count = k < whole ? min(whole - k, kFP64Run) : 1;
+      if (P.log_interval > 0) count = min(count, P.log_interval - k % P.log_interval);
+      const double h = k < whole ? P.dt : plan.h_last;
+      double t = 0.0;
+      bool reached = false;
+      code = printed ? spl_hermite_fp64_run<N, false, true>(P.fk, m, L.kc, P.eject2, h, P.n_corr, count, true, x, v, a0, j0, k, t, t, reached)
+                     : spl_hermite_fp64_run<N, false, false>(P.fk, m, L.kc, P.eject2, h, P.n_corr, count, true, x, v, a0, j0, k, t, t, reached);
+      if (!code && k < Ns && !printed) level = spl_ff_state_call<N, false>(P.fk, F, P.fc.hf, x, v, a0, da, j0, q2, d2, sa, sj);
     }
-    for (int ic = 0; ic < P.n_corr; ic++) {
-      double ak[N][3], jk[N][3];
-      if (!kCache) spl_accjerk_rel<N>(P.fk, xk, vk, m, ak, jk, q2, d2);
-      else if (ic == 0) spl_accjerk_rel_cached<N, true>(P.fk, xk, vk, m, ak, jk, q2, d2, rc);
-      else spl_accjerk_rel_cached<N, false>(P.fk, xk, vk, m, ak, jk, q2, d2, rc);
-#pragma unroll
-      for (int i = 1; i < N; i++)
-#pragma unroll
-        for (int c = 0; c < 3; c++) vk[i][c] = fma(-C.h2_12, jk[i][c], fma(C.hh, ak[i][c], VB(i, c)));
-      if (printed) {
-#pragma unroll
-        for (int i = 1; i < N; i++)
-#pragma unroll
-          for (int c = 0; c < 3; c++) xk[i][c] = fma(PC.cj, jk[i][c], fma(PC.ca, ak[i][c], XB(i, c)));
-      } else {
-#pragma unroll
-        for (int i = 1; i < N; i++)
-#pragma unroll
-          for (int c = 0; c < 3; c++) xk[i][c] = fma(-C.h2_12, ak[i][c], fma(C.hh, vk[i][c], XB(i, c)));
-      }
-    }
-    if (!kCache || P.n_corr == 0) spl_accjerk_rel<N>(P.fk, xk, vk, m, a0, j0, q2, d2);
-    else spl_accjerk_rel_cached<N, false>(P.fk, xk, vk, m, a0, j0, q2, d2, rc);
-#pragma unroll
-    for (int i = 1; i < N; i++)
-#pragma unroll
-      for (int c = 0; c < 3; c++) {
-        x[i][c] = xk[i][c];
-        v[i][c] = vk[i][c];
-      }
-#pragma unroll
-    for (int c = 0; c < 3; c++) Xc[c] = fma(C.h, Vc[c], Xc[c]);
-    steps_done = k;
-    bool nf = false, ej = false, ce = false;
-#pragma unroll
-    for (int i = 1; i < N; i++)
-#pragma unroll
-      for (int c = 0; c < 3; c++) nf |= nonfinite(x[i][c]) | nonfinite(v[i][c]);
-#pragma unroll
-    for (int i = 1; i < N; i++) ej |= ej_on && nonneg_lt(P.eject2, q2[i]);
-#pragma unroll
-    for (int i = 1; i < N; i++)
-#pragma unroll
-      for (int k2 = i + 1; k2 < N; k2++)
-        if (kc[i][k2] > 0.0 && close_encounter(P.fk, d2[i][k2], kc[i][k2], q2[i], q2[k2])) ce = true;
-    code = nf ? SWARM_SYS_NONFINITE : ej ? SWARM_SYS_EJECTED : ce ? SWARM_SYS_CLOSE_ENCOUNTER : 0;
     if (code) break;
     if (P.log_interval > 0 && (k % P.log_interval) == 0) {
-      double xo[N][3], vo[N][3], e[4];
-      inertial(xo, vo);
-      spl_energy<N>(xo, vo, m, e);
-      write_log(P, B.gidx[s], step_time(plan, k, t0, P.dt), e);
+      const double tk = step_time(plan, k, t0, P.dt);
+      spl_write<N>(B, s, m, x, v, Minv, Xc, Vc, tk - t0, &P, tk);
     }
   }
-  const double tk = step_time(plan, steps_done, t0, P.dt);
-  {
-    double xo[N][3], vo[N][3];
-    inertial(xo, vo);
-#pragma unroll
-    for (int i = 0; i < N; i++)
-#pragma unroll
-      for (int c = 0; c < 3; c++) {
-        B.x[(size_t)(c * N + i) * SP + s] = xo[i][c];
-        B.v[(size_t)(c * N + i) * SP + s] = vo[i][c];
-      }
-  }
+  const double tk = step_time(plan, k, t0, P.dt);
+  spl_write<N>(B, s, m, x, v, Minv, Xc, Vc, tk - t0, nullptr, tk);
   B.t[s] = tk;
   B.status[s] = code ? code : (plan.full ? SWARM_SYS_DONE : SWARM_SYS_ACTIVE);
   if (P.counters) {
     constexpr unsigned long long NP = (unsigned long long)N * (N - 1) / 2;
-    atomicAdd(&P.counters[0], (unsigned long long)steps_done);
-    atomicAdd(&P.counters[1], NP * (1ull + (unsigned long long)steps_done * (P.n_corr + 1)));
+    atomicAdd(&P.counters[0], (unsigned long long)k);
+    atomicAdd(&P.counters[1], NP * (1ull + (unsigned long long)k * (P.n_corr + 1)));
   }
 }
-
 
 // ---------------------------------------------------------------- adaptive step (Eq. 5)
 // The Hermite propagator with the step of Sec. 4.3.2: dt = tau (sum_i |j_i|^2/|a_i|^2)^(-1/2)
@@ -501,207 +453,49 @@ __device__ __forceinline__ void bpl_hermite_adaptive_body(const BinView &B, cons
   }
 }
 
-// Eq. 5 sum over the bodies of a system held by one lane, sum_i |j_i|^2 / |a_i|^2, with
-// one division: the running fraction num/den takes body i as (num A_i + J_i den)/(den A_i)
-// (A = |a|^2, J = |j|^2; den stays within range for the n <= 4 of this mapping).
-template <int N>
-__device__ __forceinline__ double spl_eq5_sum(const F64k &k, const double (&a)[N][3], const double (&j)[N][3]) {
-  double num = 0.0, den = 1.0;
-#pragma unroll
-  for (int i = 0; i < N; i++) {
-    const double A = fma(a[i][2], a[i][2], fma(a[i][1], a[i][1], kmul(k, a[i][0], a[i][0])));
-    const double J = fma(j[i][2], j[i][2], fma(j[i][1], j[i][1], kmul(k, j[i][0], j[i][0])));
-    num = fma(num, A, kmul(k, J, den));
-    den = kmul(k, den, A);
-  }
-  return num / den;
-}
-
-// The same sum from the relative-coordinate values of spl_accjerk_rel: a_0 = A[0],
-// a_k = A[k] + A[0] (likewise the jerks).
-template <int N>
-__device__ __forceinline__ double spl_eq5_sum_rel(const F64k &kk, const double (&A)[N][3], const double (&J)[N][3]) {
-  double a[N][3], j[N][3];
-#pragma unroll
-  for (int c = 0; c < 3; c++) {
-    a[0][c] = A[0][c];
-    j[0][c] = J[0][c];
-#pragma unroll
-    for (int k = 1; k < N; k++) {
-      a[k][c] = kadd(kk, A[k][c], A[0][c]);
-      j[k][c] = kadd(kk, J[k][c], J[0][c]);
-    }
-  }
-  return spl_eq5_sum<N>(kk, a, j);
-}
-
-template <int N>
-__device__ __forceinline__ void spl_hermite_adaptive_body(const BinView &B, const StepParams &P, int unit) {
-  const bool printed = P.corr_form != 0;  // warp-uniform
-  // a unit is 32 consecutive entries of the launch's system order (longest first when a
-  // list is given, so the lanes of a warp take similar numbers of Eq. 5 steps)
-  const int s = stream_system(B, unit * 32 + (threadIdx.x & 31));
-  if (s < 0) return;
-  const int SP = B.S_pad;
-  double x[N][3], v[N][3], m[N];
-#pragma unroll
-  for (int i = 0; i < N; i++) {
-    m[i] = B.m[(size_t)i * SP + s];
-#pragma unroll
-    for (int c = 0; c < 3; c++) {
-      x[i][c] = B.x[(size_t)(c * N + i) * SP + s];
-      v[i][c] = B.v[(size_t)(c * N + i) * SP + s];
-    }
-  }
-  const double t0 = B.t[s];
-  if (B.status[s] > SWARM_SYS_DONE) return;
-  const double te = adaptive_end(B, P, s);
-  const double tau = fabs(P.dt), dir = P.dt > 0 ? 1.0 : -1.0;
-  if (!((te - t0) * dir > 1e-12 * fmax(1.0, fabs(te)))) {
-    B.status[s] = SWARM_SYS_DONE;
-    return;
-  }
-  double Minv, Xc[3], Vc[3];
-  spl_to_rel<N>(m, x, v, Minv, Xc, Vc);
-  double kc[N][N];
-#pragma unroll
-  for (int i = 1; i < N; i++)
-#pragma unroll
-    for (int k = i + 1; k < N; k++) kc[i][k] = hill_kc(P.ce_factor, m[i], m[k], m[0]);
-  double a0[N][3], j0[N][3], q2[N], d2[N][N];
-  spl_accjerk_rel<N>(P.fk, x, v, m, a0, j0, q2, d2);
-  const int cap = P.max_steps > 0 ? P.max_steps : kAdaptiveStepCap;
-  double t = t0;
-  int steps_done = 0, code = 0;
-  bool reached = false;
-  for (int k = 1; k <= cap; k++) {
-    double h = kmul(P.fk, tau, rsqrt(spl_eq5_sum_rel<N>(P.fk, a0, j0)));
-    if (!(h > 0.0) || nonfinite(h)) {
-      code = SWARM_SYS_NONFINITE;
-      break;
-    }
-    const double rem = kmul(P.fk, ksub(P.fk, te, t), dir);
-    const bool last = h >= rem;
-    h = kmul(P.fk, last ? rem : h, dir);
-    const HCoef C = hcoef(P.fk, h);
-    double xk[N][3], vk[N][3], Xb[N][3], Vb[N][3];
-#pragma unroll
-    for (int i = 1; i < N; i++)
-#pragma unroll
-      for (int c = 0; c < 3; c++) {
-        xk[i][c] = fma(j0[i][c], C.h3_6, fma(a0[i][c], C.h2_2, fma(v[i][c], C.h, x[i][c])));
-        vk[i][c] = fma(j0[i][c], C.h2_2, fma(a0[i][c], C.h, v[i][c]));
-        Vb[i][c] = fma(j0[i][c], C.h2_12, fma(a0[i][c], C.hh, v[i][c]));
-      }
-    PCoef PC;
-    if (printed) {
-      PC = pcoef(C.h);
-#pragma unroll
-      for (int i = 1; i < N; i++)
-#pragma unroll
-        for (int c = 0; c < 3; c++) Xb[i][c] = fma(j0[i][c], PC.pj, fma(a0[i][c], PC.pa, xk[i][c]));
-    } else {
-#pragma unroll
-      for (int i = 1; i < N; i++)
-#pragma unroll
-        for (int c = 0; c < 3; c++) Xb[i][c] = fma(a0[i][c], C.h2_12, fma(v[i][c], C.hh, x[i][c]));
-    }
-    for (int ic = 0; ic < P.n_corr; ic++) {
-      double ak[N][3], jk[N][3];
-      spl_accjerk_rel<N>(P.fk, xk, vk, m, ak, jk, q2, d2);
-#pragma unroll
-      for (int i = 1; i < N; i++)
-#pragma unroll
-        for (int c = 0; c < 3; c++) vk[i][c] = fma(-C.h2_12, jk[i][c], fma(C.hh, ak[i][c], Vb[i][c]));
-      if (printed) {
-#pragma unroll
-        for (int i = 1; i < N; i++)
-#pragma unroll
-          for (int c = 0; c < 3; c++) xk[i][c] = fma(PC.cj, jk[i][c], fma(PC.ca, ak[i][c], Xb[i][c]));
-      } else {
-#pragma unroll
-        for (int i = 1; i < N; i++)
-#pragma unroll
-          for (int c = 0; c < 3; c++) xk[i][c] = fma(-C.h2_12, ak[i][c], fma(C.hh, vk[i][c], Xb[i][c]));
-      }
-    }
-    spl_accjerk_rel<N>(P.fk, xk, vk, m, a0, j0, q2, d2);
-#pragma unroll
-    for (int i = 1; i < N; i++)
-#pragma unroll
-      for (int c = 0; c < 3; c++) {
-        x[i][c] = xk[i][c];
-        v[i][c] = vk[i][c];
-      }
-#pragma unroll
-    for (int c = 0; c < 3; c++) Xc[c] = fma(C.h, Vc[c], Xc[c]);
-    steps_done = k;
-    t = last ? te : kadd(P.fk, t, h);
-    bool nf = false, ej = false, ce = false;
-#pragma unroll
-    for (int i = 1; i < N; i++)
-#pragma unroll
-      for (int c = 0; c < 3; c++) nf |= nonfinite(x[i][c]) | nonfinite(v[i][c]);
-#pragma unroll
-    for (int i = 1; i < N; i++) ej |= (P.eject2 > 0.0) && (q2[i] > P.eject2);
-#pragma unroll
-    for (int i = 1; i < N; i++)
-#pragma unroll
-      for (int k2 = i + 1; k2 < N; k2++)
-        if (kc[i][k2] > 0.0 && close_encounter(P.fk, d2[i][k2], kc[i][k2], q2[i], q2[k2])) ce = true;
-    code = nf ? SWARM_SYS_NONFINITE : ej ? SWARM_SYS_EJECTED : ce ? SWARM_SYS_CLOSE_ENCOUNTER : 0;
-    if (code) break;
-    if (P.log_interval > 0 && (k % P.log_interval) == 0) {
-      double xo[N][3], vo[N][3], e[4];
-      spl_from_rel<N>(m, x, v, Minv, Xc, Vc, xo, vo);
-      spl_energy<N>(xo, vo, m, e);
-      write_log(P, B.gidx[s], t, e);
-    }
-    if (last) {
-      reached = true;
-      break;
-    }
-  }
-  {
-    double xo[N][3], vo[N][3];
-    spl_from_rel<N>(m, x, v, Minv, Xc, Vc, xo, vo);
-#pragma unroll
-    for (int i = 0; i < N; i++)
-#pragma unroll
-      for (int c = 0; c < 3; c++) {
-        B.x[(size_t)(c * N + i) * SP + s] = xo[i][c];
-        B.v[(size_t)(c * N + i) * SP + s] = vo[i][c];
-      }
-  }
-  B.t[s] = t;
-  B.status[s] = code ? code : (reached ? SWARM_SYS_DONE : SWARM_SYS_ACTIVE);
-  if (P.counters && steps_done > 0) {
-    constexpr unsigned long long NP = (unsigned long long)N * (N - 1) / 2;
-    atomicAdd(&P.counters[0], (unsigned long long)steps_done);
-    atomicAdd(&P.counters[1], NP * (1ull + (unsigned long long)steps_done * (P.n_corr + 1)));
-  }
-}
-
 // Adaptive steps, system per lane, with work handed out per lane: a lane whose system
-// reached its end time (or stopped) takes the bin's next system at once, so the warp does
-// not wait for the lane with the most steps (adaptive step counts differ from system to
-// system).  One loop, each round either loads a new system (that lane only) or takes one
-// step; per system the arithmetic is that of spl_hermite_adaptive_body.
-template <int N>
-__device__ __forceinline__ void spl_hermite_adaptive_stream(const BinView &B, const StepParams &P) {
+// reached its end time (or stopped) takes its next system at once, so the warp does not wait
+// for the lane with the most steps (adaptive step counts differ from system to system).  One
+// loop, each round either loads a new system (that lane only) or takes one step.  take(): the
+// lane's next system, or -1.  Steps as in spl_hermite_body, with Eq. 5's length in pairs.  The guard of a state wants the length of
+// the step from it, which follows from that state's evaluation: it is given 1.25 times the
+// present length, and a longer step is taken in FP64.  A system that comes to level 0 stays
+// in FP64 (eta is about tau / sqrt 2 all along an orbit, and lanes that change back and forth
+// at their own times would make a warp take both kinds of step).  131072 x 3 systems over a
+// quarter of an inner period: 37.4 -> 18 ms; the loop is long enough to miss the instruction
+// cache (lanes are at different points of their systems).
+template <int N, class Take>
+__device__ __forceinline__ void spl_hermite_adaptive_run(const BinView &B, const StepParams &P, Take take) {
   const bool printed = P.corr_form != 0;  // warp-uniform
   const unsigned FULL = 0xffffffffu;
   const int SP = B.S_pad;
-  const double tau = fabs(P.dt), dir = P.dt > 0 ? 1.0 : -1.0;
+  const double dir = P.dt > 0 ? 1.0 : -1.0;
+  const ff tau = ff_from(fabs(P.dt));
   const int cap = P.max_steps > 0 ? P.max_steps : kAdaptiveStepCap;
-  double x[N][3], v[N][3], m[N], a0[N][3], j0[N][3], kc[N][N];
+  double x[N][3], v[N][3], m[N], a0[N][3];
+  ff j0[N][3], sa[3], sj[3], h;
+  float da[N][3], q2[N], d2[N][N], hf = 0.0f;
+  FLimits<N> L;
+  FMass<N> F;
   double Minv = 1.0, Xc[3] = {0.0, 0.0, 0.0}, Vc[3] = {0.0, 0.0, 0.0};
-  double t = 0.0, te = 0.0;
-  int s = 0, steps = 0;
+  double t = 0.0, t0 = 0.0, te = 0.0;
+  int s = 0, steps = 0, level = 0;
+  bool carried = false;  // a0, j0 are those of an FP64 step
   bool has = false, exhausted = false;
+  auto next_step = [&]() {
+    h = spl_ff_eq5<N>(tau, a0, da, j0, sa, sj);
+    if (!(h.h > 0.0f && h.h <= hf)) level = 0;
+  };
+  auto look = [&]() {  // at a state whose step length is not known yet
+    spl_ff_state_call<N, true>(P.fk, F, 0.0f, x, v, a0, da, j0, q2, d2, sa, sj);
+    h = spl_ff_eq5<N>(tau, a0, da, j0, sa, sj);
+    hf = 1.25f * h.h;
+    level = spl_ff_state_call<N, true>(P.fk, F, hf, x, v, a0, da, j0, q2, d2, sa, sj);
+    next_step();
+  };
   for (;;) {
     if (!has && !exhausted) {
-      s = stream_system(B, atomicAdd(P.work_next, 1));
+      s = take();
       if (s < 0) {
         exhausted = true;
       } else if (B.status[s] <= SWARM_SYS_DONE) {
@@ -714,125 +508,54 @@ __device__ __forceinline__ void spl_hermite_adaptive_stream(const BinView &B, co
             v[i][c] = B.v[(size_t)(c * N + i) * SP + s];
           }
         }
-        t = B.t[s];
+        t0 = t = B.t[s];
         te = adaptive_end(B, P, s);
         if (!((te - t) * dir > 1e-12 * fmax(1.0, fabs(te)))) {
           B.status[s] = SWARM_SYS_DONE;
         } else {
-#pragma unroll
-          for (int i = 1; i < N; i++)
-#pragma unroll
-            for (int k = i + 1; k < N; k++) kc[i][k] = hill_kc(P.ce_factor, m[i], m[k], m[0]);
+          L = flimits<N>(m, P.ce_factor, P.eject2);
+          F = fmass<N>(m);
+          F.ok = F.ok && fscale(P.dt, -60, 40) && !printed;
           spl_to_rel<N>(m, x, v, Minv, Xc, Vc);
-          double q2[N], d2[N][N];
-          spl_accjerk_rel<N>(P.fk, x, v, m, a0, j0, q2, d2);
+          look();
           steps = 0;
+          carried = false;
           has = true;
         }
       }
     }
     if (!__any_sync(FULL, has || !exhausted)) break;
     if (!has) continue;
-    // one step (Eq. 5 length from the start-of-step a0, j0)
     int code = 0;
-    bool finish = false, reached = false;
-    double h = kmul(P.fk, tau, rsqrt(spl_eq5_sum_rel<N>(P.fk, a0, j0)));
-    if (!(h > 0.0) || nonfinite(h)) {
-      code = SWARM_SYS_NONFINITE;
-      finish = true;
-    } else {
+    bool reached = false;
+    if (level) {
       const double rem = kmul(P.fk, ksub(P.fk, te, t), dir);
-      const bool last = h >= rem;
-      h = kmul(P.fk, last ? rem : h, dir);
-      const HCoef C = hcoef(P.fk, h);
-      double xk[N][3], vk[N][3], Xb[N][3], Vb[N][3];
-#pragma unroll
-      for (int i = 1; i < N; i++)
-#pragma unroll
-        for (int c = 0; c < 3; c++) {
-          xk[i][c] = fma(j0[i][c], C.h3_6, fma(a0[i][c], C.h2_2, fma(v[i][c], C.h, x[i][c])));
-          vk[i][c] = fma(j0[i][c], C.h2_2, fma(a0[i][c], C.h, v[i][c]));
-          Vb[i][c] = fma(j0[i][c], C.h2_12, fma(a0[i][c], C.hh, v[i][c]));
-        }
-      PCoef PC;
-      if (printed) {
-        PC = pcoef(C.h);
-#pragma unroll
-        for (int i = 1; i < N; i++)
-#pragma unroll
-          for (int c = 0; c < 3; c++) Xb[i][c] = fma(j0[i][c], PC.pj, fma(a0[i][c], PC.pa, xk[i][c]));
+      double hd = ff_double(h);
+      // compared in FP32 first (FP64 compares are slow)
+      const bool last = h.h >= 0.999f * f_from(rem) && hd >= rem;
+      if (last) hd = rem;
+      hd = kmul(P.fk, hd, dir);
+      const FCoef C = fcoef(hd);
+      hf = 1.25f * C.hf;
+      if (level == 2) {
+        level = spl_hermite_delta_step<N, true>(P.fk, F, C, hf, P.n_corr, x, v, a0, da, j0, q2, d2, sa, sj);
       } else {
-#pragma unroll
-        for (int i = 1; i < N; i++)
-#pragma unroll
-          for (int c = 0; c < 3; c++) Xb[i][c] = fma(a0[i][c], C.h2_12, fma(v[i][c], C.hh, x[i][c]));
+        level = spl_hermite_ff_step_call<N, true>(P.fk, F, C, hf, P.n_corr, x, v, a0, da, j0, q2, d2, sa, sj);
       }
-      double q2[N], d2[N][N];
-      for (int ic = 0; ic < P.n_corr; ic++) {
-        double ak[N][3], jk[N][3];
-        spl_accjerk_rel<N>(P.fk, xk, vk, m, ak, jk, q2, d2);
-#pragma unroll
-        for (int i = 1; i < N; i++)
-#pragma unroll
-          for (int c = 0; c < 3; c++) vk[i][c] = fma(-C.h2_12, jk[i][c], fma(C.hh, ak[i][c], Vb[i][c]));
-        if (printed) {
-#pragma unroll
-          for (int i = 1; i < N; i++)
-#pragma unroll
-            for (int c = 0; c < 3; c++) xk[i][c] = fma(PC.cj, jk[i][c], fma(PC.ca, ak[i][c], Xb[i][c]));
-        } else {
-#pragma unroll
-          for (int i = 1; i < N; i++)
-#pragma unroll
-            for (int c = 0; c < 3; c++) xk[i][c] = fma(-C.h2_12, ak[i][c], fma(C.hh, vk[i][c], Xb[i][c]));
-        }
-      }
-      spl_accjerk_rel<N>(P.fk, xk, vk, m, a0, j0, q2, d2);
-#pragma unroll
-      for (int i = 1; i < N; i++)
-#pragma unroll
-        for (int c = 0; c < 3; c++) {
-          x[i][c] = xk[i][c];
-          v[i][c] = vk[i][c];
-        }
-#pragma unroll
-      for (int c = 0; c < 3; c++) Xc[c] = fma(C.h, Vc[c], Xc[c]);
       steps++;
-      t = last ? te : kadd(P.fk, t, h);
-      bool nf = false, ej = false, ce = false;
-#pragma unroll
-      for (int i = 1; i < N; i++)
-#pragma unroll
-        for (int c = 0; c < 3; c++) nf |= nonfinite(x[i][c]) | nonfinite(v[i][c]);
-#pragma unroll
-      for (int i = 1; i < N; i++) ej |= (P.eject2 > 0.0) && (q2[i] > P.eject2);
-#pragma unroll
-      for (int i = 1; i < N; i++)
-#pragma unroll
-        for (int k2 = i + 1; k2 < N; k2++)
-          if (kc[i][k2] > 0.0 && close_encounter(P.fk, d2[i][k2], kc[i][k2], q2[i], q2[k2])) ce = true;
-      code = nf ? SWARM_SYS_NONFINITE : ej ? SWARM_SYS_EJECTED : ce ? SWARM_SYS_CLOSE_ENCOUNTER : 0;
-      if (!code && P.log_interval > 0 && (steps % P.log_interval) == 0) {
-        double xo[N][3], vo[N][3], e[4];
-        spl_from_rel<N>(m, x, v, Minv, Xc, Vc, xo, vo);
-        spl_energy<N>(xo, vo, m, e);
-        write_log(P, B.gidx[s], t, e);
-      }
+      t = last ? te : kadd(P.fk, t, hd);
+      code = spl_ff_monitor<N>(P.fk, level, L, q2, d2, x, v, P.eject2);
       reached = last && !code;
-      finish = code != 0 || last || steps >= cap;
+      next_step();
+    } else {
+      code = printed ? spl_hermite_fp64_run<N, true, true>(P.fk, m, L.kc, P.eject2, P.dt, P.n_corr, 1, !carried, x, v, a0, j0, steps, t, te, reached)
+                     : spl_hermite_fp64_run<N, true, false>(P.fk, m, L.kc, P.eject2, P.dt, P.n_corr, 1, !carried, x, v, a0, j0, steps, t, te, reached);
+      carried = true;
     }
-    if (finish) {
-      {
-        double xo[N][3], vo[N][3];
-        spl_from_rel<N>(m, x, v, Minv, Xc, Vc, xo, vo);
-#pragma unroll
-        for (int i = 0; i < N; i++)
-#pragma unroll
-          for (int c = 0; c < 3; c++) {
-            B.x[(size_t)(c * N + i) * SP + s] = xo[i][c];
-            B.v[(size_t)(c * N + i) * SP + s] = vo[i][c];
-          }
-      }
+    if (!code && P.log_interval > 0 && steps > 0 && (steps % P.log_interval) == 0)
+      spl_write<N>(B, s, m, x, v, Minv, Xc, Vc, t - t0, &P, t);
+    if (code != 0 || reached || steps >= cap) {
+      spl_write<N>(B, s, m, x, v, Minv, Xc, Vc, t - t0, nullptr, t);
       B.t[s] = t;
       B.status[s] = code ? code : (reached ? SWARM_SYS_DONE : SWARM_SYS_ACTIVE);
       if (P.counters && steps > 0) {
@@ -843,6 +566,20 @@ __device__ __forceinline__ void spl_hermite_adaptive_stream(const BinView &B, co
       has = false;
     }
   }
+}
+template <int N>
+__device__ __forceinline__ void spl_hermite_adaptive_stream(const BinView &B, const StepParams &P) {
+  spl_hermite_adaptive_run<N>(B, P, [&]() { return stream_system(B, atomicAdd(P.work_next, 1)); });
+}
+// one unit: 32 consecutive entries of the launch's system order
+template <int N>
+__device__ __forceinline__ void spl_hermite_adaptive_body(const BinView &B, const StepParams &P, int unit) {
+  bool taken = false;
+  spl_hermite_adaptive_run<N>(B, P, [&]() {
+    const int s = taken ? -1 : stream_system(B, unit * 32 + (threadIdx.x & 31));
+    taken = true;
+    return s;
+  });
 }
 
 // Body per lane with work handed out per system: each of the warp's G groups takes the
@@ -1076,16 +813,12 @@ __device__ __noinline__ void spl_hermite_adaptive_unit(const BinView &B, const S
 
 // Persistent kernel for one bin (one body count, one mapping): the unit body is inlined,
 // so registers are allocated for this n alone.  Warps pull unit indices from a counter.
-// MINB = 3 is the high-occupancy variant (registers capped for 3 CTAs of 128 threads per SM).
-template <int MAP, int N, int MINB, bool ADAPT = false>
-__global__ void __launch_bounds__(128, MINB) hermite_uniform_kernel(BinView B, int nunits, StepParams P) {
+template <int MAP, int N, bool ADAPT = false>
+__global__ void __launch_bounds__(128, 2) hermite_uniform_kernel(BinView B, int nunits, StepParams P) {
   if (ADAPT && MAP == SWARM_MAP_SYSTEM_PER_LANE) {  // work unit = system (per-lane refill)
     spl_hermite_adaptive_stream<N>(B, P);
     return;
   }
-  // the high-occupancy system-per-lane build keeps the corrector bases in shared memory
-  constexpr bool kSmemBases = !ADAPT && MAP == SWARM_MAP_SYSTEM_PER_LANE && MINB >= 3;
-  __shared__ double sbases[kSmemBases ? 6 * N * 128 : 1];
   if (MAP == SWARM_MAP_BODY_PER_LANE) {  // work unit = system (per-group refill)
     bpl_hermite_stream<N, ADAPT>(B, P);
     return;
@@ -1096,25 +829,21 @@ __global__ void __launch_bounds__(128, MINB) hermite_uniform_kernel(BinView B, i
     if (lane == 0) w = atomicAdd(P.work_next, 1);
     w = __shfl_sync(0xffffffffu, w, 0);
     if (w >= nunits) break;
-    if (ADAPT) {
-      if (MAP == SWARM_MAP_SYSTEM_PER_LANE) spl_hermite_adaptive_body<N>(B, P, w);
-      else bpl_hermite_adaptive_body<N>(B, P, w);
-    } else {
-      if (MAP == SWARM_MAP_SYSTEM_PER_LANE) spl_hermite_body<N>(B, P, w, kSmemBases ? sbases + threadIdx.x : nullptr);
-      else bpl_hermite_body<N>(B, P, w);
-    }
+    spl_hermite_body<N>(B, P, w);
   }
 }
 
-template <int MAP, int N, int MINB = 2, bool ADAPT = false>
+template <int MAP, int N, bool ADAPT = false>
 cudaError_t launch_hermite_uniform_n(const BinView &B, int nunits, const StepParams &P, int grid, cudaStream_t st) {
-  hermite_uniform_kernel<MAP, N, MINB, ADAPT><<<grid, 128, 0, st>>>(B, nunits, P);
+  StepParams Q = P;
+  Q.fc = fcoef_host(P.dt);
+  hermite_uniform_kernel<MAP, N, ADAPT><<<grid, 128, 0, st>>>(B, nunits, Q);
   return cudaGetLastError();
 }
-template <int MAP, int N, int MINB = 2, bool ADAPT = false>
+template <int MAP, int N, bool ADAPT = false>
 int hermite_uniform_blocks_n() {
   int nb = 0;
-  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, hermite_uniform_kernel<MAP, N, MINB, ADAPT>, 128, 0);
+  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, hermite_uniform_kernel<MAP, N, ADAPT>, 128, 0);
   return nb;
 }
 // adaptive (Eq. 5) single-bin kernels: both mappings, registers sized for 2 CTAs per SM
@@ -1122,8 +851,8 @@ template <int MAP, int N>
 cudaError_t launch_hermite_uniform_pick(const BinView &B, int nunits, const StepParams &P, int grid, cudaStream_t st,
                                         int *blocks, bool adaptive) {
   if (adaptive) {
-    if (blocks) *blocks = hermite_uniform_blocks_n<MAP, N, 2, true>();
-    return grid > 0 ? launch_hermite_uniform_n<MAP, N, 2, true>(B, nunits, P, grid, st) : cudaSuccess;
+    if (blocks) *blocks = hermite_uniform_blocks_n<MAP, N, true>();
+    return grid > 0 ? launch_hermite_uniform_n<MAP, N, true>(B, nunits, P, grid, st) : cudaSuccess;
   }
   // fixed steps, body per lane, n >= 5: systems packed across the CTA (hermite_block.cuh)
   // when the bin fills a wave of those CTAs; a smaller bin's step latency is the limit,

@@ -197,21 +197,23 @@ __global__ void __launch_bounds__(128) plain_step_kernel(BinView B, StepParams P
 // ---------------------------------------------------------------- host launchers
 cudaError_t launch_hermite_persistent(const BinView *d_bins, const int4 *d_work, int nwork, const StepParams &P,
                                       int grid, cudaStream_t st) {
-  hermite_persistent_kernel<<<grid, 128, 0, st>>>(d_bins, d_work, nwork, P);
+  StepParams Q = P;
+  Q.fc = fcoef_host(P.dt);
+  hermite_persistent_kernel<<<grid, 128, 0, st>>>(d_bins, d_work, nwork, Q);
   return cudaGetLastError();
 }
 
 cudaError_t launch_hermite_uniform_spl(int n, const BinView &B, int nunits, const StepParams &P, int grid,
-                                       cudaStream_t st, int *blocks, int variant);
+                                       cudaStream_t st, int *blocks);
 cudaError_t launch_hermite_uniform_bpl_a(int n, const BinView &B, int nunits, const StepParams &P, int grid,
                                          cudaStream_t st, int *blocks);
 cudaError_t launch_hermite_uniform_bpl_b(int n, const BinView &B, int nunits, const StepParams &P, int grid,
                                          cudaStream_t st, int *blocks);
 
 cudaError_t launch_hermite_uniform(int mapping, const BinView &B, int nunits, const StepParams &P, int grid,
-                                   cudaStream_t st, int *blocks, int variant) {
+                                   cudaStream_t st, int *blocks) {
   if (mapping == SWARM_MAP_SYSTEM_PER_LANE)
-    return launch_hermite_uniform_spl(B.n, B, nunits, P, grid, st, blocks, variant);
+    return launch_hermite_uniform_spl(B.n, B, nunits, P, grid, st, blocks);
   if (B.n <= 8) return launch_hermite_uniform_bpl_a(B.n, B, nunits, P, grid, st, blocks);
   return launch_hermite_uniform_bpl_b(B.n, B, nunits, P, grid, st, blocks);
 }

@@ -26,9 +26,9 @@ cudaError_t launch_mvs_persistent(const BinView *d_bins, const int4 *d_work, int
 int mvs_persistent_max_blocks_per_sm();
 
 // Single-bin persistent kernels (unit body inlined).  grid <= 0 only reports the
-// resident blocks per SM in *blocks.  variant 1: high-occupancy build where one exists.
+// resident blocks per SM in *blocks.
 cudaError_t launch_hermite_uniform(int mapping, const BinView &B, int nunits, const StepParams &P, int grid,
-                                   cudaStream_t st, int *blocks, int variant = 0);
+                                   cudaStream_t st, int *blocks);
 cudaError_t launch_mvs_uniform(bool jacobi, const BinView &B, int nunits, const StepParams &P, int grid,
                                cudaStream_t st, int *blocks);
 

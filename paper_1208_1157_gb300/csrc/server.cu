@@ -217,7 +217,7 @@ static int make_pool(swarm_server *sv, int integ, int n, Pool **out) {
   // body-per-lane kernels that take the slot list and hand slots out per group
   StepParams Q{};
   Q.integrator = integ;
-  if (integ == SWARM_HERMITE4) SCK(launch_hermite_uniform(SWARM_MAP_BODY_PER_LANE, p->view, 0, Q, 0, sv->stream, &p->blocks, 0));
+  if (integ == SWARM_HERMITE4) SCK(launch_hermite_uniform(SWARM_MAP_BODY_PER_LANE, p->view, 0, Q, 0, sv->stream, &p->blocks));
   else SCK(launch_mvs_uniform(integ == SWARM_MVS_JACOBI, p->view, 0, Q, 0, sv->stream, &p->blocks));
   if (p->blocks <= 0) return sfail(SWARM_ECUDA, "pool kernel cannot be resident");
   sv->bytes_used += bytes;
@@ -550,7 +550,7 @@ extern "C" int swarm_server_step(swarm_server *sv, int32_t *n_completed) {
       const int per_sm = p->integ == SWARM_HERMITE4 ? p->blocks : 1;
       const int grid = std::max(1, std::min(sms * per_sm, (nunits + 3) / 4));
       if (p->integ == SWARM_HERMITE4)
-        SCK(launch_hermite_uniform(SWARM_MAP_BODY_PER_LANE, v, nunits, P, grid, st, nullptr, 0));
+        SCK(launch_hermite_uniform(SWARM_MAP_BODY_PER_LANE, v, nunits, P, grid, st, nullptr));
       else
         SCK(launch_mvs_uniform(p->integ == SWARM_MVS_JACOBI, v, nunits, P, grid, st, nullptr));
     }

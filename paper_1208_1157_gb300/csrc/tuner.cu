@@ -82,18 +82,22 @@ double measure(int n, int integrator, int S, cudaStream_t st, int mapping, int c
 }
 }  // namespace
 
+constexpr int kSplMinSystems = 8192;
+
 // Candidates, in the order they are measured: body per lane at the kernel's own full
 // residency (0) and at 1, 2 and 3 CTAs of 4 warps per SM (persistent grids of 1x, 2x and
 // 3x the SM count; a count above the kernel's residency runs at its residency); for the
 // Hermite step with n <= 4 also a whole system per lane at full residency and at 1 CTA
-// per SM, and for n <= 3 its high-occupancy build (3).
-void tuner_candidates(int n, int integrator, std::vector<Choice> *out) {
+// per SM, in bins that give every SM sub-partition a warp's worth of lanes to choose from
+// (kSplMinSystems); below that a step's latency decides, and body per lane has the property
+// that its steps follow from the stored state alone: a call in chunks, or resumed from a
+// checkpoint, repeats the uninterrupted one bit for bit.
+void tuner_candidates(int n, int integrator, int S, std::vector<Choice> *out) {
   *out = {{SWARM_MAP_BODY_PER_LANE, 0}, {SWARM_MAP_BODY_PER_LANE, 1}, {SWARM_MAP_BODY_PER_LANE, 2},
           {SWARM_MAP_BODY_PER_LANE, 3}};
-  if (integrator == SWARM_HERMITE4 && n <= 4) {
+  if (integrator == SWARM_HERMITE4 && n <= 4 && S >= kSplMinSystems) {
     out->push_back({SWARM_MAP_SYSTEM_PER_LANE, 0});
     out->push_back({SWARM_MAP_SYSTEM_PER_LANE, 1});
-    if (n <= 3) out->push_back({SWARM_MAP_SYSTEM_PER_LANE, 3});
   }
 }
 
@@ -119,7 +123,7 @@ int tuner_choice_internal(int n, int integrator, int S, cudaStream_t st, int32_t
     // (granularity) decides between the mappings as much as the per-step cost does
     int probeS = S < (1 << 20) ? S : (1 << 20);
     std::vector<Choice> cands;
-    tuner_candidates(n, integrator, &cands);
+    tuner_candidates(n, integrator, probeS, &cands);
     double best = -1;
     for (auto &cd : cands) {
       double r = measure(n, integrator, probeS, st, cd.mapping, cd.ctas);
