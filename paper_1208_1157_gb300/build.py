@@ -20,6 +20,9 @@ OUT = os.path.join(HERE, "_build")
 OBJ = os.path.join(OUT, "obj")
 LIB = os.path.join(OUT, "libswarm_gb300.so")
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
+# register cap of device functions that are called out of line (kernels have their launch bounds):
+# the body-per-lane Hermite kernels run three CTAs of 128 threads per SM
+SOURCE_FLAGS = {"hermite_uniform_bpl_a.cu": ["-maxrregcount", "168"], "hermite_uniform_bpl_b.cu": ["-maxrregcount", "168"]}
 FLAGS = ARCH + ["-O3", "-std=c++17", "-lineinfo", "-rdc=true", "-Xcompiler", "-fPIC", "-I", INCLUDE]
 
 
@@ -46,7 +49,7 @@ def build(force: bool = False, verbose: bool = False, jobs: int | None = None) -
         if not force and os.path.exists(obj) and os.path.getmtime(obj) >= max(os.path.getmtime(src), hm):
             return obj, False
         tmp = obj + f".tmp{os.getpid()}"
-        cmd = [cmd0] + FLAGS + ["-c", src, "-o", tmp]
+        cmd = [cmd0] + FLAGS + SOURCE_FLAGS.get(os.path.basename(src), []) + ["-c", src, "-o", tmp]
         r = subprocess.run(cmd, capture_output=True, text=True)
         if r.returncode != 0:
             raise RuntimeError(f"nvcc failed for {os.path.basename(src)}:\n{r.stderr[-4000:]}")

@@ -166,7 +166,9 @@ struct Ring {
 
 // MON: also return q2 (squared distance of this body to body 0) and d2[r] (squared
 // distance of this lane's pair in round r) for the monitor.
-template <int N, bool MON>
+// UNROLL: rounds unrolled (1: a loop, for callers bound to few registers; the FP64 pipe is the
+// bound either way).
+template <int N, bool MON, int UNROLL = Ring<N>::RF>
 __device__ __forceinline__ void ring_accjerk(const F64k &k, const double (&x)[3], const double (&v)[3], double m, int b, int base,
                                              double (&a)[3], double (&jk)[3], double &q2,
                                              double (&d2)[Ring<N>::RT > 0 ? Ring<N>::RT : 1]) {
@@ -176,7 +178,7 @@ __device__ __forceinline__ void ring_accjerk(const F64k &k, const double (&x)[3]
     jk[c] = 0.0;
   }
   q2 = 0.0;
-#pragma unroll
+#pragma unroll (UNROLL > 0 ? UNROLL : 1)
   for (int r = 1; r <= Ring<N>::RF; r++) {
     int p = b + r;
     if (p >= N) p -= N;

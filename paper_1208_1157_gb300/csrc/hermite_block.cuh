@@ -12,7 +12,9 @@
 // slot, a barrier, then takes the reactions of the pairs (b - r, b) from their slots.
 // Every unordered pair is evaluated once per evaluation, as in the warp ring (whose
 // accumulation order per body differs: own shares first here, then the reactions).
-// Systems are handed out per group as in bpl_hermite_stream (fixed steps only).
+// Systems are handed out per group as in bpl_hermite_stream (fixed steps only).  Used for the
+// printed corrector, whose steps are wholly FP64; the time-symmetric one's run in
+// hermite_bpl_ff.cuh, 3 to 4 times faster.
 #pragma once
 #include <algorithm>
 

@@ -55,6 +55,17 @@ __device__ __forceinline__ void fcorrect(const FCoef &C, const ff &a0, const ff 
   G = ff_norm(ff_fma_raw(C.h2_12, ff_neg(D), ff_mul_raw(C.hh, W)));
 }
 
+// The correction to a prediction (x + G, v + W) from D = a_k - a_0 - h j_0 and E = j_k - j_0:
+// u = hh D - h^2/12 E in v, y = hh u - h^2/12 D in x.
+__device__ __forceinline__ void fcorrect_delta(const FCoef &C, const ff &D, const ff &E, ff &y, ff &u) {
+  u = ff_fma_raw(ff_neg(C.h2_12), E, ff_mul_raw(C.hh, D));
+  y = ff_fma_raw(ff_neg(C.h2_12), D, ff_mul_raw(C.hh, u));
+}
+__device__ __forceinline__ void fcorrect_delta32(const FCoef &C, float D, float E, float &y, float &u) {
+  u = __fmaf_rn(C.hh.h, D, -C.h2_12.h * E);
+  y = __fmaf_rn(C.hh.h, u, -C.h2_12.h * D);
+}
+
 // Smallness conditions of a state: E = h^2 mu/r^3 (eta^2), S = bound on the perturbing
 // accelerations' rounding over 2^-45, V2 = |v|^2 of the body.  Level 0: FP64 steps; 1: pairs
 // carry the weights listed above; 2: eta < 0.0134 too, where the FP32 parts of
@@ -73,6 +84,19 @@ __device__ __forceinline__ bool frange(float r2) { return r2 > 0x1p-40f && r2 < 
 __device__ __forceinline__ bool fscale(double v, int lo, int hi) {
   const int e = (__double2hiint(v) & 0x7ff00000) >> 20;
   return e > 1023 + lo && e < 1023 + hi;
+}
+
+// ---------------------------------------------------------------- adaptive step (Eq. 5)
+// The Hermite propagator with the step of Sec. 4.3.2: dt = tau (sum_i |j_i|^2/|a_i|^2)^(-1/2)
+// from the values at the start of the step, clamped so that the last step lands on the
+// system's end time.  P.dt carries tau (its sign gives the direction).  A launch takes at
+// most P.max_steps (or 2^24) steps per system; a system that has not reached its end time
+// then stays ACTIVE.  The system-per-lane versions run on coordinates relative to body 0
+// like spl_hermite_body; Eq. 5 takes the inertial a and jerk rebuilt from them.
+constexpr int kAdaptiveStepCap = 1 << 24;
+
+__device__ __forceinline__ double adaptive_end(const BinView &B, const StepParams &P, int s) {
+  return B.t_end ? B.t_end[s] : (P.t_end_dev ? *P.t_end_dev : P.t_end);
 }
 
 // FP64 part of one planet's pull towards body 0: M = mu / |X|^3 and q2 = |X|^2; rho^3 and
@@ -119,6 +143,32 @@ __device__ __forceinline__ void fjerk_dir32(const ff (&x)[3], const ff (&v)[3], 
   const float c = -3.0f * rv * rho2;
 #pragma unroll
   for (int i = 0; i < 3; i++) w[i] = __fmaf_rn(c, x[i].h, v[i].h);
+}
+
+// Change of a pair's terms T = s x, Z = s (u + c x) (x, u its difference vectors, s = 1/|x|^3,
+// p = 1/|x|^2, c = -3 (x.u) p) when x, u move by d, e, in FP32: the algebraic difference, not a
+// linearisation, so its error is 2^-22 of the change itself.
+__device__ __forceinline__ void fpair_delta(const float (&x)[3], const float (&u)[3], const float (&d)[3],
+                                            const float (&e)[3], float s, float p, float c, float (&DT)[3],
+                                            float (&DZ)[3]) {
+  float xn[3], e2 = 0.0f, rv = 0.0f;
+#pragma unroll
+  for (int q = 0; q < 3; q++) {
+    e2 = __fmaf_rn(d[q], __fmaf_rn(2.0f, x[q], d[q]), e2);
+    xn[q] = x[q] + d[q];
+    rv = __fmaf_rn(d[q], u[q], __fmaf_rn(xn[q], e[q], rv));
+  }
+  e2 *= p;                                               // |x + d|^2 / |x|^2 - 1
+  const float f = __fmaf_rn(e2, e2, -e2);                // 1/(1 + e2) - 1
+  const float t = e2 * __fmaf_rn(1.875f, e2, -1.5f);     // (1 + e2)^(-3/2) - 1
+  const float dc = __fmaf_rn(c, f, __fmaf_rn(f, -3.0f * rv * p, -3.0f * rv * p));
+#pragma unroll
+  for (int q = 0; q < 3; q++) {
+    DT[q] = s * __fmaf_rn(t, xn[q], d[q]);
+    const float w = __fmaf_rn(c, x[q], u[q]);
+    const float dw = __fmaf_rn(c, d[q], __fmaf_rn(dc, xn[q], e[q]));
+    DZ[q] = s * __fmaf_rn(t, w + dw, dw);
+  }
 }
 
 // ---------------------------------------------------------------- system per lane
@@ -318,32 +368,10 @@ __device__ __forceinline__ void spl_eval_ff(const FMass<N> &F, const ff (&X)[N][
 template <int N>
 __device__ __forceinline__ void spl_delta(const FMass<N> &F, const SplGeo<N> &g, const float (&dX)[N][3],
                                           const float (&dV)[N][3], float (&DA)[N][3], float (&DJ)[N][3]) {
-  // one pair: x, u its difference vectors, d, e their changes; T = s x, Z = s (u + c x)
-  auto pair = [](const float (&x)[3], const float (&u)[3], const float (&d)[3], const float (&e)[3], float s, float p,
-                 float c, float (&DT)[3], float (&DZ)[3]) {
-    float xn[3], e2 = 0.0f, rv = 0.0f;
-#pragma unroll
-    for (int q = 0; q < 3; q++) {
-      e2 = __fmaf_rn(d[q], __fmaf_rn(2.0f, x[q], d[q]), e2);
-      xn[q] = x[q] + d[q];
-      rv = __fmaf_rn(d[q], u[q], __fmaf_rn(xn[q], e[q], rv));
-    }
-    e2 *= p;                                               // |x + d|^2 / |x|^2 - 1
-    const float f = __fmaf_rn(e2, e2, -e2);                // 1/(1 + e2) - 1
-    const float t = e2 * __fmaf_rn(1.875f, e2, -1.5f);     // (1 + e2)^(-3/2) - 1
-    const float dc = __fmaf_rn(c, f, __fmaf_rn(f, -3.0f * rv * p, -3.0f * rv * p));
-#pragma unroll
-    for (int q = 0; q < 3; q++) {
-      DT[q] = s * __fmaf_rn(t, xn[q], d[q]);
-      const float w = __fmaf_rn(c, x[q], u[q]);
-      const float dw = __fmaf_rn(c, d[q], __fmaf_rn(dc, xn[q], e[q]));
-      DZ[q] = s * __fmaf_rn(t, w + dw, dw);
-    }
-  };
   float T[N][3], Z[N][3];
 #pragma unroll
   for (int k = 1; k < N; k++) {
-    pair(g.X[k], g.V[k], dX[k], dV[k], g.s[0][k], g.p[0][k], g.c[0][k], T[k], Z[k]);
+    fpair_delta(g.X[k], g.V[k], dX[k], dV[k], g.s[0][k], g.p[0][k], g.c[0][k], T[k], Z[k]);
 #pragma unroll
     for (int q = 0; q < 3; q++) {
       DA[k][q] = -F.muf[k].h * T[k][q];
@@ -365,7 +393,7 @@ __device__ __forceinline__ void spl_delta(const FMass<N> &F, const SplGeo<N> &g,
         d[q] = dX[k][q] - dX[i][q];
         e[q] = dV[k][q] - dV[i][q];
       }
-      pair(x, u, d, e, g.s[i][k], g.p[i][k], g.c[i][k], t, z);
+      fpair_delta(x, u, d, e, g.s[i][k], g.p[i][k], g.c[i][k], t, z);
 #pragma unroll
       for (int q = 0; q < 3; q++) {
         DA[i][q] = __fmaf_rn(F.m[k].h, t[q] - T[k][q], DA[i][q]);
@@ -423,15 +451,12 @@ __device__ __forceinline__ int spl_hermite_delta_step(const F64k &kk, const FMas
   for (int k = 1; k < N; k++)
 #pragma unroll
     for (int c = 0; c < 3; c++) da[k][c] = DJ[k][c] = 0.0f;
-  // corrections to the prediction: dv = hh D - h^2/12 E, dx = hh dv - h^2/12 D
   for (int ic = 1; ic < n_corr; ic++) {
 #pragma unroll
     for (int k = 1; k < N; k++)
 #pragma unroll
       for (int c = 0; c < 3; c++) {
-        const float d = D[k][c].h + da[k][c], e = E[k][c].h + DJ[k][c];
-        dV[k][c] = __fmaf_rn(C.hh.h, d, -C.h2_12.h * e);
-        dX[k][c] = __fmaf_rn(C.hh.h, dV[k][c], -C.h2_12.h * d);
+        fcorrect_delta32(C, D[k][c].h + da[k][c], E[k][c].h + DJ[k][c], dX[k][c], dV[k][c]);
       }
     spl_delta<N>(F, g, dX, dV, da, DJ);
   }
@@ -439,9 +464,8 @@ __device__ __forceinline__ int spl_hermite_delta_step(const F64k &kk, const FMas
   for (int k = 1; k < N; k++)
 #pragma unroll
     for (int c = 0; c < 3; c++) {
-      const ff d = ff_make(D[k][c].h, D[k][c].l + da[k][c]), e = ff_make(E[k][c].h, E[k][c].l + DJ[k][c]);
-      const ff u = ff_fma_raw(ff_neg(C.h2_12), e, ff_mul_raw(C.hh, d));
-      const ff y = ff_fma_raw(ff_neg(C.h2_12), d, ff_mul_raw(C.hh, u));
+      ff y, u;
+      fcorrect_delta(C, ff_make(D[k][c].h, D[k][c].l + da[k][c]), ff_make(E[k][c].h, E[k][c].l + DJ[k][c]), y, u);
       dV[k][c] = u.h + u.l;
       dX[k][c] = y.h + y.l;
       x[k][c] = ff_addto(x[k][c], ff_add(G[k][c], y));
@@ -583,7 +607,7 @@ __device__ __forceinline__ int spl_monitor(const F64k &kk, const double (&x)[N][
 // evaluations carried from step to step, so that a system that stays at level 0 costs what an
 // FP64 kernel's does.
 template <int N, bool ADAPT, bool PRINTED>
-__device__ __noinline__ int spl_hermite_fp64_run(const F64k &kk, const double (&m)[N], const double (&kc)[N][N],
+static __device__ __noinline__ int spl_hermite_fp64_run(const F64k &kk, const double (&m)[N], const double (&kc)[N][N],
                                                  double eject2, double hh, int n_corr, int count, bool first,
                                                  double (&xs)[N][3], double (&vs)[N][3], double (&as)[N][3],
                                                  ff (&jb)[N][3], int &done, double &ts, double te, bool &reached) {
@@ -709,14 +733,14 @@ __device__ __forceinline__ int spl_ff_state(const F64k &kk, const FMass<N> &F, f
 // Both out of line, for what is not on the hot path (a step is some 3300 instructions, 53 KB:
 // the loops have to stay within the instruction cache).
 template <int N, bool STAR>
-__device__ __noinline__ int spl_ff_state_call(const F64k &kk, const FMass<N> &F, float hf, const double (&x)[N][3],
+static __device__ __noinline__ int spl_ff_state_call(const F64k &kk, const FMass<N> &F, float hf, const double (&x)[N][3],
                                               const double (&v)[N][3], double (&a0)[N][3], float (&da)[N][3],
                                               ff (&j0)[N][3], float (&q2)[N], float (&d2)[N][N], ff (&sa)[3],
                                               ff (&sj)[3]) {
   return spl_ff_state<N, STAR>(kk, F, hf, x, v, a0, da, j0, q2, d2, sa, sj);
 }
 template <int N, bool STAR>
-__device__ __noinline__ int spl_hermite_ff_step_call(const F64k &kk, const FMass<N> &F, const FCoef &C, float hf,
+static __device__ __noinline__ int spl_hermite_ff_step_call(const F64k &kk, const FMass<N> &F, const FCoef &C, float hf,
                                                      int n_corr, double (&x)[N][3], double (&v)[N][3],
                                                      double (&a0)[N][3], float (&da)[N][3], ff (&j0)[N][3],
                                                      float (&q2)[N], float (&d2)[N][N], ff (&sa)[3], ff (&sj)[3]) {
@@ -747,7 +771,7 @@ __device__ __forceinline__ FLimits<N> flimits(const double (&m)[N], double ce_fa
   return L;
 }
 template <int N>
-__device__ __noinline__ int spl_ff_monitor_fp64(const F64k &kk, const double (&x)[N][3], const double (&v)[N][3],
+static __device__ __noinline__ int spl_ff_monitor_fp64(const F64k &kk, const double (&x)[N][3], const double (&v)[N][3],
                                                 const double (&kc)[N][N], double eject2) {
   double q2[N], d2[N][N];
 #pragma unroll

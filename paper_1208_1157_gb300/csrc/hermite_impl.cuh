@@ -3,175 +3,11 @@
 #pragma once
 #include "hermite.cuh"
 #include "hermite_block.cuh"
+#include "hermite_bpl_ff.cuh"
 #include "hermite_ff.cuh"
 #include "kernels.h"
 
 namespace swarm {
-
-// ---------------------------------------------------------------- body per lane
-// One work unit = one warp's G = 32/N systems of a bin, integrated for the whole call.
-template <int N>
-__device__ __forceinline__ void bpl_hermite_body(const BinView &B, const StepParams &P, int unit) {
-  const bool printed = P.corr_form != 0;  // warp-uniform
-  using R = Ring<N>;
-  constexpr int G = R::G;
-  constexpr int RT = R::RT > 0 ? R::RT : 1;
-  const unsigned FULL = 0xffffffffu;
-  const int lane = threadIdx.x & 31;
-  int g = lane / N, b = lane - g * N;
-  const bool lane_ok = g < G;
-  if (!lane_ok) {  // spare lanes mirror group 0 so every shuffle stays well defined
-    g = 0;
-    b = lane - G * N;
-  }
-  const int base = g * N;
-  const int s0 = unit * G;
-  int s = s0 + g;
-  const bool sys_ok = lane_ok && s < B.S;
-  if (s >= B.S) s = s0;
-  const int SP = B.S_pad;
-
-  double x[3], v[3];
-#pragma unroll
-  for (int c = 0; c < 3; c++) {
-    x[c] = B.x[(size_t)(c * N + b) * SP + s];
-    v[c] = B.v[(size_t)(c * N + b) * SP + s];
-  }
-  const double m = B.m[(size_t)b * SP + s];
-  const double t0 = B.t[s];
-  const int st0 = B.status[s];
-  const double m0 = shfl(m, base);
-  const bool runnable = sys_ok && st0 <= SWARM_SYS_DONE;
-  const LaunchPlan plan = launch_plan(B, P, s, t0, runnable);
-  const int Ns = plan.N;
-  const int Nmax = __reduce_max_sync(FULL, Ns);
-  if (Nmax == 0) {
-    if (runnable && b == 0) B.status[s] = SWARM_SYS_DONE;
-    return;
-  }
-
-  // close-encounter coefficients of this lane's pairs (planet pairs only)
-  double kc[RT];
-#pragma unroll
-  for (int r = 1; r <= RT; r++) {
-    int p = b + r;
-    if (p >= N) p -= N;
-    double mp = shfl(m, base + p);
-    kc[r - 1] = (b != 0 && p != 0 && RT == R::RT) ? hill_kc(P.ce_factor, m, mp, m0) : 0.0;
-  }
-
-  double a0[3], j0[3], q2, d2[RT];
-  ring_accjerk<N, false>(P.fk, x, v, m, b, base, a0, j0, q2, d2);
-  const HCoef cdt = hcoef(P.dt);
-  const HCoef clast = hcoef(plan.h_last);
-  bool alive = runnable;
-  int steps_done = 0;
-
-  for (int k = 1; k <= Nmax; k++) {
-    const bool active = alive && (k <= Ns);
-    if (!__any_sync(FULL, active)) break;
-    const HCoef C = hsel(k == Ns && !plan.exact, clast, cdt);
-    // Eq. 3 predictor and the step-invariant parts of the corrector
-    double xk[3], vk[3], Xb[3], Vb[3];
-#pragma unroll
-    for (int c = 0; c < 3; c++) {
-      xk[c] = fma(j0[c], C.h3_6, fma(a0[c], C.h2_2, fma(v[c], C.h, x[c])));
-      vk[c] = fma(j0[c], C.h2_2, fma(a0[c], C.h, v[c]));
-      Vb[c] = fma(j0[c], C.h2_12, fma(a0[c], C.hh, v[c]));
-    }
-    PCoef PC;
-    if (printed) {
-      PC = pcoef(C.h);
-#pragma unroll
-      for (int c = 0; c < 3; c++) Xb[c] = fma(j0[c], PC.pj, fma(a0[c], PC.pa, xk[c]));
-    } else {
-#pragma unroll
-      for (int c = 0; c < 3; c++) Xb[c] = fma(a0[c], C.h2_12, fma(v[c], C.hh, x[c]));
-    }
-    // corrector passes (time-symmetric form of Eq. 4)
-    for (int ic = 0; ic < P.n_corr; ic++) {
-      double ak[3], jk[3];
-      ring_accjerk<N, false>(P.fk, xk, vk, m, b, base, ak, jk, q2, d2);
-#pragma unroll
-      for (int c = 0; c < 3; c++) vk[c] = fma(-C.h2_12, jk[c], fma(C.hh, ak[c], Vb[c]));
-      if (printed) {
-#pragma unroll
-        for (int c = 0; c < 3; c++) xk[c] = fma(PC.cj, jk[c], fma(PC.ca, ak[c], Xb[c]));
-      } else {
-#pragma unroll
-        for (int c = 0; c < 3; c++) xk[c] = fma(-C.h2_12, ak[c], fma(C.hh, vk[c], Xb[c]));
-      }
-    }
-    // third evaluation: next step's a0, j0 and the monitor's distances
-    double an[3], jn[3];
-    ring_accjerk<N, true>(P.fk, xk, vk, m, b, base, an, jn, q2, d2);
-    if (active) {
-#pragma unroll
-      for (int c = 0; c < 3; c++) {
-        x[c] = xk[c];
-        v[c] = vk[c];
-        a0[c] = an[c];
-        j0[c] = jn[c];
-      }
-      steps_done = k;
-    }
-    // monitor
-    const bool nf = nonfinite(x[0]) | nonfinite(x[1]) | nonfinite(x[2]) | nonfinite(v[0]) | nonfinite(v[1]) |
-                    nonfinite(v[2]);
-    const bool ej = (b != 0) && (P.eject2 > 0.0) && (q2 > P.eject2);
-    bool ce = false;
-#pragma unroll
-    for (int r = 1; r <= RT; r++) {
-      int p = b + r;
-      if (p >= N) p -= N;
-      double q2p = shfl(q2, base + p);
-      if (kc[r - 1] > 0.0 && close_encounter(P.fk, d2[r - 1], kc[r - 1], q2, q2p)) ce = true;
-    }
-    const unsigned gm = ((1u << N) - 1u) << base;
-    const unsigned bnf = __ballot_sync(FULL, active && nf) & gm;
-    const unsigned bej = __ballot_sync(FULL, active && ej) & gm;
-    const unsigned bce = __ballot_sync(FULL, active && ce) & gm;
-    const int code = bnf ? SWARM_SYS_NONFINITE : bej ? SWARM_SYS_EJECTED : bce ? SWARM_SYS_CLOSE_ENCOUNTER : 0;
-    if (active && code) {
-      const double tk = step_time(plan, k, t0, P.dt);
-      if (sys_ok) {
-#pragma unroll
-        for (int c = 0; c < 3; c++) {
-          B.x[(size_t)(c * N + b) * SP + s] = x[c];
-          B.v[(size_t)(c * N + b) * SP + s] = v[c];
-        }
-        if (b == 0) {
-          B.t[s] = tk;
-          B.status[s] = code;
-        }
-      }
-      alive = false;
-    }
-    if (P.log_interval > 0 && (k % P.log_interval) == 0) {
-      double e[4];
-      ring_energy<N>(x, v, m, b, base, e);
-      if (active && !code && b == 0 && sys_ok) write_log(P, B.gidx[s], step_time(plan, k, t0, P.dt), e);
-    }
-  }
-  if (alive && sys_ok) {
-    if (Ns > 0) {
-#pragma unroll
-      for (int c = 0; c < 3; c++) {
-        B.x[(size_t)(c * N + b) * SP + s] = x[c];
-        B.v[(size_t)(c * N + b) * SP + s] = v[c];
-      }
-    }
-    if (b == 0) {
-      if (Ns > 0) B.t[s] = step_time(plan, Ns, t0, P.dt);
-      B.status[s] = plan.full ? SWARM_SYS_DONE : SWARM_SYS_ACTIVE;
-    }
-  }
-  if (P.counters && sys_ok && b == 0 && steps_done > 0) {
-    constexpr unsigned long long NP = (unsigned long long)N * (N - 1) / 2;
-    atomicAdd(&P.counters[0], (unsigned long long)steps_done);
-    atomicAdd(&P.counters[1], NP * (1ull + (unsigned long long)steps_done * (P.n_corr + 1)));
-  }
-}
 
 // ---------------------------------------------------------------- system per lane
 // Each lane integrates one system in coordinates relative to body 0, X_k = x_k - x_0 and
@@ -282,174 +118,6 @@ __device__ __forceinline__ void spl_hermite_body(const BinView &B, const StepPar
     constexpr unsigned long long NP = (unsigned long long)N * (N - 1) / 2;
     atomicAdd(&P.counters[0], (unsigned long long)k);
     atomicAdd(&P.counters[1], NP * (1ull + (unsigned long long)k * (P.n_corr + 1)));
-  }
-}
-
-// ---------------------------------------------------------------- adaptive step (Eq. 5)
-// The Hermite propagator with the step of Sec. 4.3.2: dt = tau (sum_i |j_i|^2/|a_i|^2)^(-1/2)
-// from the values at the start of the step, clamped so that the last step lands on the
-// system's end time.  P.dt carries tau (its sign gives the direction).  A launch takes at
-// most P.max_steps (or 2^24) steps per system; a system that has not reached its end time
-// then stays ACTIVE.  The system-per-lane versions run on coordinates relative to body 0
-// like spl_hermite_body; Eq. 5 takes the inertial a and jerk rebuilt from them.
-constexpr int kAdaptiveStepCap = 1 << 24;
-
-__device__ __forceinline__ double adaptive_end(const BinView &B, const StepParams &P, int s) {
-  return B.t_end ? B.t_end[s] : (P.t_end_dev ? *P.t_end_dev : P.t_end);
-}
-
-template <int N>
-__device__ __forceinline__ void bpl_hermite_adaptive_body(const BinView &B, const StepParams &P, int unit) {
-  const bool printed = P.corr_form != 0;  // warp-uniform
-  using R = Ring<N>;
-  constexpr int G = R::G;
-  constexpr int RT = R::RT > 0 ? R::RT : 1;
-  const unsigned FULL = 0xffffffffu;
-  const int lane = threadIdx.x & 31;
-  int g = lane / N, b = lane - g * N;
-  const bool lane_ok = g < G;
-  if (!lane_ok) {
-    g = 0;
-    b = lane - G * N;
-  }
-  const int base = g * N;
-  const int s0 = unit * G;
-  int s = s0 + g;
-  const bool sys_ok = lane_ok && s < B.S;
-  if (s >= B.S) s = s0;
-  const int SP = B.S_pad;
-  double x[3], v[3];
-#pragma unroll
-  for (int c = 0; c < 3; c++) {
-    x[c] = B.x[(size_t)(c * N + b) * SP + s];
-    v[c] = B.v[(size_t)(c * N + b) * SP + s];
-  }
-  const double m = B.m[(size_t)b * SP + s];
-  const double t0 = B.t[s];
-  const int st0 = B.status[s];
-  const double m0 = shfl(m, base);
-  const bool runnable = sys_ok && st0 <= SWARM_SYS_DONE;
-  const double te = adaptive_end(B, P, s);
-  const double tau = fabs(P.dt), dir = P.dt > 0 ? 1.0 : -1.0;
-  bool alive = runnable && ((te - t0) * dir > 1e-12 * fmax(1.0, fabs(te)));
-  if (!__any_sync(FULL, alive)) {
-    if (runnable && b == 0) B.status[s] = SWARM_SYS_DONE;
-    return;
-  }
-  double kc[RT];
-#pragma unroll
-  for (int r = 1; r <= RT; r++) {
-    int p = b + r;
-    if (p >= N) p -= N;
-    double mp = shfl(m, base + p);
-    kc[r - 1] = (b != 0 && p != 0 && RT == R::RT) ? hill_kc(P.ce_factor, m, mp, m0) : 0.0;
-  }
-  double a0[3], j0[3], q2, d2[RT];
-  ring_accjerk<N, false>(P.fk, x, v, m, b, base, a0, j0, q2, d2);
-  const int cap = P.max_steps > 0 ? P.max_steps : kAdaptiveStepCap;
-  double t = t0;
-  int steps_done = 0, code = 0;
-  bool reached = false, ran = alive;
-  for (int k = 1; k <= cap; k++) {
-    if (!__any_sync(FULL, alive)) break;
-    // Eq. 5 over the system's bodies (group sum of this lane's |j|^2/|a|^2)
-    const double ratio = (j0[0] * j0[0] + j0[1] * j0[1] + j0[2] * j0[2]) / (a0[0] * a0[0] + a0[1] * a0[1] + a0[2] * a0[2]);
-    const double ssum = grp_sum<N>(ratio, b, base);
-    double h = tau * rsqrt(ssum);
-    const double rem = kmul(P.fk, ksub(P.fk, te, t), dir);
-    const bool last = h >= rem;
-    const bool bad = !(h > 0.0) || nonfinite(h);
-    h = kmul(P.fk, last ? rem : h, dir);
-    const HCoef C = hcoef(P.fk, h);
-    double xk[3], vk[3], Xb[3], Vb[3];
-#pragma unroll
-    for (int c = 0; c < 3; c++) {
-      xk[c] = fma(j0[c], C.h3_6, fma(a0[c], C.h2_2, fma(v[c], C.h, x[c])));
-      vk[c] = fma(j0[c], C.h2_2, fma(a0[c], C.h, v[c]));
-      Vb[c] = fma(j0[c], C.h2_12, fma(a0[c], C.hh, v[c]));
-    }
-    PCoef PC;
-    if (printed) {
-      PC = pcoef(C.h);
-#pragma unroll
-      for (int c = 0; c < 3; c++) Xb[c] = fma(j0[c], PC.pj, fma(a0[c], PC.pa, xk[c]));
-    } else {
-#pragma unroll
-      for (int c = 0; c < 3; c++) Xb[c] = fma(a0[c], C.h2_12, fma(v[c], C.hh, x[c]));
-    }
-    for (int ic = 0; ic < P.n_corr; ic++) {
-      double ak[3], jk[3];
-      ring_accjerk<N, false>(P.fk, xk, vk, m, b, base, ak, jk, q2, d2);
-#pragma unroll
-      for (int c = 0; c < 3; c++) vk[c] = fma(-C.h2_12, jk[c], fma(C.hh, ak[c], Vb[c]));
-      if (printed) {
-#pragma unroll
-        for (int c = 0; c < 3; c++) xk[c] = fma(PC.cj, jk[c], fma(PC.ca, ak[c], Xb[c]));
-      } else {
-#pragma unroll
-        for (int c = 0; c < 3; c++) xk[c] = fma(-C.h2_12, ak[c], fma(C.hh, vk[c], Xb[c]));
-      }
-    }
-    double an[3], jn[3];
-    ring_accjerk<N, true>(P.fk, xk, vk, m, b, base, an, jn, q2, d2);
-    const bool active = alive && !bad;
-    if (active) {
-#pragma unroll
-      for (int c = 0; c < 3; c++) {
-        x[c] = xk[c];
-        v[c] = vk[c];
-        a0[c] = an[c];
-        j0[c] = jn[c];
-      }
-      steps_done = k;
-      t = last ? te : kadd(P.fk, t, h);
-    }
-    const bool nf = nonfinite(x[0]) | nonfinite(x[1]) | nonfinite(x[2]) | nonfinite(v[0]) | nonfinite(v[1]) |
-                    nonfinite(v[2]);
-    const bool ej = (b != 0) && (P.eject2 > 0.0) && (q2 > P.eject2);
-    bool ce = false;
-#pragma unroll
-    for (int r = 1; r <= RT; r++) {
-      int p = b + r;
-      if (p >= N) p -= N;
-      double q2p = shfl(q2, base + p);
-      if (kc[r - 1] > 0.0 && close_encounter(P.fk, d2[r - 1], kc[r - 1], q2, q2p)) ce = true;
-    }
-    const unsigned gm = ((1u << N) - 1u) << base;
-    const unsigned bnf = __ballot_sync(FULL, alive && (nf || bad)) & gm;
-    const unsigned bej = __ballot_sync(FULL, active && ej) & gm;
-    const unsigned bce = __ballot_sync(FULL, active && ce) & gm;
-    const int c2 = bnf ? SWARM_SYS_NONFINITE : bej ? SWARM_SYS_EJECTED : bce ? SWARM_SYS_CLOSE_ENCOUNTER : 0;
-    if (alive && c2) {
-      code = c2;
-      alive = false;
-    } else if (active && last) {
-      reached = true;
-      alive = false;
-    }
-    if (P.log_interval > 0 && (k % P.log_interval) == 0) {
-      double e[4];
-      ring_energy<N>(x, v, m, b, base, e);
-      if (active && !c2 && b == 0 && sys_ok) write_log(P, B.gidx[s], t, e);
-    }
-  }
-  if (sys_ok && ran) {
-#pragma unroll
-    for (int c = 0; c < 3; c++) {
-      B.x[(size_t)(c * N + b) * SP + s] = x[c];
-      B.v[(size_t)(c * N + b) * SP + s] = v[c];
-    }
-    if (b == 0) {
-      B.t[s] = t;
-      B.status[s] = code ? code : (reached ? SWARM_SYS_DONE : SWARM_SYS_ACTIVE);
-    }
-  } else if (runnable && b == 0) {
-    B.status[s] = SWARM_SYS_DONE;  // already at its end time
-  }
-  if (P.counters && sys_ok && b == 0 && steps_done > 0) {
-    constexpr unsigned long long NP = (unsigned long long)N * (N - 1) / 2;
-    atomicAdd(&P.counters[0], (unsigned long long)steps_done);
-    atomicAdd(&P.counters[1], NP * (1ull + (unsigned long long)steps_done * (P.n_corr + 1)));
   }
 }
 
@@ -582,221 +250,10 @@ __device__ __forceinline__ void spl_hermite_adaptive_body(const BinView &B, cons
   });
 }
 
-// Body per lane with work handed out per system: each of the warp's G groups takes the
-// bin's next system as soon as its own one reached its end time or stopped (fixed steps:
-// stops and per-system end times; adaptive steps: step counts differ from system to
-// system).  A refill round loads the new systems and evaluates their a0, j0 (the other
-// groups re-evaluate their unchanged state, which gives the same values); per system
-// the arithmetic is that of bpl_hermite_body / bpl_hermite_adaptive_body.
-template <int N, bool ADAPT>
-__device__ __forceinline__ void bpl_hermite_stream(const BinView &B, const StepParams &P) {
-  const bool printed = P.corr_form != 0;  // warp-uniform
-  using R = Ring<N>;
-  constexpr int G = R::G;
-  constexpr int RT = R::RT > 0 ? R::RT : 1;
-  constexpr unsigned long long NP = (unsigned long long)N * (N - 1) / 2;
-  const unsigned FULL = 0xffffffffu;
-  const int lane = threadIdx.x & 31;
-  int g = lane / N, b = lane - g * N;
-  const bool lane_ok = g < G;
-  if (!lane_ok) {  // spare lanes mirror group 0 (same broadcasts, same state)
-    g = 0;
-    b = lane - G * N;
-  }
-  const int base = g * N;
-  const int SP = B.S_pad;
-  const unsigned gm = ((1u << N) - 1u) << base;
-  const double tau = fabs(P.dt), dir = P.dt > 0 ? 1.0 : -1.0;
-  const int cap = P.max_steps > 0 ? P.max_steps : kAdaptiveStepCap;
-  const HCoef cdt = hcoef(P.dt);
-
-  int s = 0;
-  bool has = false, exhausted = false;
-  double x[3] = {0.0, 0.0, 0.0}, v[3] = {0.0, 0.0, 0.0}, m = 1.0, a0[3], j0[3], kc[RT];
-  LaunchPlan plan;
-  plan.N = 0;
-  plan.full = 1;
-  plan.exact = 1;
-  plan.h_last = P.dt;
-  plan.t_end = P.t_end;
-  HCoef clast = cdt;  // coefficients of a shortened last step (fixed steps)
-  double t = 0.0, t0 = 0.0, te = 0.0;  // fixed steps: t is formed from t0 when needed
-  int steps = 0;
-#pragma unroll
-  for (int r = 0; r < RT; r++) kc[r] = 0.0;
-
-  for (;;) {
-    // ---- refill: groups without a system take the bin's next one
-    const bool need = !has && !exhausted;
-    if (__any_sync(FULL, need)) {
-      int sn = 0;
-      if (need && lane_ok && b == 0) sn = atomicAdd(P.work_next, 1);
-      sn = __shfl_sync(FULL, sn, base);
-      const int ss = stream_system(B, sn);
-      const bool take = need && ss >= 0;
-      if (need && ss < 0) exhausted = true;
-      if (take) {
-        s = ss;
-#pragma unroll
-        for (int c = 0; c < 3; c++) {
-          x[c] = B.x[(size_t)(c * N + b) * SP + s];
-          v[c] = B.v[(size_t)(c * N + b) * SP + s];
-        }
-        m = B.m[(size_t)b * SP + s];
-      }
-      const double m0 = shfl(m, base);
-#pragma unroll
-      for (int r = 1; r <= RT; r++) {
-        int p = b + r;
-        if (p >= N) p -= N;
-        double mp = shfl(m, base + p);
-        const double k = (b != 0 && p != 0 && RT == R::RT) ? hill_kc(P.ce_factor, m, mp, m0) : 0.0;
-        if (take) kc[r - 1] = k;
-      }
-      double an[3], jn[3], q2, d2[RT];
-      ring_accjerk<N, false>(P.fk, x, v, m, b, base, an, jn, q2, d2);
-      if (take) {
-#pragma unroll
-        for (int c = 0; c < 3; c++) {
-          a0[c] = an[c];
-          j0[c] = jn[c];
-        }
-        t0 = B.t[s];
-        t = t0;
-        steps = 0;
-        const bool runnable = B.status[s] <= SWARM_SYS_DONE;
-        bool go;
-        if (!ADAPT) {
-          plan = launch_plan(B, P, s, t0, runnable);
-          go = runnable && plan.N > 0;
-          clast = hcoef(plan.exact ? P.dt : plan.h_last);
-        } else {
-          te = adaptive_end(B, P, s);
-          go = runnable && ((te - t0) * dir > 1e-12 * fmax(1.0, fabs(te)));
-        }
-        has = go;
-        if (runnable && !go && lane_ok && b == 0) B.status[s] = SWARM_SYS_DONE;
-      }
-      continue;
-    }
-    if (!__any_sync(FULL, has)) break;
-
-    // ---- one step for every group holding a system
-    const bool alive = has;
-    HCoef C;
-    bool last, bad = false;
-    double h = 0.0;
-    if (!ADAPT) {
-      last = steps + 1 == plan.N;
-      C = hsel(last, clast, cdt);
-    } else {
-      const double ratio = (j0[0] * j0[0] + j0[1] * j0[1] + j0[2] * j0[2]) / (a0[0] * a0[0] + a0[1] * a0[1] + a0[2] * a0[2]);
-      const double ssum = grp_sum<N>(ratio, b, base);
-      h = tau * rsqrt(ssum);
-      const double rem = kmul(P.fk, ksub(P.fk, te, t), dir);
-      last = h >= rem;
-      bad = !(h > 0.0) || nonfinite(h);
-      h = kmul(P.fk, last ? rem : h, dir);
-      C = hcoef(P.fk, h);
-    }
-    double xk[3], vk[3], Xb[3], Vb[3];
-#pragma unroll
-    for (int c = 0; c < 3; c++) {
-      xk[c] = fma(j0[c], C.h3_6, fma(a0[c], C.h2_2, fma(v[c], C.h, x[c])));
-      vk[c] = fma(j0[c], C.h2_2, fma(a0[c], C.h, v[c]));
-      Vb[c] = fma(j0[c], C.h2_12, fma(a0[c], C.hh, v[c]));
-    }
-    PCoef PC;
-    if (printed) {
-      PC = pcoef(C.h);
-#pragma unroll
-      for (int c = 0; c < 3; c++) Xb[c] = fma(j0[c], PC.pj, fma(a0[c], PC.pa, xk[c]));
-    } else {
-#pragma unroll
-      for (int c = 0; c < 3; c++) Xb[c] = fma(a0[c], C.h2_12, fma(v[c], C.hh, x[c]));
-    }
-    double q2, d2[RT];
-    for (int ic = 0; ic < P.n_corr; ic++) {
-      double ak[3], jk[3];
-      ring_accjerk<N, false>(P.fk, xk, vk, m, b, base, ak, jk, q2, d2);
-#pragma unroll
-      for (int c = 0; c < 3; c++) vk[c] = fma(-C.h2_12, jk[c], fma(C.hh, ak[c], Vb[c]));
-      if (printed) {
-#pragma unroll
-        for (int c = 0; c < 3; c++) xk[c] = fma(PC.cj, jk[c], fma(PC.ca, ak[c], Xb[c]));
-      } else {
-#pragma unroll
-        for (int c = 0; c < 3; c++) xk[c] = fma(-C.h2_12, ak[c], fma(C.hh, vk[c], Xb[c]));
-      }
-    }
-    double an[3], jn[3];
-    ring_accjerk<N, true>(P.fk, xk, vk, m, b, base, an, jn, q2, d2);
-    const bool active = alive && !bad;
-    if (active) {
-#pragma unroll
-      for (int c = 0; c < 3; c++) {
-        x[c] = xk[c];
-        v[c] = vk[c];
-        a0[c] = an[c];
-        j0[c] = jn[c];
-      }
-      steps++;
-      if (ADAPT) t = last ? te : kadd(P.fk, t, h);
-    }
-    const bool nf = nonfinite(x[0]) | nonfinite(x[1]) | nonfinite(x[2]) | nonfinite(v[0]) | nonfinite(v[1]) |
-                    nonfinite(v[2]);
-    const bool ej = (b != 0) && (P.eject2 > 0.0) && (q2 > P.eject2);
-    bool ce = false;
-#pragma unroll
-    for (int r = 1; r <= RT; r++) {
-      int p = b + r;
-      if (p >= N) p -= N;
-      double q2p = shfl(q2, base + p);
-      if (kc[r - 1] > 0.0 && close_encounter(P.fk, d2[r - 1], kc[r - 1], q2, q2p)) ce = true;
-    }
-    const unsigned bnf = __ballot_sync(FULL, alive && (nf || bad)) & gm;
-    const unsigned bej = __ballot_sync(FULL, active && ej) & gm;
-    const unsigned bce = __ballot_sync(FULL, active && ce) & gm;
-    int code = bnf ? SWARM_SYS_NONFINITE : bej ? SWARM_SYS_EJECTED : bce ? SWARM_SYS_CLOSE_ENCOUNTER : 0;
-    if (!alive) code = 0;
-    const bool reached = active && last && !code;
-    const bool capped = ADAPT && active && steps >= cap;
-    const bool finish = alive && (code != 0 || reached || capped);
-    if (!ADAPT && (finish || (P.log_interval > 0 && active && (steps % P.log_interval) == 0)))
-      t = step_time(plan, steps, t0, P.dt);
-    if (P.log_interval > 0) {
-      const bool need_log = active && !code && (steps % P.log_interval) == 0;
-      if (__any_sync(FULL, need_log)) {
-        double e4[4];
-        ring_energy<N>(x, v, m, b, base, e4);
-        if (need_log && lane_ok && b == 0) write_log(P, B.gidx[s], t, e4);
-      }
-    }
-    if (finish && lane_ok) {
-#pragma unroll
-      for (int c = 0; c < 3; c++) {
-        B.x[(size_t)(c * N + b) * SP + s] = x[c];
-        B.v[(size_t)(c * N + b) * SP + s] = v[c];
-      }
-      if (b == 0) {
-        B.t[s] = t;
-        if (code) B.status[s] = code;
-        else if (ADAPT) B.status[s] = reached ? SWARM_SYS_DONE : SWARM_SYS_ACTIVE;
-        else B.status[s] = plan.full ? SWARM_SYS_DONE : SWARM_SYS_ACTIVE;
-        if (P.counters && steps > 0) {
-          atomicAdd(&P.counters[0], (unsigned long long)steps);
-          atomicAdd(&P.counters[1], NP * (1ull + (unsigned long long)steps * (P.n_corr + 1)));
-        }
-      }
-    }
-    if (finish) has = false;
-  }
-}
-
 // Out-of-line copies called by the multi-body-count dispatcher kernel.
 template <int N>
 __device__ __noinline__ void bpl_hermite_unit(const BinView &B, const StepParams &P, int unit) {
-  bpl_hermite_body<N>(B, P, unit);
+  bpl_hermite_body<N, false>(B, P, unit);
 }
 template <int N>
 __device__ __noinline__ void spl_hermite_unit(const BinView &B, const StepParams &P, int unit) {
@@ -804,7 +261,7 @@ __device__ __noinline__ void spl_hermite_unit(const BinView &B, const StepParams
 }
 template <int N>
 __device__ __noinline__ void bpl_hermite_adaptive_unit(const BinView &B, const StepParams &P, int unit) {
-  bpl_hermite_adaptive_body<N>(B, P, unit);
+  bpl_hermite_body<N, true>(B, P, unit);
 }
 template <int N>
 __device__ __noinline__ void spl_hermite_adaptive_unit(const BinView &B, const StepParams &P, int unit) {
@@ -814,7 +271,7 @@ __device__ __noinline__ void spl_hermite_adaptive_unit(const BinView &B, const S
 // Persistent kernel for one bin (one body count, one mapping): the unit body is inlined,
 // so registers are allocated for this n alone.  Warps pull unit indices from a counter.
 template <int MAP, int N, bool ADAPT = false>
-__global__ void __launch_bounds__(128, 2) hermite_uniform_kernel(BinView B, int nunits, StepParams P) {
+__global__ void __launch_bounds__(128, MAP == SWARM_MAP_BODY_PER_LANE ? 3 : 2) hermite_uniform_kernel(BinView B, int nunits, StepParams P) {
   if (ADAPT && MAP == SWARM_MAP_SYSTEM_PER_LANE) {  // work unit = system (per-lane refill)
     spl_hermite_adaptive_stream<N>(B, P);
     return;
@@ -854,11 +311,12 @@ cudaError_t launch_hermite_uniform_pick(const BinView &B, int nunits, const Step
     if (blocks) *blocks = hermite_uniform_blocks_n<MAP, N, true>();
     return grid > 0 ? launch_hermite_uniform_n<MAP, N, true>(B, nunits, P, grid, st) : cudaSuccess;
   }
-  // fixed steps, body per lane, n >= 5: systems packed across the CTA (hermite_block.cuh)
-  // when the bin fills a wave of those CTAs; a smaller bin's step latency is the limit,
-  // and the warp ring's shuffles are shorter than the block ring's barriers there
+  // the printed corrector's steps are FP64: body per lane, n >= 5, packed across the CTA
+  // (hermite_block.cuh) when the bin fills a wave of those CTAs; a smaller bin's step latency
+  // is the limit, and the warp ring's shuffles are shorter than the block ring's barriers
+  // there
   if constexpr (MAP == SWARM_MAP_BODY_PER_LANE && N >= kBlockRingMinN) {
-    if (block_ring_pays(B, N, BlockRing<N>::T, BlockRing<N>::CPS, P.concurrent != 0)) return launch_hermite_block_n<N>(B, nunits, P, grid, st, blocks);
+    if (P.corr_form && block_ring_pays(B, N, BlockRing<N>::T, BlockRing<N>::CPS, P.concurrent != 0)) return launch_hermite_block_n<N>(B, nunits, P, grid, st, blocks);
   }
   if (blocks) *blocks = hermite_uniform_blocks_n<MAP, N>();
   return grid > 0 ? launch_hermite_uniform_n<MAP, N>(B, nunits, P, grid, st) : cudaSuccess;
