@@ -15,9 +15,11 @@
 // busy), so three CTAs per SM (168 registers).  Per step of 5041 systems, wholly in FP64 ->
 // now: n = 3 6.5 -> 4.7 us, 5 20.7 -> 6.7, 8 52.3 -> 9.7, 11 89.4 -> 22.8, 15 120.8 -> 33.0
 // (packed over the CTA for n = 7, 11, 15 before); 65536 systems of 3..15 bodies over 100
-// steps: 69.2 -> 20.1 ms.  A step of 0.02 orbits (level 0), n = 8: 39.9 -> 57 us.
+// steps: 69.2 -> 18.3 ms.  A step of 0.02 orbits (level 0), n = 8: 39.9 -> 56 us.
+// 2048 systems of 16..32 bodies (one per warp, n a run-time value) over 50 steps: 13.6 -> 4.7 ms.
 #pragma once
 #include "hermite_ff.cuh"
+#include "hermite_wide.cuh"
 
 namespace swarm {
 
@@ -32,37 +34,42 @@ __device__ __forceinline__ ff shfl_ff(const ff &a, int src) {
   return ff_make(__shfl_sync(0xffffffffu, a.h, src), __shfl_sync(0xffffffffu, a.l, src));
 }
 
-// the ring over the N - 1 planets: RF rounds with reaction, and for an even number a last one
-// in which both lanes of a pair take their own share
+// A body's place in its group, and its masses.  N = 0: a group is the warp, of n bodies (16..32,
+// a run-time value).
 template <int N>
-struct RingP {
-  static constexpr int NP = N - 1;
-  static constexpr int RF = (NP - 1) / 2;
-  static constexpr bool HALF = NP % 2 == 0;
-  static constexpr int RT = RF + (HALF ? 1 : 0);
-  static constexpr int RA = RT > 0 ? RT : 1;
+struct BplBody {
+  int b, base, nn;
+  double m0;   // body 0's mass
+  ff m0f, mf;  // and this body's, as pairs
+  __device__ __forceinline__ int n() const { return N ? N : nn; }
+  __device__ __forceinline__ unsigned mask() const { return n() == 32 ? 0xffffffffu : ((1u << n()) - 1u) << base; }
+  // the ring over the n - 1 planets: RF rounds with reaction, and for an even number a last one in
+  // which both lanes of a pair take their own share (RT in all)
+  __device__ __forceinline__ int RF() const { return (n() - 2) / 2; }
+  __device__ __forceinline__ int RT() const { return (n() - 1) / 2; }
+  __device__ __forceinline__ int next(int r) const {  // lane r planets after b's
+    int p = (b > 0 ? b - 1 : 0) + r;
+    if (p >= n() - 1) p -= n() - 1;
+    return base + 1 + p;
+  }
+  __device__ __forceinline__ int prev(int r) const {
+    int p = (b > 0 ? b - 1 : 0) - r;
+    if (p < 0) p += n() - 1;
+    return base + 1 + p;
+  }
 };
 template <int N>
-constexpr int kRingUnroll = RingP<N>::RT <= 2 ? RingP<N>::RA : 1;
+constexpr int kRoundsA = N ? (N > 2 ? (N - 1) / 2 : 1) : kWideRounds;  // sizes of per-round arrays
 template <int N>
-__device__ __forceinline__ int ring_next(int base, int b, int r) {  // lane r planets after b's
-  int p = (b > 0 ? b - 1 : 0) + r;
-  if (p >= N - 1) p -= N - 1;
-  return base + 1 + p;
-}
-template <int N>
-__device__ __forceinline__ int ring_prev(int base, int b, int r) {
-  int p = (b > 0 ? b - 1 : 0) - r;
-  if (p < 0) p += N - 1;
-  return base + 1 + p;
-}
+constexpr int kRingUnroll = N && (N - 1) / 2 <= 2 ? kRoundsA<N> : 1;
+
 // sum over a group's lanes, valid in its first lane
 template <int N>
-__device__ __forceinline__ ff grp_sum_ff(ff t, int b) {
+__device__ __forceinline__ ff grp_sum_ff(const BplBody<N> &g, ff t) {
 #pragma unroll
-  for (int off = 1; off < N; off <<= 1) {
+  for (int off = 1; off < (N ? N : 32); off <<= 1) {
     ff o = ff_make(__shfl_down_sync(0xffffffffu, t.h, off), __shfl_down_sync(0xffffffffu, t.l, off));
-    if (b + off >= N) o = ff_make(0.0f, 0.0f);
+    if (g.b + off >= g.n()) o = ff_make(0.0f, 0.0f);
     t = ff_add_raw(t, o);
   }
   return ff_norm(t);
@@ -78,13 +85,6 @@ struct BplEval {
   bool range, near;
   float X[3], V[3], s, p, c;  // relative to body 0, for `bpl_delta`
 };
-template <int N>
-struct BplBody {
-  int b, base;
-  double m0;   // body 0's mass
-  ff m0f, mf;  // and this body's, as pairs
-};
-
 // FULL: body 0's pull in FP64 from x, the perturbers' jerks in pairs; else everything from the
 // pairs xf, those jerks in FP32.  STATE: the guard's terms too, and whether a pair is near the
 // close-encounter limit of `kcf` (indexed by round).  With more than two rounds they are a loop,
@@ -93,7 +93,7 @@ struct BplBody {
 template <int N, bool FULL, bool STATE>
 __device__ __forceinline__ void bpl_eval_ff(const F64k &k, const BplBody<N> &g, const double (&x)[3], const ff (&xf)[3],
                                             const ff (&v)[3], const float *kcf, BplEval<N> &R) {
-  using RP = RingP<N>;
+  constexpr int KS = N ? 1 : 32;  // stride of kcf
   ff X[3], V[3], rho3, rho2, w[3], T[3], Z[3];
   const bool star = g.b == 0;
 #pragma unroll
@@ -137,8 +137,8 @@ __device__ __forceinline__ void bpl_eval_ff(const F64k &k, const BplBody<N> &g, 
     R.S = 0.0f;
   }
 #pragma unroll kRingUnroll<N>
-  for (int r = 1; r <= RP::RT; r++) {
-    const int p = ring_next<N>(g.base, g.b, r), q = ring_prev<N>(g.base, g.b, r);
+  for (int r = 1; r <= g.RT(); r++) {
+    const int p = g.next(r), q = g.prev(r);
     ff dx[3], u[3], z[3], s3, s2;
 #pragma unroll
     for (int c = 0; c < 3; c++) dx[c] = ff_sub_raw(shfl_ff(X[c], p), X[c]);
@@ -177,10 +177,10 @@ __device__ __forceinline__ void bpl_eval_ff(const F64k &k, const BplBody<N> &g, 
       const float t = R.q2 + __shfl_sync(0xffffffffu, R.q2, p);
       sg = s3.h * (1.41422f * t) * rsqrtf(t);
       R.S = __fmaf_rn(mp.h, sg, R.S);
-      R.near |= !(r2.h >= kcf[r - 1] * t);
+      R.near |= !(r2.h >= kcf[(r - 1) * KS] * t);
       R.range = R.range && frange(r2.h);
     }
-    if (r <= RP::RF) {  // the pair that lane q evaluated with this one
+    if (r <= g.RF()) {  // the pair that lane q evaluated with this one
       const ff mq = ff_neg(shfl_ff(g.mf, q));
 #pragma unroll
       for (int c = 0; c < 3; c++) {
@@ -194,7 +194,7 @@ __device__ __forceinline__ void bpl_eval_ff(const F64k &k, const BplBody<N> &g, 
   const ff mm = star ? ff_make(0.0f, 0.0f) : g.mf;
 #pragma unroll
   for (int c = 0; c < 3; c++) {
-    const ff sa = grp_sum_ff<N>(ff_mul(mm, T[c]), g.b), sj = grp_sum_ff<N>(ff_mul(mm, Z[c]), g.b);
+    const ff sa = grp_sum_ff<N>(g, ff_mul(mm, T[c])), sj = grp_sum_ff<N>(g, ff_mul(mm, Z[c]));
     const ff a = FULL ? ff_norm(R.P[c]) : ff_fma(ff_neg(g.m0f), T[c], R.P[c]);
     const ff j = ff_fma(ff_neg(g.m0f), Z[c], Q[c]);
     R.P[c] = ff_sel(star, sa, a);
@@ -207,18 +207,18 @@ __device__ __forceinline__ int bpl_level(const BplBody<N> &g, const BplEval<N> &
   int lv = 2;
   if (g.b != 0) lv = R.range ? fguard(hf, hf * hf * R.e1, R.S, R.V2) : 0;
   if (!ok) lv = 0;
-  const unsigned gm = ((1u << N) - 1u) << g.base;
+  const unsigned gm = g.mask();
   const unsigned n0 = __ballot_sync(0xffffffffu, lv == 0) & gm, n1 = __ballot_sync(0xffffffffu, lv == 1) & gm;
   return n0 ? 0 : n1 ? 1 : 2;
 }
 
 // sum of a float over a group's lanes, valid in its first lane
 template <int N>
-__device__ __forceinline__ float grp_sum32(float t, int b) {
+__device__ __forceinline__ float grp_sum32(const BplBody<N> &g, float t) {
 #pragma unroll
-  for (int off = 1; off < N; off <<= 1) {
+  for (int off = 1; off < (N ? N : 32); off <<= 1) {
     const float o = __shfl_down_sync(0xffffffffu, t, off);
-    t += b + off < N ? o : 0.0f;
+    t += g.b + off < g.n() ? o : 0.0f;
   }
   return t;
 }
@@ -227,7 +227,6 @@ __device__ __forceinline__ float grp_sum32(float t, int b) {
 template <int N>
 __device__ __forceinline__ void bpl_delta(const BplBody<N> &g, const BplEval<N> &R, const float (&dX)[3],
                                           const float (&dV)[3], float (&DA)[3], float (&DJ)[3]) {
-  using RP = RingP<N>;
   const unsigned FULL = 0xffffffffu;
   const bool star = g.b == 0;
   float d[3], e[3], T[3], Z[3], P[3], Q[3];
@@ -239,8 +238,8 @@ __device__ __forceinline__ void bpl_delta(const BplBody<N> &g, const BplEval<N> 
   }
   fpair_delta(R.X, R.V, d, e, R.s, R.p, R.c, T, Z);
 #pragma unroll kRingUnroll<N>
-  for (int r = 1; r <= RP::RT; r++) {
-    const int p = ring_next<N>(g.base, g.b, r), q = ring_prev<N>(g.base, g.b, r);
+  for (int r = 1; r <= g.RT(); r++) {
+    const int p = g.next(r), q = g.prev(r);
     float x[3], u[3], dd[3], ee[3], t[3], z[3];
     const float mp = __shfl_sync(FULL, g.mf.h, p);
 #pragma unroll
@@ -259,7 +258,7 @@ __device__ __forceinline__ void bpl_delta(const BplBody<N> &g, const BplEval<N> 
       P[c] = __fmaf_rn(mp, t[c], P[c]);
       Q[c] = __fmaf_rn(mp, z[c], Q[c]);
     }
-    if (r <= RP::RF) {
+    if (r <= g.RF()) {
       const float mq = -__shfl_sync(FULL, g.mf.h, q);
 #pragma unroll
       for (int c = 0; c < 3; c++) {
@@ -270,8 +269,8 @@ __device__ __forceinline__ void bpl_delta(const BplBody<N> &g, const BplEval<N> 
   }
 #pragma unroll
   for (int c = 0; c < 3; c++) {
-    const float sa = grp_sum32<N>(star ? 0.0f : __fmul_rn(g.mf.h, T[c]), g.b);
-    const float sj = grp_sum32<N>(star ? 0.0f : __fmul_rn(g.mf.h, Z[c]), g.b);
+    const float sa = grp_sum32<N>(g, star ? 0.0f : __fmul_rn(g.mf.h, T[c]));
+    const float sj = grp_sum32<N>(g, star ? 0.0f : __fmul_rn(g.mf.h, Z[c]));
     DA[c] = star ? sa : __fmaf_rn(-g.m0f.h, T[c], P[c]);
     DJ[c] = star ? sj : __fmaf_rn(-g.m0f.h, Z[c], Q[c]);
   }
@@ -333,28 +332,46 @@ static __device__ __noinline__ void bpl_eval_ff_call(const F64k &k, const BplBod
 }
 
 // ---------------------------------------------------------------- FP64 steps (guard not met)
-// Out of line; every lane of the warp takes part in the shuffles.
+// Out of line; every lane of the warp takes part in the shuffles.  kc, d2: per round of the ring
+// over all n bodies, in registers' place (local memory) or, for N = 0, this lane's column of
+// shared memory.
 template <int N>
-static __device__ __noinline__ void bpl_fp64_eval(const F64k &k, const double (&x)[3], const double (&v)[3], double m, int b,
-                                           int base, double (&a)[3], double (&j)[3], double &q2,
-                                           double (&d2)[Ring<N>::RT > 0 ? Ring<N>::RT : 1]) {
-  double a_[3], j_[3], q_, d_[Ring<N>::RT > 0 ? Ring<N>::RT : 1];
-  ring_accjerk<N, true, 1>(k, x, v, m, b, base, a_, j_, q_, d_);
+struct BplRounds {
+  static constexpr int RT = Ring<N>::RT > 0 ? Ring<N>::RT : 1;
+  double kc[RT], d2[RT];
+  __device__ __forceinline__ double &kcr(int r) { return kc[r - 1]; }
+  __device__ __forceinline__ double &d2r(int r) { return d2[r - 1]; }
+};
+template <>
+struct BplRounds<0> {
+  double *kc, *d2;
+  __device__ __forceinline__ double &kcr(int r) { return kc[(r - 1) * 32]; }
+  __device__ __forceinline__ double &d2r(int r) { return d2[(r - 1) * 32]; }
+};
+template <int N>
+static __device__ __noinline__ void bpl_fp64_eval(const F64k &k, const double (&x)[3], const double (&v)[3], double m,
+                                                  const BplBody<N> &g, double (&a)[3], double (&j)[3], double &q2,
+                                                  BplRounds<N> &rd) {
+  double a_[3], j_[3], q_;
+  if constexpr (N == 0) {
+    wring_accjerk<true, 1>(k, x, v, m, g.b, wide_ring(g.nn), a_, j_, q_, rd.d2, 0);
+  } else {
+    ring_accjerk<N, true, 1>(k, x, v, m, g.b, g.base, a_, j_, q_, rd.d2);
+  }
 #pragma unroll
   for (int c = 0; c < 3; c++) {
     a[c] = a_[c];
     j[c] = j_[c];
   }
   q2 = q_;
-#pragma unroll
-  for (int r = 0; r < Ring<N>::RT; r++) d2[r] = d_[r];
 }
 template <int N>
-static __device__ __noinline__ void bpl_fp64_advance(const F64k &k, double h, int n_corr, bool printed, double m, int b,
-                                              int base, const double (&a0)[3], const double (&j0)[3], double (&x)[3],
-                                              double (&v)[3]) {
+static __device__ __noinline__ void bpl_fp64_advance(const F64k &k, double h, int n_corr, bool printed, double m,
+                                                     const BplBody<N> &g, const double (&a0)[3],
+                                                     const double (&j0)[3], double (&x)[3], double (&v)[3],
+                                                     BplRounds<N> &rd) {
   const HCoef C = hcoef(h);
-  double xk[3], vk[3], Xb[3], Vb[3], q2, d2[Ring<N>::RT > 0 ? Ring<N>::RT : 1];
+  double xk[3], vk[3], Xb[3], Vb[3], q2;
   // Eq. 3 predictor and the step-invariant parts of the corrector
 #pragma unroll
   for (int c = 0; c < 3; c++) {
@@ -374,7 +391,7 @@ static __device__ __noinline__ void bpl_fp64_advance(const F64k &k, double h, in
 #pragma unroll 1
   for (int ic = 0; ic < n_corr; ic++) {
     double ak[3], jk[3];
-    bpl_fp64_eval<N>(k, xk, vk, m, b, base, ak, jk, q2, d2);
+    bpl_fp64_eval<N>(k, xk, vk, m, g, ak, jk, q2, rd);
 #pragma unroll
     for (int c = 0; c < 3; c++) vk[c] = fma(-C.h2_12, jk[c], fma(C.hh, ak[c], Vb[c]));
     if (printed) {
@@ -399,28 +416,28 @@ static __device__ __noinline__ void bpl_fp64_advance(const F64k &k, double h, in
 // system, or -1 (every lane calls it).  A refill round loads the new systems and evaluates
 // them (the other groups re-evaluate their unchanged state and keep what they have).
 template <int N, bool ADAPT, class Take>
-__device__ __forceinline__ void bpl_hermite_run(const BinView &B, const StepParams &P, Take take) {
+__device__ __forceinline__ void bpl_hermite_run(const BinView &B, const StepParams &P, BplRounds<N> &rd, float *kcf,
+                                                Take take) {
+  constexpr int KS = N ? 1 : 32;
   const bool printed = P.corr_form != 0;  // warp-uniform
   const bool carry = B.S >= kCarryMinSystems;
-  using R64 = Ring<N>;
-  using RP = RingP<N>;
-  constexpr int G = R64::G;
-  constexpr int RT = R64::RT > 0 ? R64::RT : 1;
-  constexpr unsigned long long NP = (unsigned long long)N * (N - 1) / 2;
+  BplBody<N> g;
+  g.nn = B.n;
+  const int n = g.n(), G = N ? 32 / n : 1;
+  const int rt = n / 2;  // rounds of the ring over all n bodies
   const unsigned FULL = 0xffffffffu;
   const int lane = threadIdx.x & 31;
-  BplBody<N> g;
-  int grp = lane / N;
-  g.b = lane - grp * N;
+  int grp = lane / n;
+  g.b = lane - grp * n;
   const bool lane_ok = grp < G;
   if (!lane_ok) {  // spare lanes mirror group 0 (same broadcasts, same state)
     grp = 0;
-    g.b = lane - G * N;
+    g.b = lane - G * n;
   }
-  g.base = grp * N;
+  g.base = grp * n;
   const int b = g.b;
   const int SP = B.S_pad;
-  const unsigned gm = ((1u << N) - 1u) << g.base;
+  const unsigned gm = g.mask();
   const double dir = P.dt > 0 ? 1.0 : -1.0;
   const int cap = P.max_steps > 0 ? P.max_steps : kAdaptiveStepCap;
   const ff tau = ff_from(fabs(P.dt));
@@ -431,8 +448,8 @@ __device__ __forceinline__ void bpl_hermite_run(const BinView &B, const StepPara
   // the state's acceleration is a0 + da; j0: FP64, or (level > 0) the bits of a pair
   double x[3] = {0.0, 0.0, 0.0}, v[3] = {0.0, 0.0, 0.0}, m = 1.0, a0[3] = {0.0, 0.0, 0.0}, j0[3] = {0.0, 0.0, 0.0};
   float da[3] = {0.0f, 0.0f, 0.0f};
-  double kc[RT];            // FP64 ring's close-encounter coefficients
-  float kcf[RP::RA];        // the planets' ring's, doubled and rounded up
+  // rd.kc: close-encounter coefficients of the FP64 ring; kcf: the planets' ring's, doubled and
+  // rounded up
   LaunchPlan plan;
   plan.N = 0;
   plan.full = 1;
@@ -443,10 +460,8 @@ __device__ __forceinline__ void bpl_hermite_run(const BinView &B, const StepPara
   ff h = ff_make(0.0f, 0.0f);          // ADAPT: length of the next step of a group in pairs
   g.m0 = 1.0;
   g.m0f = g.mf = ff_make(1.0f, 0.0f);
-#pragma unroll
-  for (int r = 0; r < RT; r++) kc[r] = 0.0;
-#pragma unroll
-  for (int r = 0; r < RP::RA; r++) kcf[r] = 0.0f;
+  for (int r = 1; r <= rt; r++) rd.kcr(r) = 0.0;
+  for (int r = 1; r <= g.RT(); r++) kcf[(r - 1) * KS] = 0.0f;
   auto to_bits = [](const ff &f) { return __hiloint2double(__float_as_int(f.h), __float_as_int(f.l)); };
   auto to_pair = [](double d) { return ff_make(__int_as_float(__double2hiint(d)), __int_as_float(__double2loint(d))); };
 
@@ -458,7 +473,7 @@ __device__ __forceinline__ void bpl_hermite_run(const BinView &B, const StepPara
       A[c] = ff_from(an[c]);
       A[c] = ff_norm(ff_make(A[c].h, A[c].l + dn[c]));
     }
-    const ff sum = shfl_ff(grp_sum_ff<N>(ff_div(ff_norm2(J), ff_norm2(A)), b), g.base);
+    const ff sum = shfl_ff(grp_sum_ff<N>(g, ff_div(ff_norm2(J), ff_norm2(A))), g.base);
     return ff_mul(tau, ff_rsqrt(sum));
   };
 
@@ -473,26 +488,24 @@ __device__ __forceinline__ void bpl_hermite_run(const BinView &B, const StepPara
         s = ss;
 #pragma unroll
         for (int c = 0; c < 3; c++) {
-          x[c] = B.x[(size_t)(c * N + b) * SP + s];
-          v[c] = B.v[(size_t)(c * N + b) * SP + s];
+          x[c] = B.x[(size_t)(c * n + b) * SP + s];
+          v[c] = B.v[(size_t)(c * n + b) * SP + s];
         }
         m = B.m[(size_t)b * SP + s];
       }
       const double m0 = shfl(m, g.base);
       const bool sc = (__ballot_sync(FULL, !fscale(m, -60, 40)) & gm) == 0 && fscale(P.dt, -60, 40);
-#pragma unroll
-      for (int r = 1; r <= RT; r++) {
+      for (int r = 1; r <= rt; r++) {
         int p = b + r;
-        if (p >= N) p -= N;
+        if (p >= n) p -= n;
         const double mp = shfl(m, g.base + p);
-        const double kk = (b != 0 && p != 0 && RT == R64::RT) ? hill_kc(P.ce_factor, m, mp, m0) : 0.0;
-        if (got) kc[r - 1] = kk;
+        const double kk = (b != 0 && p != 0) ? hill_kc(P.ce_factor, m, mp, m0) : 0.0;
+        if (got) rd.kcr(r) = kk;
       }
-#pragma unroll
-      for (int r = 1; r <= RP::RT; r++) {
-        const double mp = shfl(m, ring_next<N>(g.base, b, r));
+      for (int r = 1; r <= g.RT(); r++) {
+        const double mp = shfl(m, g.next(r));
         const float kk = 2.004f * (float)hill_kc(P.ce_factor, m, mp, m0);
-        if (got) kcf[r - 1] = kk;
+        if (got) kcf[(r - 1) * KS] = kk;
       }
       if (got) {
         scaled = sc;
@@ -520,8 +533,8 @@ __device__ __forceinline__ void bpl_hermite_run(const BinView &B, const StepPara
       }
       const int lv = bpl_level<N>(g, E, hf, sc2 && hf > 0.0f && !printed);
       if (__any_sync(FULL, got && !lv)) {
-        double a_[3], j_[3], q_, d_[RT];
-        bpl_fp64_eval<N>(P.fk, x, v, m, b, g.base, a_, j_, q_, d_);
+        double a_[3], j_[3], q_;
+        bpl_fp64_eval<N>(P.fk, x, v, m, g, a_, j_, q_, rd);
         if (!lv)
 #pragma unroll
           for (int c = 0; c < 3; c++) {
@@ -575,7 +588,9 @@ __device__ __forceinline__ void bpl_hermite_run(const BinView &B, const StepPara
       double hs = ff_double(h);
       if (__any_sync(FULL, alive && !kind)) {
         const double ratio = (j0[0] * j0[0] + j0[1] * j0[1] + j0[2] * j0[2]) / (a0[0] * a0[0] + a0[1] * a0[1] + a0[2] * a0[2]);
-        const double ssum = grp_sum<N>(ratio, b, g.base);
+        double ssum;
+        if constexpr (N == 0) ssum = warp_sum(lane_ok ? ratio : 0.0);
+        else ssum = grp_sum<N>(ratio, b, g.base);
         if (!kind) hs = fabs(P.dt) * rsqrt(ssum);
       }
       const double rem = kmul(P.fk, ksub(P.fk, te, t), dir);
@@ -613,7 +628,7 @@ __device__ __forceinline__ void bpl_hermite_run(const BinView &B, const StepPara
           xn[c] = x[c];
           vn[c] = v[c];
         }
-        bpl_fp64_advance<N>(P.fk, hd, P.n_corr, printed, m, b, g.base, a0, j0, xn, vn);
+        bpl_fp64_advance<N>(P.fk, hd, P.n_corr, printed, m, g, a0, j0, xn, vn, rd);
         if (active && kind == 0)
 #pragma unroll
           for (int c = 0; c < 3; c++) {
@@ -725,8 +740,8 @@ __device__ __forceinline__ void bpl_hermite_run(const BinView &B, const StepPara
     if (carry && kind == 2 && !lv) near = true;
     int code = 0;
     if (__any_sync(FULL, alive && near)) {  // in FP64: a0, j0 of groups that need them, the exact tests
-      double a_[3], j_[3], q2, d2[RT];
-      bpl_fp64_eval<N>(P.fk, x, v, m, b, g.base, a_, j_, q2, d2);
+      double a_[3], j_[3], q2;
+      bpl_fp64_eval<N>(P.fk, x, v, m, g, a_, j_, q2, rd);
       if (!lv)
 #pragma unroll
         for (int c = 0; c < 3; c++) {
@@ -738,12 +753,12 @@ __device__ __forceinline__ void bpl_hermite_run(const BinView &B, const StepPara
                       nonfinite(v[2]);
       const bool ej = (b != 0) && (P.eject2 > 0.0) && (q2 > P.eject2);
       bool ce = false;
-#pragma unroll
-      for (int r = 1; r <= RT; r++) {
+      for (int r = 1; r <= rt; r++) {
         int p = b + r;
-        if (p >= N) p -= N;
+        if (p >= n) p -= n;
         const double q2p = shfl(q2, g.base + p);
-        if (kc[r - 1] > 0.0 && close_encounter(P.fk, d2[r - 1], kc[r - 1], q2, q2p)) ce = true;
+        const double kc = rd.kcr(r);
+        if (kc > 0.0 && close_encounter(P.fk, rd.d2r(r), kc, q2, q2p)) ce = true;
       }
       const unsigned bnf = __ballot_sync(FULL, alive && (nf || bad)) & gm;
       const unsigned bej = __ballot_sync(FULL, active && ej) & gm;
@@ -774,15 +789,16 @@ __device__ __forceinline__ void bpl_hermite_run(const BinView &B, const StepPara
       const bool need_log = active && !code && (steps % P.log_interval) == 0;
       if (__any_sync(FULL, need_log)) {
         double e4[4];
-        ring_energy<N>(x, v, m, b, g.base, e4);
+        if constexpr (N == 0) wring_energy(x, v, m, b, lane_ok, wide_ring(n), e4);
+        else ring_energy<N>(x, v, m, b, g.base, e4);
         if (need_log && lane_ok && b == 0) write_log(P, B.gidx[s], t, e4);
       }
     }
     if (finish && lane_ok) {
 #pragma unroll
       for (int c = 0; c < 3; c++) {
-        B.x[(size_t)(c * N + b) * SP + s] = x[c];
-        B.v[(size_t)(c * N + b) * SP + s] = v[c];
+        B.x[(size_t)(c * n + b) * SP + s] = x[c];
+        B.v[(size_t)(c * n + b) * SP + s] = v[c];
       }
       if (b == 0) {
         B.t[s] = t;
@@ -791,6 +807,7 @@ __device__ __forceinline__ void bpl_hermite_run(const BinView &B, const StepPara
         else B.status[s] = plan.full ? SWARM_SYS_DONE : SWARM_SYS_ACTIVE;
         if (P.counters && steps > 0) {
           atomicAdd(&P.counters[0], (unsigned long long)steps);
+          const unsigned long long NP = (unsigned long long)n * (n - 1) / 2;
           atomicAdd(&P.counters[1], NP * (1ull + (unsigned long long)steps * (P.n_corr + 1)));
         }
       }
@@ -801,7 +818,9 @@ __device__ __forceinline__ void bpl_hermite_run(const BinView &B, const StepPara
 // the bin's next systems, one by one
 template <int N, bool ADAPT>
 __device__ __forceinline__ void bpl_hermite_stream(const BinView &B, const StepParams &P) {
-  bpl_hermite_run<N, ADAPT>(B, P, [&](bool need, bool leader, int base) {
+  BplRounds<N> rd;
+  float kcf[kRoundsA<N>];
+  bpl_hermite_run<N, ADAPT>(B, P, rd, kcf, [&](bool need, bool leader, int base) {
     int sn = 0;
     if (need && leader) sn = atomicAdd(P.work_next, 1);
     sn = __shfl_sync(0xffffffffu, sn, base);
@@ -812,10 +831,29 @@ __device__ __forceinline__ void bpl_hermite_stream(const BinView &B, const StepP
 template <int N, bool ADAPT>
 __device__ __forceinline__ void bpl_hermite_body(const BinView &B, const StepParams &P, int unit) {
   bool taken = false;
-  bpl_hermite_run<N, ADAPT>(B, P, [&](bool, bool, int base) {
+  BplRounds<N> rd;
+  float kcf[kRoundsA<N>];
+  bpl_hermite_run<N, ADAPT>(B, P, rd, kcf, [&](bool, bool, int base) {
     const int s = taken ? -1 : unit * (32 / N) + base / N;
     taken = true;
     return s < B.S ? s : -1;
+  });
+}
+
+// systems of 16..32 bodies, one per warp; shared memory of the warp: kc, d2 [16][32] FP64, kcf
+// [16][32] FP32
+template <bool ADAPT>
+__device__ __forceinline__ void wide_hermite_stream(const BinView &B, const StepParams &P, double *kc, double *d2,
+                                                    float *kcf) {
+  const int lane = threadIdx.x & 31;
+  BplRounds<0> rd;
+  rd.kc = kc + lane;
+  rd.d2 = d2 + lane;
+  bpl_hermite_run<0, ADAPT>(B, P, rd, kcf + lane, [&](bool need, bool leader, int base) {
+    int sn = 0;
+    if (need && leader) sn = atomicAdd(P.work_next, 1);
+    sn = __shfl_sync(0xffffffffu, sn, base);
+    return stream_system(B, sn);
   });
 }
 
