@@ -22,8 +22,8 @@ LIB = os.path.join(OUT, "libswarm_gb300.so")
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 # register cap of device functions that are called out of line (kernels have their launch bounds):
 # the body-per-lane Hermite kernels run three CTAs of 128 threads per SM
-SOURCE_FLAGS = {"hermite_uniform_bpl_a.cu": ["-maxrregcount", "168"], "hermite_uniform_bpl_b.cu": ["-maxrregcount", "168"],
-                "hermite_wide.cu": ["-maxrregcount", "168"]}
+SOURCE_FLAGS = {f: ["-maxrregcount", "168"] for f in ("hermite_uniform_bpl_a.cu", "hermite_uniform_bpl_b.cu", "hermite_wide.cu",
+                                                       "rkck_fixed_b.cu", "rkck_adaptive_b.cu")}
 FLAGS = ARCH + ["-O3", "-std=c++17", "-lineinfo", "-rdc=true", "-Xcompiler", "-fPIC", "-I", INCLUDE]
 
 

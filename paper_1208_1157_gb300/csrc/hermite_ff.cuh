@@ -801,6 +801,32 @@ __device__ __forceinline__ int spl_ff_monitor(const F64k &kk, int level, const F
   return near ? spl_ff_monitor_fp64<N>(kk, x, v, L.kc, eject2) : 0;
 }
 
+// The inertial state (barycentre moved by its velocity times `elapsed`) into the bin, or its
+// energy record into the log.
+template <int N>
+__device__ __forceinline__ void spl_write(const BinView &B, int s, const double (&m)[N], const double (&x)[N][3],
+                                          const double (&v)[N][3], double Minv, const double (&Xc)[3],
+                                          const double (&Vc)[3], double elapsed, const StepParams *log, double t) {
+  const int SP = B.S_pad;
+  double xo[N][3], vo[N][3], Xe[3];
+#pragma unroll
+  for (int c = 0; c < 3; c++) Xe[c] = fma(elapsed, Vc[c], Xc[c]);
+  spl_from_rel<N>(m, x, v, Minv, Xe, Vc, xo, vo);
+  if (log) {
+    double e[4];
+    spl_energy<N>(xo, vo, m, e);
+    write_log(*log, B.gidx[s], t, e);
+    return;
+  }
+#pragma unroll
+  for (int i = 0; i < N; i++)
+#pragma unroll
+    for (int c = 0; c < 3; c++) {
+      B.x[(size_t)(c * N + i) * SP + s] = xo[i][c];
+      B.v[(size_t)(c * N + i) * SP + s] = vo[i][c];
+    }
+}
+
 // 1/a, and 1/sqrt(a), as pairs
 __device__ __forceinline__ ff ff_div(const ff &a, const ff &b) {
   const float r = __frcp_rn(b.h);

@@ -27,30 +27,6 @@ namespace swarm {
 // with 50 FP64 and 3250 other instructions per step; 16384 x 4 over 400 steps 10.8 -> 4.1 ms;
 // steps of 0.003 and 0.02 orbits (levels 1 and 0), 100 of them: 9.5 -> 4.1 and 9.6 ms.
 template <int N>
-__device__ __forceinline__ void spl_write(const BinView &B, int s, const double (&m)[N], const double (&x)[N][3],
-                                          const double (&v)[N][3], double Minv, const double (&Xc)[3],
-                                          const double (&Vc)[3], double elapsed, const StepParams *log, double t) {
-  const int SP = B.S_pad;
-  double xo[N][3], vo[N][3], Xe[3];
-#pragma unroll
-  for (int c = 0; c < 3; c++) Xe[c] = fma(elapsed, Vc[c], Xc[c]);
-  spl_from_rel<N>(m, x, v, Minv, Xe, Vc, xo, vo);
-  if (log) {
-    double e[4];
-    spl_energy<N>(xo, vo, m, e);
-    write_log(*log, B.gidx[s], t, e);
-    return;
-  }
-#pragma unroll
-  for (int i = 0; i < N; i++)
-#pragma unroll
-    for (int c = 0; c < 3; c++) {
-      B.x[(size_t)(c * N + i) * SP + s] = xo[i][c];
-      B.v[(size_t)(c * N + i) * SP + s] = vo[i][c];
-    }
-}
-
-template <int N>
 __device__ __forceinline__ void spl_hermite_body(const BinView &B, const StepParams &P, int unit) {
   const bool printed = P.corr_form != 0;  // warp-uniform
   const int s = unit * 32 + (threadIdx.x & 31);

@@ -1,5 +1,5 @@
 // Single-bin persistent Runge-Kutta Cash-Karp kernels (fixed steps), n = 2..8.
-#include "rkck_impl.cuh"
+#include "rkck_ff.cuh"
 
 namespace swarm {
 
