@@ -23,7 +23,9 @@ ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 # register cap of device functions that are called out of line (kernels have their launch bounds):
 # the body-per-lane Hermite kernels run three CTAs of 128 threads per SM
 SOURCE_FLAGS = {f: ["-maxrregcount", "168"] for f in ("hermite_uniform_bpl_a.cu", "hermite_uniform_bpl_b.cu", "hermite_wide.cu",
-                                                       "rkck_fixed_b.cu", "rkck_adaptive_b.cu")}
+                                                       "rkck_fixed_b.cu", "rkck_adaptive_b.cu", "mvs_uniform_dh_a.cu",
+                                                       "mvs_uniform_dh_b.cu", "mvs_uniform_jac_a.cu",
+                                                       "mvs_uniform_jac_b.cu")}
 FLAGS = ARCH + ["-O3", "-std=c++17", "-lineinfo", "-rdc=true", "-Xcompiler", "-fPIC", "-I", INCLUDE]
 
 

@@ -658,16 +658,16 @@ static int run_persistent(swarm_ensemble *e, const StepParams &P0, int integrato
     if (m == SWARM_MAP_SYSTEM_PER_LANE && (!hermite_family(integrator) || e->bins[i].n > 4))
       m = SWARM_MAP_BODY_PER_LANE;
     maps[i] = m;
-    // MVS calls of 5000 steps or more: one CTA of 4 warps per SM (one warp per SM
-    // sub-partition) unless set.  Such calls end with a few long-lived systems whose step
-    // latency alone sets the time, and a second warp on their sub-partition doubles it
-    // (16384 x 8 compact ensemble, chunked calls: 1e4 steps 189 ms at one CTA per SM, 213
-    // at two; 1e5 steps 1.04 s against 1.43 s; 5000 steps even); shorter calls take the
-    // tuner's choice (over 2000 steps 2-3 CTAs per SM are ahead, 1.88e8 against 1.64e8
-    // system-steps/s, as the FP64 pipe goes from 73 to 91 %).
+    // MVS calls of 10000 steps or more: one CTA of 4 warps per SM (one warp per SM
+    // sub-partition) unless set; two from 5000 steps on.  Such calls end with a few long-lived
+    // systems whose step latency alone sets the time, and more warps on their sub-partition
+    // lengthen it (16384 x 8 compact ensemble, chunked calls at one, two, three CTAs per SM:
+    // 2000 steps 32.0, 22.1, 22.0 ms; 5000 54.5, 44.4, 50.3; 1e4 84.2, 82.2, 96.8; 1e5 605,
+    // 746, 877); shorter calls take the tuner's choice.
     if ((integrator == SWARM_MVS_DH || integrator == SWARM_MVS_JACOBI) && !e->ctas_per_sm) {
       const double span = std::max(std::fabs(P.t_end - e->t_lo), std::fabs(P.t_end - e->t_hi)) / std::fabs(P.dt);
-      if (span >= 5000) bin_ctas[i] = 1;
+      if (span >= 10000) bin_ctas[i] = 1;
+      else if (span >= 5000) bin_ctas[i] = 2;
     }
     // adaptive system per lane: the kernel's full residency (131072 x 3 systems over a
     // quarter of an inner period: 17.1 ms at two CTAs per SM, 28.9 ms at one, whose single
@@ -757,11 +757,8 @@ static int run_persistent(swarm_ensemble *e, const StepParams &P0, int integrato
     }
   }
   // Long MVS calls run as chunks of L steps (graph-replayed), and before each chunk every
-  // MVS bin's list is compacted to its runnable systems: the stream kernel then fills only
-  // as many groups per warp as the survivors need: the survivors start every chunk spread
-  // evenly over the warps, and once they are fewer than the warps each one runs spread
-  // over a whole warp (its step latency is what a long call waits on).  16384 x 8 compact
-  // ensemble: 2000 steps 1.74e8 -> 1.87e8 system-steps/s, 1e5 steps 1.32 -> 1.18 s.
+  // MVS bin's list is compacted to its runnable systems: the survivors start every chunk
+  // spread evenly over the warps, each warp holding only as many as that takes.
   const bool mvs = integrator == SWARM_MVS_DH || integrator == SWARM_MVS_JACOBI;
   const double call_span = std::max(std::fabs(P.t_end - e->t_lo), std::fabs(P.t_end - e->t_hi)) / std::fabs(P.dt);
   int chunk_steps = e->steps_per_launch;

@@ -22,6 +22,7 @@ __device__ __forceinline__ ff ff_make(float h, float l) {
   r.l = l;
   return r;
 }
+__device__ __forceinline__ constexpr ff ff_const(double d) { return ff{(float)d, (float)(d - (double)(float)d)}; }
 __device__ __forceinline__ ff ff_sel(bool p, const ff &a, const ff &b) { return ff_make(p ? a.h : b.h, p ? a.l : b.l); }
 __device__ __forceinline__ ff ff_neg(const ff &a) { return ff_make(-a.h, -a.l); }
 // a + b exactly (|a| >= |b| or a = 0)

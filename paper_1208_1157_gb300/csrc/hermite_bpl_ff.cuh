@@ -494,7 +494,7 @@ __device__ __forceinline__ void bpl_hermite_run(const BinView &B, const StepPara
         m = B.m[(size_t)b * SP + s];
       }
       const double m0 = shfl(m, g.base);
-      const bool sc = (__ballot_sync(FULL, !fscale(m, -60, 40)) & gm) == 0 && fscale(P.dt, -60, 40);
+      const bool sc = (__ballot_sync(FULL, !fmass_ok(m, b == 0)) & gm) == 0 && fscale(P.dt, -60, 40);
       for (int r = 1; r <= rt; r++) {
         int p = b + r;
         if (p >= n) p -= n;

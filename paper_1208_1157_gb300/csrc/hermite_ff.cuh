@@ -86,6 +86,10 @@ __device__ __forceinline__ bool fscale(double v, int lo, int hi) {
   return e > 1023 + lo && e < 1023 + hi;
 }
 
+// a body's mass (test particles have tiny ones: what underflows of a planet's pull is below any
+// rounding of body 0's)
+__device__ __forceinline__ bool fmass_ok(double m, bool star) { return fscale(m, star ? -60 : -100, 40); }
+
 // ---------------------------------------------------------------- adaptive step (Eq. 5)
 // The Hermite propagator with the step of Sec. 4.3.2: dt = tau (sum_i |j_i|^2/|a_i|^2)^(-1/2)
 // from the values at the start of the step, clamped so that the last step lands on the
@@ -188,7 +192,7 @@ __device__ __forceinline__ FMass<N> fmass(const double (&m)[N]) {
     f.mu[i] = m[0] + m[i];
     f.m[i] = ff_from(m[i]);
     f.muf[i] = ff_from(f.mu[i]);
-    f.ok = f.ok && fscale(m[i], -60, 40);
+    f.ok = f.ok && fmass_ok(m[i], i == 0);
   }
   return f;
 }

@@ -47,7 +47,9 @@ __global__ void __launch_bounds__(128, 2)
 
 cudaError_t launch_mvs_persistent(const BinView *d_bins, const int4 *d_work, int nwork, const StepParams &P, int grid,
                                   cudaStream_t st) {
-  mvs_persistent_kernel<<<grid, 128, 0, st>>>(d_bins, d_work, nwork, P);
+  StepParams Q = P;
+  Q.fc = fcoef_host(P.dt);
+  mvs_persistent_kernel<<<grid, 128, 0, st>>>(d_bins, d_work, nwork, Q);
   return cudaGetLastError();
 }
 

@@ -1,5 +1,5 @@
 // Single-bin persistent MVS kernels (democratic heliocentric), n = 2..8.
-#include "mvs_impl.cuh"
+#include "mvs_ff.cuh"
 
 namespace swarm {
 

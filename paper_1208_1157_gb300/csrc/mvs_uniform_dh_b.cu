@@ -1,5 +1,5 @@
 // Single-bin persistent MVS kernels (democratic heliocentric), n = 9..15.
-#include "mvs_impl.cuh"
+#include "mvs_ff.cuh"
 
 namespace swarm {
 

@@ -1,5 +1,5 @@
 // Instantiations of the MVS work-unit function (democratic heliocentric coordinates, n = 2..8).
-#include "mvs_impl.cuh"
+#include "mvs_ff.cuh"
 
 namespace swarm {
 template __device__ void bpl_mvs_unit<2, false>(const BinView &, const StepParams &, int);

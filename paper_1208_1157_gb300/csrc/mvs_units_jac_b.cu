@@ -1,5 +1,5 @@
 // Instantiations of the MVS work-unit function (Jacobi coordinates, n = 9..15).
-#include "mvs_impl.cuh"
+#include "mvs_ff.cuh"
 
 namespace swarm {
 template __device__ void bpl_mvs_unit<9, true>(const BinView &, const StepParams &, int);

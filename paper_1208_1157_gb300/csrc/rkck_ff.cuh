@@ -19,7 +19,6 @@
 
 namespace swarm {
 
-__device__ __forceinline__ constexpr ff ff_const(double d) { return ff{(float)d, (float)(d - (double)(float)d)}; }
 // sum of constants times pairs
 __device__ __forceinline__ ff ff_lin(double c, const ff &a) { return ff_mul_raw(ff_const(c), a); }
 __device__ __forceinline__ ff ff_lin(double c, const ff &a, const ff &s) { return ff_fma_raw(ff_const(c), a, s); }
@@ -830,7 +829,7 @@ __device__ __forceinline__ void bpl_rkck_stream(const BinView &B, const StepPara
         m = B.m[(size_t)b * SP + s];
       }
       const double m0 = shfl(m, g.base);
-      const bool sc = (__ballot_sync(FULL, !fscale(m, -60, 40)) & gm) == 0;
+      const bool sc = (__ballot_sync(FULL, !fmass_ok(m, b == 0)) & gm) == 0;
       for (int r = 1; r <= ARing<N>::RT; r++) {
         int p = b + r;
         if (p >= N) p -= N;
