@@ -74,7 +74,9 @@ void free_pool(Pool *q) {
 
 constexpr int kStageSlots = 1 << 16;  // slot indices one staging batch can carry
 
-constexpr int kSide = 8;  // forked streams for the pools' concurrent launches
+// forked streams for the pools' concurrent launches: one per pool (body count and integrator),
+// up to 32 (24 requests on 8 streams 7.3 ms, on 32 6.0 ms)
+constexpr int kSide = 32;
 
 struct Request {
   int64_t id = 0;
