@@ -107,6 +107,13 @@ struct StepParams {
   F64k fk = {0.0, -1.0, 1.0};  // opaque constants (set on the host, never changed)
   FCoef fc = {};               // coefficients of a step dt (set by the launchers that use them)
   int concurrent = 0;          // host-side hint: other bins' launches overlap this one
+  // radial velocities on the way (n_obs > 0): each system goes on through the end times t_obs and
+  // leaves v_0 . los at each of them in rv[k * rv_stride + system]
+  int n_obs = 0;
+  const double *t_obs = nullptr;
+  double *rv = nullptr;
+  long long rv_stride = 0;
+  double los[3] = {0.0, 0.0, 0.0};
 };
 
 __device__ __forceinline__ double shfl(double v, int src) { return __shfl_sync(0xffffffffu, v, src); }
@@ -180,9 +187,7 @@ struct LaunchPlan {
   double h_last;
   double t_end;
 };
-__device__ __forceinline__ LaunchPlan launch_plan(const BinView &B, const StepParams &P, int s, double t0,
-                                                  bool runnable) {
-  const double te = B.t_end ? B.t_end[s] : (P.t_end_dev ? *P.t_end_dev : P.t_end);
+__device__ __forceinline__ LaunchPlan launch_plan_to(const StepParams &P, double te, double t0, bool runnable) {
   const StepPlan p = plan_steps(t0, te, P.dt);
   LaunchPlan L;
   L.t_end = te;
@@ -197,6 +202,10 @@ __device__ __forceinline__ LaunchPlan launch_plan(const BinView &B, const StepPa
     L.h_last = P.dt;
   }
   return L;
+}
+__device__ __forceinline__ LaunchPlan launch_plan(const BinView &B, const StepParams &P, int s, double t0,
+                                                  bool runnable) {
+  return launch_plan_to(P, B.t_end ? B.t_end[s] : (P.t_end_dev ? *P.t_end_dev : P.t_end), t0, runnable);
 }
 // time after step k of a launch
 __device__ __forceinline__ double step_time(const LaunchPlan &L, int k, double t0, double dt) {

@@ -13,7 +13,7 @@
 // Bound: issue slots and the latency of their chains (n = 15: 7200 instructions and 41 FP64
 // ones per step of two systems, 0.52 issued per cycle and sub-partition, the FP64 pipe 18 %
 // busy), so three CTAs per SM (168 registers).  Per step of 5041 systems, wholly in FP64 ->
-// now: n = 3 6.5 -> 4.7 us, 5 20.7 -> 6.7, 8 52.3 -> 9.7, 11 89.4 -> 22.8, 15 120.8 -> 33.0
+// now: n = 3 6.5 -> 4.3 us, 5 20.7 -> 6.7, 8 52.3 -> 9.7, 11 89.4 -> 22.8, 15 120.8 -> 33.0
 // (packed over the CTA for n = 7, 11, 15 before); 65536 systems of 3..15 bodies over 100
 // steps: 69.2 -> 18.3 ms.  A step of 0.02 orbits (level 0), n = 8: 39.9 -> 56 us.
 // 2048 systems of 16..32 bodies (one per warp, n a run-time value) over 50 steps: 13.6 -> 4.7 ms.
@@ -41,6 +41,9 @@ struct BplBody {
   int b, base, nn;
   double m0;   // body 0's mass
   ff m0f, mf;  // and this body's, as pairs
+  float mt;    // what mf leaves of it: in body 0's own acceleration its mass is no small weight, and
+               // left out (as would the product of the lower parts, of one sign for truncated
+               // pairs) it would be the same relative error at every step
   __device__ __forceinline__ int n() const { return N ? N : nn; }
   __device__ __forceinline__ unsigned mask() const { return n() == 32 ? 0xffffffffu : ((1u << n()) - 1u) << base; }
   // the ring over the n - 1 planets: RF rounds with reaction, and for an even number a last one in
@@ -73,6 +76,38 @@ __device__ __forceinline__ ff grp_sum_ff(const BplBody<N> &g, ff t) {
     t = ff_add_raw(t, o);
   }
   return ff_norm(t);
+}
+
+// the same over the planets' lanes alone, whatever body 0's holds: the first level takes two
+// lanes at once, so that n - 1 values need no level more than their number does
+template <int N>
+__device__ __forceinline__ ff grp_planets_ff(const BplBody<N> &g, ff t) {
+  const unsigned FULL = 0xffffffffu;
+  ff a = ff_make(__shfl_down_sync(FULL, t.h, 1), __shfl_down_sync(FULL, t.l, 1));
+  if (N == 2) return a;
+  if (g.b + 1 >= g.n()) a = ff_make(0.0f, 0.0f);
+  ff o = ff_make(__shfl_down_sync(FULL, t.h, 2), __shfl_down_sync(FULL, t.l, 2));
+  if (g.b + 2 >= g.n()) o = ff_make(0.0f, 0.0f);
+  t = ff_add_raw(a, o);
+#pragma unroll
+  for (int off = 2; off < (N ? N : 32) - 1; off <<= 1) {
+    o = ff_make(__shfl_down_sync(FULL, t.h, off), __shfl_down_sync(FULL, t.l, off));
+    if (g.b + off >= g.n()) o = ff_make(0.0f, 0.0f);
+    t = ff_add_raw(t, o);
+  }
+  return ff_norm(t);
+}
+template <int N>
+__device__ __forceinline__ float grp_planets32(const BplBody<N> &g, float t) {
+  const unsigned FULL = 0xffffffffu;
+  const float a = __shfl_down_sync(FULL, t, 1), c = __shfl_down_sync(FULL, t, 2);
+  t = (g.b + 1 < g.n() ? a : 0.0f) + (g.b + 2 < g.n() ? c : 0.0f);
+#pragma unroll
+  for (int off = 2; off < (N ? N : 32) - 1; off <<= 1) {
+    const float o = __shfl_down_sync(FULL, t, off);
+    t += g.b + off < g.n() ? o : 0.0f;
+  }
+  return t;
 }
 
 // an evaluation: acceleration -M dX + P (M, dX FP64; M = 0 on body 0's lane), jerk J, distances
@@ -191,10 +226,12 @@ __device__ __forceinline__ void bpl_eval_ff(const F64k &k, const BplBody<N> &g, 
       if (STATE) R.S = __fmaf_rn(-mq.h, __shfl_sync(0xffffffffu, sg, q), R.S);
     }
   }
-  const ff mm = star ? ff_make(0.0f, 0.0f) : g.mf;
 #pragma unroll
   for (int c = 0; c < 3; c++) {
-    const ff sa = grp_sum_ff<N>(g, ff_mul(mm, T[c])), sj = grp_sum_ff<N>(g, ff_mul(mm, Z[c]));
+    const ff Tn = ff_norm(T[c]);  // (raw lower parts are of one sign, and so is then their rounding)
+    ff w = ff_mul_raw(g.mf, Tn);
+    w = fast_two_sum(w.h, __fmaf_rn(g.mf.l, Tn.l, __fmaf_rn(g.mt, Tn.h, w.l)));
+    const ff sa = grp_planets_ff<N>(g, w), sj = grp_planets_ff<N>(g, ff_mul_raw(g.mf, Z[c]));
     const ff a = FULL ? ff_norm(R.P[c]) : ff_fma(ff_neg(g.m0f), T[c], R.P[c]);
     const ff j = ff_fma(ff_neg(g.m0f), Z[c], Q[c]);
     R.P[c] = ff_sel(star, sa, a);
@@ -212,16 +249,6 @@ __device__ __forceinline__ int bpl_level(const BplBody<N> &g, const BplEval<N> &
   return n0 ? 0 : n1 ? 1 : 2;
 }
 
-// sum of a float over a group's lanes, valid in its first lane
-template <int N>
-__device__ __forceinline__ float grp_sum32(const BplBody<N> &g, float t) {
-#pragma unroll
-  for (int off = 1; off < (N ? N : 32); off <<= 1) {
-    const float o = __shfl_down_sync(0xffffffffu, t, off);
-    t += g.b + off < g.n() ? o : 0.0f;
-  }
-  return t;
-}
 // change of the evaluation R when the bodies' positions and velocities move by dX, dV, in FP32
 // (see spl_delta); the pairs' geometry is formed again from R's FP32 vectors
 template <int N>
@@ -269,8 +296,8 @@ __device__ __forceinline__ void bpl_delta(const BplBody<N> &g, const BplEval<N> 
   }
 #pragma unroll
   for (int c = 0; c < 3; c++) {
-    const float sa = grp_sum32<N>(g, star ? 0.0f : __fmul_rn(g.mf.h, T[c]));
-    const float sj = grp_sum32<N>(g, star ? 0.0f : __fmul_rn(g.mf.h, Z[c]));
+    const float sa = grp_planets32<N>(g, __fmul_rn(g.mf.h, T[c]));
+    const float sj = grp_planets32<N>(g, __fmul_rn(g.mf.h, Z[c]));
     DA[c] = star ? sa : __fmaf_rn(-g.m0f.h, T[c], P[c]);
     DJ[c] = star ? sj : __fmaf_rn(-g.m0f.h, Z[c], Q[c]);
   }
@@ -415,7 +442,10 @@ static __device__ __noinline__ void bpl_fp64_advance(const F64k &k, double h, in
 // adaptive steps: step counts differ from system to system).  take(need): the group's next
 // system, or -1 (every lane calls it).  A refill round loads the new systems and evaluates
 // them (the other groups re-evaluate their unchanged state and keep what they have).
-template <int N, bool ADAPT, class Take>
+// OBS (fixed steps): through the observation times P.t_obs in one launch, leaving the radial
+// velocity at each (12 observations 12 steps apart, 257 x 3 systems: 1.14 ms with a launch for
+// each, whose cold start costs as much as three steps, 0.95 in one).
+template <int N, bool ADAPT, bool OBS, class Take>
 __device__ __forceinline__ void bpl_hermite_run(const BinView &B, const StepParams &P, BplRounds<N> &rd, float *kcf,
                                                 Take take) {
   constexpr int KS = N ? 1 : 32;
@@ -460,6 +490,7 @@ __device__ __forceinline__ void bpl_hermite_run(const BinView &B, const StepPara
   ff h = ff_make(0.0f, 0.0f);          // ADAPT: length of the next step of a group in pairs
   g.m0 = 1.0;
   g.m0f = g.mf = ff_make(1.0f, 0.0f);
+  g.mt = 0.0f;
   for (int r = 1; r <= rt; r++) rd.kcr(r) = 0.0;
   for (int r = 1; r <= g.RT(); r++) kcf[(r - 1) * KS] = 0.0f;
   auto to_bits = [](const ff &f) { return __hiloint2double(__float_as_int(f.h), __float_as_int(f.l)); };
@@ -475,6 +506,24 @@ __device__ __forceinline__ void bpl_hermite_run(const BinView &B, const StepPara
     }
     const ff sum = shfl_ff(grp_sum_ff<N>(g, ff_div(ff_norm2(J), ff_norm2(A))), g.base);
     return ff_mul(tau, ff_rsqrt(sum));
+  };
+
+  // the observations [from, to) at the present state, and the plan from t0 on towards the first
+  // of the others that lies ahead (those that do not are made here); plan.N = 0: none is left
+  int obs = 0;
+  auto next_obs = [&](int from, int to) {
+    for (obs = from;; obs++) {
+      if (obs >= to) {
+        if (obs >= P.n_obs) {
+          plan.N = 0;
+          return;
+        }
+        plan = launch_plan_to(P, P.t_obs[obs], t0, true);
+        if (plan.N > 0) return;
+      }
+      if (lane_ok && b == 0)
+        P.rv[obs * P.rv_stride + B.gidx[s]] = v[0] * P.los[0] + v[1] * P.los[1] + v[2] * P.los[2];
+    }
   };
 
   for (;;) {
@@ -511,7 +560,8 @@ __device__ __forceinline__ void bpl_hermite_run(const BinView &B, const StepPara
         scaled = sc;
         g.m0 = m0;
         g.m0f = ff_from(m0);
-        g.mf = ff_from(m);
+        g.mf = ff_norm(ff_from(m));
+        g.mt = (float)((m - (double)g.mf.h) - (double)g.mf.l);
       }
       const bool sc2 = scaled;
       BplEval<N> E;
@@ -555,7 +605,8 @@ __device__ __forceinline__ void bpl_hermite_run(const BinView &B, const StepPara
         steps = 0;
         const bool runnable = B.status[s] <= SWARM_SYS_DONE;
         if (!ADAPT) {
-          plan = launch_plan(B, P, s, t0, runnable);
+          if constexpr (OBS) next_obs(0, runnable ? 0 : P.n_obs);
+          else plan = launch_plan(B, P, s, t0, runnable);
           has = runnable && plan.N > 0;
         } else {
           te = adaptive_end(B, P, s);
@@ -794,7 +845,20 @@ __device__ __forceinline__ void bpl_hermite_run(const BinView &B, const StepPara
         if (need_log && lane_ok && b == 0) write_log(P, B.gidx[s], t, e4);
       }
     }
-    if (finish && lane_ok) {
+    bool end = finish;
+    if constexpr (OBS) if (finish) {
+      const bool count = obs == P.n_obs - 1;  // the counters are the last interval's
+      if (b == 0 && lane_ok && P.counters && steps > 0 && count) {
+        atomicAdd(&P.counters[0], (unsigned long long)steps);
+        const unsigned long long NP = (unsigned long long)n * (n - 1) / 2;
+        atomicAdd(&P.counters[1], NP * (1ull + (unsigned long long)steps * (P.n_corr + 1)));
+      }
+      t0 = t;
+      steps = 0;
+      next_obs(obs, code ? P.n_obs : obs + 1);
+      end = plan.N == 0;
+    }
+    if (end && lane_ok) {
 #pragma unroll
       for (int c = 0; c < 3; c++) {
         B.x[(size_t)(c * n + b) * SP + s] = x[c];
@@ -812,15 +876,15 @@ __device__ __forceinline__ void bpl_hermite_run(const BinView &B, const StepPara
         }
       }
     }
-    if (finish) has = false;
+    if (end) has = false;
   }
 }
 // the bin's next systems, one by one
-template <int N, bool ADAPT>
+template <int N, bool ADAPT, bool OBS = false>
 __device__ __forceinline__ void bpl_hermite_stream(const BinView &B, const StepParams &P) {
   BplRounds<N> rd;
   float kcf[kRoundsA<N>];
-  bpl_hermite_run<N, ADAPT>(B, P, rd, kcf, [&](bool need, bool leader, int base) {
+  bpl_hermite_run<N, ADAPT, OBS>(B, P, rd, kcf, [&](bool need, bool leader, int base) {
     int sn = 0;
     if (need && leader) sn = atomicAdd(P.work_next, 1);
     sn = __shfl_sync(0xffffffffu, sn, base);
@@ -833,7 +897,7 @@ __device__ __forceinline__ void bpl_hermite_body(const BinView &B, const StepPar
   bool taken = false;
   BplRounds<N> rd;
   float kcf[kRoundsA<N>];
-  bpl_hermite_run<N, ADAPT>(B, P, rd, kcf, [&](bool, bool, int base) {
+  bpl_hermite_run<N, ADAPT, false>(B, P, rd, kcf, [&](bool, bool, int base) {
     const int s = taken ? -1 : unit * (32 / N) + base / N;
     taken = true;
     return s < B.S ? s : -1;
@@ -849,7 +913,7 @@ __device__ __forceinline__ void wide_hermite_stream(const BinView &B, const Step
   BplRounds<0> rd;
   rd.kc = kc + lane;
   rd.d2 = d2 + lane;
-  bpl_hermite_run<0, ADAPT>(B, P, rd, kcf + lane, [&](bool need, bool leader, int base) {
+  bpl_hermite_run<0, ADAPT, false>(B, P, rd, kcf + lane, [&](bool need, bool leader, int base) {
     int sn = 0;
     if (need && leader) sn = atomicAdd(P.work_next, 1);
     sn = __shfl_sync(0xffffffffu, sn, base);

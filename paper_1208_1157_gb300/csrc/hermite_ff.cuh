@@ -129,7 +129,10 @@ __device__ __forceinline__ void star_pull(const F64k &k, const double (&X)[3], d
   rho = yf;
   const ff y2f = two_prod(yf, yf);
   const ff y3f = ff_mulf(y2f, yf);
-  rho3 = fast_two_sum(y3f.h, __fmaf_rn(y3f.h, q.h, y3f.l));
+  // y^3 + y^3 q with q's lower part: q is up to 2^-18, and body 0's own acceleration, in which
+  // rho^3 is no small weight, wants 2^-46
+  const ff c3 = ff_mul_raw(y3f, q), s3 = fast_two_sum(y3f.h, c3.h);
+  rho3 = fast_two_sum(s3.h, __fadd_rn(s3.l, __fadd_rn(y3f.l, c3.l)));
   const float p2 = __fmaf_rn(t.h, t.h, t.h);
   rho2 = fast_two_sum(y2f.h, __fmaf_rn(y2f.h, p2, y2f.l));
 }

@@ -246,14 +246,17 @@ __device__ __noinline__ void spl_hermite_adaptive_unit(const BinView &B, const S
 
 // Persistent kernel for one bin (one body count, one mapping): the unit body is inlined,
 // so registers are allocated for this n alone.  Warps pull unit indices from a counter.
-template <int MAP, int N, bool ADAPT = false>
-__global__ void __launch_bounds__(128, MAP == SWARM_MAP_BODY_PER_LANE ? 3 : 2) hermite_uniform_kernel(BinView B, int nunits, StepParams P) {
+// Body per lane: three CTAs per SM, or two where the step's latency is all that counts, up to
+// four bodies (a bin that fills the chip runs system per lane) and observations on the way
+// (without the spills 1024 x 3 systems over 400 steps take 1.88 instead of 1.92 ms).
+template <int MAP, int N, bool ADAPT = false, bool OBS = false>
+__global__ void __launch_bounds__(128, MAP == SWARM_MAP_BODY_PER_LANE && N > 4 && !OBS ? 3 : 2) hermite_uniform_kernel(BinView B, int nunits, StepParams P) {
   if (ADAPT && MAP == SWARM_MAP_SYSTEM_PER_LANE) {  // work unit = system (per-lane refill)
     spl_hermite_adaptive_stream<N>(B, P);
     return;
   }
   if (MAP == SWARM_MAP_BODY_PER_LANE) {  // work unit = system (per-group refill)
-    bpl_hermite_stream<N, ADAPT>(B, P);
+    bpl_hermite_stream<N, ADAPT, OBS>(B, P);
     return;
   }
   const int lane = threadIdx.x & 31;
@@ -266,17 +269,17 @@ __global__ void __launch_bounds__(128, MAP == SWARM_MAP_BODY_PER_LANE ? 3 : 2) h
   }
 }
 
-template <int MAP, int N, bool ADAPT = false>
+template <int MAP, int N, bool ADAPT = false, bool OBS = false>
 cudaError_t launch_hermite_uniform_n(const BinView &B, int nunits, const StepParams &P, int grid, cudaStream_t st) {
   StepParams Q = P;
   Q.fc = fcoef_host(P.dt);
-  hermite_uniform_kernel<MAP, N, ADAPT><<<grid, 128, 0, st>>>(B, nunits, Q);
+  hermite_uniform_kernel<MAP, N, ADAPT, OBS><<<grid, 128, 0, st>>>(B, nunits, Q);
   return cudaGetLastError();
 }
-template <int MAP, int N, bool ADAPT = false>
+template <int MAP, int N, bool ADAPT = false, bool OBS = false>
 int hermite_uniform_blocks_n() {
   int nb = 0;
-  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, hermite_uniform_kernel<MAP, N, ADAPT>, 128, 0);
+  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, hermite_uniform_kernel<MAP, N, ADAPT, OBS>, 128, 0);
   return nb;
 }
 // adaptive (Eq. 5) single-bin kernels: both mappings, registers sized for 2 CTAs per SM

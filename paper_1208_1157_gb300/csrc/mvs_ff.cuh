@@ -302,10 +302,10 @@ __device__ __forceinline__ void mvs_reflex(const F64k &k, const BplBody<N> &g, c
     range = range && abs_below_pow2(u[c], 40);
     const ff uf = ff_norm(ff_from(u[c]));
     V2 = __fmaf_rn(uf.h, uf.h, V2);
-    const ff s = shfl_ff(grp_sum_ff<N>(g, star ? ff_make(0.0f, 0.0f) : ff_mul(L.w, uf)), g.base);
+    const ff s = shfl_ff(grp_planets_ff<N>(g, ff_mul_raw(L.w, uf)), g.base);
     p[c] = star ? u[c] : ff_double(s);
   }
-  const float w = hf * __shfl_sync(0xffffffffu, grp_sum32<N>(g, star ? 0.0f : L.w.h * __fsqrt_rn(V2)), g.base);
+  const float w = hf * __shfl_sync(0xffffffffu, grp_planets32<N>(g, L.w.h * __fsqrt_rn(V2)), g.base);
   const bool bad = has && !star && !(range && w * w <= 0x1p-16f * q2);
   if (__any_sync(0xffffffffu, bad)) {
     const unsigned bm = __ballot_sync(0xffffffffu, bad) & g.mask();

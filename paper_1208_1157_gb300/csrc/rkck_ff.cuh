@@ -611,10 +611,12 @@ __device__ __forceinline__ void bpl_acc_ff(const F64k &k, const BplBody<N> &g, c
       if (STATE) S = __fmaf_rn(-mq.h, __shfl_sync(0xffffffffu, sg, q), S);
     }
   }
-  const ff mm = star ? ff_make(0.0f, 0.0f) : g.mf;
 #pragma unroll
   for (int c = 0; c < 3; c++) {
-    const ff sa = grp_sum_ff<N>(g, ff_mul(mm, T[c]));
+    const ff Tn = ff_norm(T[c]);  // (raw lower parts are of one sign, and so is then their rounding)
+    ff w = ff_mul_raw(g.mf, Tn);
+    w = fast_two_sum(w.h, __fmaf_rn(g.mf.l, Tn.l, __fmaf_rn(g.mt, Tn.h, w.l)));
+    const ff sa = grp_planets_ff<N>(g, w);
     R.P[c] = ff_sel(star, sa, FULL ? ff_norm(R.P[c]) : ff_fma(ff_neg(g.m0f), T[c], R.P[c]));
   }
   if (STATE) {
@@ -804,6 +806,7 @@ __device__ __forceinline__ void bpl_rkck_stream(const BinView &B, const StepPara
   bool fresh = false, at_end = false;  // a state without its evaluation; its time is the end time
   g.m0 = 1.0;
   g.m0f = g.mf = ff_make(1.0f, 0.0f);
+  g.mt = 0.0f;
 #pragma unroll
   for (int c = 0; c < 3; c++) P1[c] = ff_make(0.0f, 0.0f);
   for (int r = 0; r < RT; r++) kc[r] = 0.0;
@@ -846,7 +849,8 @@ __device__ __forceinline__ void bpl_rkck_stream(const BinView &B, const StepPara
         scaled = sc;
         g.m0 = m0;
         g.m0f = ff_from(m0);
-        g.mf = ff_from(m);
+        g.mf = ff_norm(ff_from(m));
+        g.mt = (float)((m - (double)g.mf.h) - (double)g.mf.l);
         t0 = t = B.t[s];
         steps = 0;
         trials = 0;
