@@ -192,7 +192,9 @@ int swarm_query_stats(const swarm_ensemble *ens, swarm_stats *out);
  * this integrator and dt; the times must run in the direction of dt) and record the
  * radial velocities on the device; rv[n_obs][n_sys] (host) is copied once at the end.
  * A system that stops keeps its state, so its later records repeat its value at the stop
- * (the status array tells).  swarm_query_stats then describes the last interval. */
+ * (the status array tells).  swarm_query_stats then counts the last interval's steps; its
+ * kernel time and launches are that interval's or, where one launch per body count goes
+ * through all of them (fixed-step Hermite), the call's. */
 int swarm_query_rv(const swarm_ensemble *ens, const double *los, double *rv);
 int swarm_observe_rv(swarm_ensemble *ens, const double *t_obs, int32_t n_obs, int integrator, double dt,
                      const double *los, double *rv);

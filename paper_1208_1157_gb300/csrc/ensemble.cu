@@ -113,6 +113,9 @@ struct swarm_ensemble {
   // longest-first system lists of the bins for the adaptive integrators
   int32_t *d_order = nullptr;
   int *d_order_scratch = nullptr;
+  // radial velocities and observation times of swarm_observe_rv (grows to the largest call)
+  double *d_obs = nullptr;
+  size_t obs_bytes = 0;
   cudaGraphExec_t graph = nullptr;
   std::vector<double> graph_key;
   swarm_stats stats{};
@@ -263,6 +266,7 @@ static void free_all(swarm_ensemble *e) {
   for (auto ev : e->side_done) cudaEventDestroy(ev);
   if (e->fork_ev) cudaEventDestroy(e->fork_ev);
   if (e->d_order) cudaFree(e->d_order);
+  if (e->d_obs) cudaFree(e->d_obs);
   if (e->d_order_scratch) cudaFree(e->d_order_scratch);
 }
 
@@ -636,6 +640,10 @@ static bool adaptive(int integrator) {
   return integrator == SWARM_HERMITE4_ADAPTIVE || integrator == SWARM_RKCK_ADAPTIVE;
 }
 
+// A call through observation times (P0.n_obs > 0) is one launch per bin where every bin's kernel
+// goes through them by itself: fixed-step Hermite, body per lane.  Otherwise kObsNotTaken, with
+// nothing enqueued.
+constexpr int kObsNotTaken = 1;
 static int run_persistent(swarm_ensemble *e, const StepParams &P0, int integrator) {
   StepParams P = P0;
   std::vector<int> maps(e->bins.size()), bin_ctas(e->bins.size(), e->ctas_per_sm);
@@ -681,6 +689,9 @@ static int run_persistent(swarm_ensemble *e, const StepParams &P0, int integrato
     if (integrator == SWARM_HERMITE4_ADAPTIVE && m == SWARM_MAP_SYSTEM_PER_LANE && !e->ctas_per_sm)
       bin_ctas[i] = P.corr_form ? 1 : 0;
   }
+  if (P.n_obs > 0)
+    for (int m : maps)
+      if (m != SWARM_MAP_BODY_PER_LANE) return kObsNotTaken;
   int rc = build_work(e, maps);
   if (rc) return rc;
   std::vector<int> wide;  // bins of 16..32 bodies
@@ -859,7 +870,12 @@ static int run_persistent(swarm_ensemble *e, const StepParams &P0, int integrato
   return SWARM_OK;
 }
 
-static int integrate_impl(swarm_ensemble *e, double t_end, int integrator, double dt, bool sync) {
+struct ObsCall {
+  int n;
+  const double *t, *los;  // device times
+  double *rv;             // [n][n_sys]
+};
+static int integrate_impl(swarm_ensemble *e, double t_end, int integrator, double dt, bool sync, const ObsCall *obs = nullptr) {
   if (!e) return fail(SWARM_EINVAL, "ensemble is NULL");
   if (integrator < SWARM_HERMITE4 || integrator > SWARM_RKCK_ADAPTIVE)
     return fail(SWARM_EINVAL, "unknown integrator %d", integrator);
@@ -869,6 +885,13 @@ static int integrate_impl(swarm_ensemble *e, double t_end, int integrator, doubl
   if (e->mapping == SWARM_MAP_PLAIN_PER_STEP && (integrator != SWARM_HERMITE4 || e->corr_form))
     return fail(SWARM_EINVAL, "the plain per-step baseline exists for the fixed-step time-symmetric Hermite only");
   StepParams P = make_params(e, t_end, integrator, dt);
+  if (obs) {
+    P.n_obs = obs->n;
+    P.t_obs = obs->t;
+    P.rv = obs->rv;
+    P.rv_stride = e->n_sys;
+    for (int c = 0; c < 3; c++) P.los[c] = obs->los[c];
+  }
   CK(cudaMemsetAsync(e->d_counters, 0, sizeof(unsigned long long) * 4, e->stream));
   e->launches = 0;
   CK(cudaEventRecord(e->ev0, e->stream));
@@ -1032,17 +1055,41 @@ extern "C" int swarm_observe_rv(swarm_ensemble *e, const double *t_obs, int32_t 
     if (k > 0 && (t_obs[k] - t_obs[k - 1]) * dt < 0.0)
       return fail(SWARM_EINVAL, "observation times must run in the direction of dt");
   }
-  double *d_rec = nullptr;
-  CK(cudaMalloc(&d_rec, sizeof(double) * (size_t)n_obs * e->n_sys));
-  for (int k = 0; k < n_obs && rc == SWARM_OK; k++) {
-    rc = integrate_impl(e, t_obs[k], integrator, dt, false);
-    if (rc == SWARM_OK) rc = enqueue_rv(e, los, d_rec + (size_t)k * e->n_sys);
+  // the records and the times
+  const size_t nrec = (size_t)n_obs * e->n_sys, bytes = sizeof(double) * (nrec + n_obs);
+  if (bytes > e->obs_bytes) {
+    CK(cudaStreamSynchronize(e->stream));
+    if (e->d_obs) cudaFree(e->d_obs);
+    e->d_obs = nullptr;
+    e->obs_bytes = 0;
+    CK(cudaMalloc(&e->d_obs, bytes));
+    e->obs_bytes = bytes;
+  }
+  double *d_rec = e->d_obs;
+  // One call through all the times where the kernels can take them: not with the options that
+  // cut a call up or choose another kernel, nor where an interval would be refused.
+  bool one = integrator == SWARM_HERMITE4 && n_obs > 1 && e->steps_per_launch <= 0 && !e->single_launch && !e->corr_form &&
+             (e->mapping == SWARM_MAP_AUTO || e->mapping == SWARM_MAP_BODY_PER_LANE) && dt != 0.0 && std::isfinite(dt);
+  for (int k = 0; k < n_obs && one; k++) {
+    const double lo = k ? t_obs[k - 1] : e->t_lo, hi = k ? t_obs[k - 1] : e->t_hi;
+    one = std::max(std::fabs(t_obs[k] - lo), std::fabs(t_obs[k] - hi)) / std::fabs(dt) <= kMaxCallSteps;
+  }
+  rc = kObsNotTaken;
+  if (one) {
+    CK(cudaMemcpyAsync(d_rec + nrec, t_obs, sizeof(double) * n_obs, cudaMemcpyHostToDevice, e->stream));
+    const ObsCall obs{n_obs, d_rec + nrec, los, d_rec};
+    rc = integrate_impl(e, t_obs[n_obs - 1], integrator, dt, false, &obs);
+  }
+  if (rc == kObsNotTaken) {
+    rc = SWARM_OK;
+    for (int k = 0; k < n_obs && rc == SWARM_OK; k++) {
+      rc = integrate_impl(e, t_obs[k], integrator, dt, false);
+      if (rc == SWARM_OK) rc = enqueue_rv(e, los, d_rec + (size_t)k * e->n_sys);
+    }
   }
   cudaError_t ce = cudaSuccess;
-  if (rc == SWARM_OK)
-    ce = cudaMemcpyAsync(rv, d_rec, sizeof(double) * (size_t)n_obs * e->n_sys, cudaMemcpyDeviceToHost, e->stream);
+  if (rc == SWARM_OK) ce = cudaMemcpyAsync(rv, d_rec, sizeof(double) * nrec, cudaMemcpyDeviceToHost, e->stream);
   cudaError_t se = cudaStreamSynchronize(e->stream);
-  cudaFree(d_rec);
   if (rc) return rc;
   CK(ce);
   CK(se);

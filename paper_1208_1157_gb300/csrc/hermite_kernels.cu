@@ -212,10 +212,17 @@ cudaError_t launch_hermite_uniform_bpl_a(int n, const BinView &B, int nunits, co
 cudaError_t launch_hermite_uniform_bpl_b(int n, const BinView &B, int nunits, const StepParams &P, int grid,
                                          cudaStream_t st, int *blocks);
 
+cudaError_t launch_hermite_obs_bpl_a(int n, const BinView &B, int nunits, const StepParams &P, int grid,
+                                     cudaStream_t st, int *blocks);
+cudaError_t launch_hermite_obs_bpl_b(int n, const BinView &B, int nunits, const StepParams &P, int grid,
+                                     cudaStream_t st, int *blocks);
 cudaError_t launch_hermite_uniform(int mapping, const BinView &B, int nunits, const StepParams &P, int grid,
                                    cudaStream_t st, int *blocks) {
   if (mapping == SWARM_MAP_SYSTEM_PER_LANE)
     return launch_hermite_uniform_spl(B.n, B, nunits, P, grid, st, blocks);
+  if (P.n_obs > 0)
+    return B.n <= 8 ? launch_hermite_obs_bpl_a(B.n, B, nunits, P, grid, st, blocks)
+                    : launch_hermite_obs_bpl_b(B.n, B, nunits, P, grid, st, blocks);
   if (B.n <= 4) return launch_hermite_uniform_bpl_s(B.n, B, nunits, P, grid, st, blocks);
   if (B.n <= 8) return launch_hermite_uniform_bpl_a(B.n, B, nunits, P, grid, st, blocks);
   return launch_hermite_uniform_bpl_b(B.n, B, nunits, P, grid, st, blocks);
