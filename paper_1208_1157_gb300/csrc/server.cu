@@ -57,18 +57,13 @@ struct Pool {
   std::set<int> free_slots;    // lowest slots are handed out first
   std::vector<int64_t> owner;  // request id per slot, -1 if free
   std::vector<int32_t> owner_sys;  // the slot's system within its request
-  int32_t *d_list = nullptr;   // occupied slots of the current round (device)
-  std::vector<int32_t> h_list;
   int32_t *h_status = nullptr; // pinned copy of the slots' status after a round
-  int *d_next = nullptr;       // work counter of the pool's launch
   int blocks = 0;              // resident CTAs per SM of the pool's kernel
   size_t bytes = 0;
 };
 
 void free_pool(Pool *q) {
   cudaFree(q->block);
-  cudaFree(q->d_list);
-  cudaFree(q->d_next);
   cudaFreeHost(q->h_status);
 }
 
@@ -93,39 +88,85 @@ struct Request {
   std::vector<int32_t> out_status;
 };
 
-// scatter one request's systems into pool slots
-__global__ void admit_kernel(BinView B, double *t_end_slots, const int *__restrict__ slots, int n_sys,
-                             const double *__restrict__ pos, const double *__restrict__ vel,
-                             const double *__restrict__ mass, double t0, double t_end) {
-  int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= n_sys) return;
-  const int s = slots[i], n = B.n;
-  for (int b = 0; b < n; b++) {
-    for (int c = 0; c < 3; c++) {
-      B.x[(size_t)(c * n + b) * B.S_pad + s] = pos[3 * ((size_t)i * n + b) + c];
-      B.v[(size_t)(c * n + b) * B.S_pad + s] = vel[3 * ((size_t)i * n + b) + c];
-    }
-    B.m[(size_t)b * B.S_pad + s] = mass[(size_t)i * n + b];
-  }
-  B.t[s] = t0;
-  B.status[s] = SWARM_SYS_ACTIVE;
-  t_end_slots[s] = t_end;
+// What the staging kernels need of up to kBatch parts (a request's systems on admission, a
+// pool's finished ones on retirement): one launch for all of them, blockIdx.y the part, a thread
+// per body component.  (A launch each with a thread per system, its loads one after the other: 30 us
+// per pool; all pools of a round in one: 5 us.)
+constexpr int kBatch = 32;
+struct StagePart {
+  double *x, *v, *m, *t, *t_end_slots;
+  int32_t *status;
+  int n, S_pad, n_sys, slots;  // slots: offset into the slot list
+  size_t stage;                // offset into the staging buffer: pos, vel, then mass or time and status
+  double t0, t_end;
+};
+struct StageBatch {
+  StagePart part[kBatch];
+};
+static StagePart stage_part(const Pool &p, int n_sys, size_t s_off, size_t d_off) {
+  StagePart q{};
+  q.x = p.view.x;
+  q.v = p.view.v;
+  q.m = const_cast<double *>(p.view.m);
+  q.t = p.view.t;
+  q.t_end_slots = p.t_end;
+  q.status = p.view.status;
+  q.n = p.n;
+  q.S_pad = p.view.S_pad;
+  q.n_sys = n_sys;
+  q.slots = (int)s_off;
+  q.stage = d_off;
+  return q;
+}
+// blocks of 256 threads for the largest part
+static dim3 stage_grid(const StageBatch &b, int parts) {
+  int most = 1;
+  for (int i = 0; i < parts; i++) most = std::max(most, (int)((3ll * b.part[i].n * b.part[i].n_sys + 255) / 256));
+  return dim3((unsigned)most, (unsigned)parts);
 }
 
-// gather finished systems of one pool (the listed slots, in list order) and free their slots
-__global__ void retire_kernel(BinView B, const int *__restrict__ slots, int n_sys, double *__restrict__ pos,
-                              double *__restrict__ vel, double *__restrict__ time, int32_t *__restrict__ status) {
-  int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= n_sys) return;
-  const int s = slots[i], n = B.n;
-  for (int b = 0; b < n; b++)
-    for (int c = 0; c < 3; c++) {
-      pos[3 * ((size_t)i * n + b) + c] = B.x[(size_t)(c * n + b) * B.S_pad + s];
-      vel[3 * ((size_t)i * n + b) + c] = B.v[(size_t)(c * n + b) * B.S_pad + s];
-    }
-  time[i] = B.t[s];
-  status[i] = B.status[s];
-  B.status[s] = kFree;
+// scatter requests' systems into pool slots
+__global__ void admit_kernel(StageBatch batch, const int *__restrict__ slots, const double *__restrict__ stage) {
+  const StagePart &p = batch.part[blockIdx.y];
+  const int e = blockIdx.x * blockDim.x + threadIdx.x, n3 = 3 * p.n;
+  if (e >= p.n_sys * n3) return;
+  const int i = e / n3, r = e - i * n3, b = r / 3, c = r - 3 * b, s = slots[p.slots + i];
+  const double *pos = stage + p.stage, *vel = pos + (size_t)p.n_sys * n3, *mass = vel + (size_t)p.n_sys * n3;
+  p.x[(size_t)(c * p.n + b) * p.S_pad + s] = pos[e];
+  p.v[(size_t)(c * p.n + b) * p.S_pad + s] = vel[e];
+  if (c == 0) p.m[(size_t)b * p.S_pad + s] = mass[(size_t)i * p.n + b];
+  if (r == 0) {
+    p.t[s] = p.t0;
+    p.status[s] = SWARM_SYS_ACTIVE;
+    p.t_end_slots[s] = p.t_end;
+  }
+}
+
+// gather finished systems of the pools (the listed slots, in list order) and free their slots
+__global__ void retire_kernel(StageBatch batch, const int *__restrict__ slots, double *__restrict__ stage) {
+  const StagePart &p = batch.part[blockIdx.y];
+  const int e = blockIdx.x * blockDim.x + threadIdx.x, n3 = 3 * p.n;
+  if (e >= p.n_sys * n3) return;
+  const int i = e / n3, r = e - i * n3, b = r / 3, c = r - 3 * b, s = slots[p.slots + i];
+  double *pos = stage + p.stage, *vel = pos + (size_t)p.n_sys * n3, *time = vel + (size_t)p.n_sys * n3;
+  pos[e] = p.x[(size_t)(c * p.n + b) * p.S_pad + s];
+  vel[e] = p.v[(size_t)(c * p.n + b) * p.S_pad + s];
+  if (r == 0) {
+    time[i] = p.t[s];
+    ((int32_t *)(time + p.n_sys))[i] = p.status[s];
+    p.status[s] = kFree;
+  }
+}
+
+// the pools' statuses to their pinned host copies
+struct StatusBatch {
+  const int32_t *from[kBatch];
+  int32_t *to[kBatch];
+  int n[kBatch];
+};
+__global__ void status_kernel(StatusBatch b) {
+  const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  if (i < b.n[blockIdx.y]) b.to[blockIdx.y][i] = b.from[blockIdx.y][i];
 }
 
 __global__ void fill_status_kernel(int32_t *st, int n, int v) {
@@ -152,7 +193,12 @@ struct swarm_server {
   cudaStream_t side[kSide] = {};
   cudaEvent_t side_done[kSide] = {};
   cudaEvent_t fork_ev = nullptr;
-  unsigned long long *d_counters = nullptr;
+  // the occupied slots of a round, pool after pool (device and pinned), and the launches' work
+  // counters: one copy and one memset per round
+  int32_t *d_lists = nullptr, *h_lists = nullptr;
+  int *d_next = nullptr;
+  size_t list_cap = 0, next_cap = 0;
+  unsigned long long *d_counters = nullptr, *h_counters = nullptr;
   cudaEvent_t ev0 = nullptr, ev1 = nullptr;
   swarm_server_stats stats{};
 };
@@ -212,10 +258,7 @@ static int make_pool(swarm_server *sv, int integ, int n, Pool **out) {
   for (int i = 0; i < cap; i++) p->free_slots.insert(p->free_slots.end(), i);
   p->owner.assign(cap, -1);
   p->owner_sys.assign(cap, -1);
-  SCK(cudaMalloc(&p->d_list, sizeof(int32_t) * cap));
-  SCK(cudaMalloc(&p->d_next, sizeof(int)));
   SCK(cudaMallocHost(&p->h_status, sizeof(int32_t) * cap));
-  p->h_list.reserve(cap);
   // body-per-lane kernels that take the slot list and hand slots out per group
   StepParams Q{};
   Q.integrator = integ;
@@ -244,6 +287,7 @@ extern "C" int swarm_server_create(const swarm_server_config *cfg, void *cuda_st
   SCK(cudaMalloc(&sv->d_slots, sizeof(int) * kStageSlots));
   SCK(cudaMallocHost(&sv->h_slots, sizeof(int) * kStageSlots));
   SCK(cudaMalloc(&sv->d_counters, sizeof(unsigned long long) * 4));
+  SCK(cudaMallocHost(&sv->h_counters, sizeof(unsigned long long) * 4));
   SCK(cudaEventCreate(&sv->ev0));
   SCK(cudaEventCreate(&sv->ev1));
   SCK(cudaEventCreateWithFlags(&sv->fork_ev, cudaEventDisableTiming));
@@ -270,6 +314,10 @@ extern "C" void swarm_server_destroy(swarm_server *sv) {
   cudaFreeHost(sv->h_stage);
   cudaFreeHost(sv->h_slots);
   cudaFree(sv->d_counters);
+  cudaFreeHost(sv->h_counters);
+  cudaFree(sv->d_lists);
+  cudaFreeHost(sv->h_lists);
+  cudaFree(sv->d_next);
   cudaEventDestroy(sv->ev0);
   cudaEventDestroy(sv->ev1);
   delete sv;
@@ -332,19 +380,23 @@ static int admit(swarm_server *sv) {
   };
   std::vector<Item> batch;
   size_t d_used = 0, s_used = 0;
-  auto flush = [&]() -> int {
+  auto flush = [&](bool more) -> int {
     if (batch.empty()) return SWARM_OK;
     SCK(cudaMemcpyAsync(sv->d_stage, sv->h_stage, sizeof(double) * d_used, cudaMemcpyHostToDevice, sv->stream));
     SCK(cudaMemcpyAsync(sv->d_slots, sv->h_slots, sizeof(int) * s_used, cudaMemcpyHostToDevice, sv->stream));
-    for (auto &it : batch) {
-      Request *r = it.r;
-      const size_t nb = (size_t)it.count * r->n;
-      const double *dpos = sv->d_stage + it.d_off, *dvel = dpos + 3 * nb, *dmass = dvel + 3 * nb;
-      admit_kernel<<<(it.count + 127) / 128, 128, 0, sv->stream>>>(r->pool->view, r->pool->t_end, sv->d_slots + it.s_off,
-                                                                    it.count, dpos, dvel, dmass, r->t0, r->t_end);
+    for (size_t i0 = 0; i0 < batch.size(); i0 += kBatch) {
+      StageBatch sb;
+      const int k = (int)std::min<size_t>(kBatch, batch.size() - i0);
+      for (int i = 0; i < k; i++) {
+        const Item &it = batch[i0 + i];
+        sb.part[i] = stage_part(*it.r->pool, it.count, it.s_off, it.d_off);
+        sb.part[i].t0 = it.r->t0;
+        sb.part[i].t_end = it.r->t_end;
+      }
+      admit_kernel<<<stage_grid(sb, k), 256, 0, sv->stream>>>(sb, sv->d_slots, sv->d_stage);
       SCK(cudaGetLastError());
     }
-    SCK(cudaStreamSynchronize(sv->stream));  // the staging buffers are reused by the next batch
+    if (more) SCK(cudaStreamSynchronize(sv->stream));  // the next batch reuses the staging buffers
     batch.clear();
     d_used = s_used = 0;
     return SWARM_OK;
@@ -370,7 +422,7 @@ static int admit(swarm_server *sv) {
     if (k > 0) {
       const size_t nb = (size_t)k * r->n;
       if (d_used + 7 * nb > sv->stage_doubles || s_used + k > (size_t)kStageSlots) {
-        int rc = flush();
+        int rc = flush(true);
         if (rc) return rc;
       }
       const int first = r->admitted;
@@ -406,12 +458,12 @@ static int admit(swarm_server *sv) {
     std::vector<double>().swap(r->mass);
     it = sv->queue.erase(it);
   }
-  return flush();
+  return flush(false);  // (step() waits for the stream before it writes them again)
 }
 
-// Retirement, system by system: the statuses of every occupied pool come back in one
-// round of copies; every slot whose system reached its end time or stopped is gathered
-// (one kernel per pool over the list of its finished slots, the batch in one copy to the
+// Retirement, system by system: the round has left the statuses of every occupied pool in
+// its host copy; every slot whose system reached its end time or stopped is gathered
+// (one launch over the lists of the pools' finished slots, the batch in one copy to the
 // pinned staging buffer), its result goes to its request's host buffer and the slot is
 // free for the next admission.  A request completes with its last system.
 static int retire(swarm_server *sv, int32_t *n_completed) {
@@ -419,11 +471,9 @@ static int retire(swarm_server *sv, int32_t *n_completed) {
   for (auto &kv : sv->pools) {
     Pool *p = kv.second.get();
     if ((int)p->free_slots.size() == p->cap) continue;
-    SCK(cudaMemcpyAsync(p->h_status, p->view.status, sizeof(int32_t) * p->cap, cudaMemcpyDeviceToHost, sv->stream));
     occ.push_back(p);
   }
   if (occ.empty()) return SWARM_OK;
-  SCK(cudaStreamSynchronize(sv->stream));
   struct Item {
     Pool *p;
     int count;
@@ -434,12 +484,11 @@ static int retire(swarm_server *sv, int32_t *n_completed) {
   auto flush = [&]() -> int {
     if (batch.empty()) return SWARM_OK;
     SCK(cudaMemcpyAsync(sv->d_slots, sv->h_slots, sizeof(int) * s_used, cudaMemcpyHostToDevice, sv->stream));
-    for (auto &it : batch) {
-      const size_t nb = (size_t)it.count * it.p->n;
-      double *dpos = sv->d_stage + it.d_off, *dvel = dpos + 3 * nb, *dtime = dvel + 3 * nb;
-      int32_t *dstat = (int32_t *)(dtime + it.count);
-      retire_kernel<<<(it.count + 127) / 128, 128, 0, sv->stream>>>(it.p->view, sv->d_slots + it.s_off, it.count, dpos,
-                                                                     dvel, dtime, dstat);
+    for (size_t i0 = 0; i0 < batch.size(); i0 += kBatch) {
+      StageBatch sb;
+      const int k = (int)std::min<size_t>(kBatch, batch.size() - i0);
+      for (int i = 0; i < k; i++) sb.part[i] = stage_part(*batch[i0 + i].p, batch[i0 + i].count, batch[i0 + i].s_off, batch[i0 + i].d_off);
+      retire_kernel<<<stage_grid(sb, k), 256, 0, sv->stream>>>(sb, sv->d_slots, sv->d_stage);
       SCK(cudaGetLastError());
     }
     SCK(cudaMemcpyAsync(sv->h_stage, sv->d_stage, sizeof(double) * d_used, cudaMemcpyDeviceToHost, sv->stream));
@@ -522,17 +571,39 @@ extern "C" int swarm_server_step(swarm_server *sv, int32_t *n_completed) {
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     const int K = std::min((int)run.size(), kSide);
+    size_t slots = 0;
+    for (Pool *p : run) slots += (size_t)p->cap;
+    if (slots > sv->list_cap) {
+      cudaFree(sv->d_lists);
+      cudaFreeHost(sv->h_lists);
+      sv->d_lists = sv->h_lists = nullptr;
+      sv->list_cap = 0;
+      SCK(cudaMalloc(&sv->d_lists, sizeof(int32_t) * slots));
+      SCK(cudaMallocHost(&sv->h_lists, sizeof(int32_t) * slots));
+      sv->list_cap = slots;
+    }
+    if (run.size() > sv->next_cap) {
+      cudaFree(sv->d_next);
+      sv->d_next = nullptr;
+      sv->next_cap = 0;
+      SCK(cudaMalloc(&sv->d_next, sizeof(int) * run.size()));
+      sv->next_cap = run.size();
+    }
+    std::vector<size_t> first(run.size() + 1, 0);
+    for (size_t i = 0; i < run.size(); i++) {
+      int32_t *l = sv->h_lists + first[i];
+      for (int slot = 0; slot < run[i]->cap; slot++)
+        if (run[i]->owner[slot] >= 0) *l++ = slot;
+      first[i + 1] = (size_t)(l - sv->h_lists);
+    }
+    SCK(cudaMemcpyAsync(sv->d_lists, sv->h_lists, sizeof(int32_t) * first.back(), cudaMemcpyHostToDevice, sv->stream));
+    SCK(cudaMemsetAsync(sv->d_next, 0, sizeof(int) * run.size(), sv->stream));
     SCK(cudaEventRecord(sv->fork_ev, sv->stream));
     for (int j = 0; j < K; j++) SCK(cudaStreamWaitEvent(sv->side[j], sv->fork_ev, 0));
     for (size_t i = 0; i < run.size(); i++) {
       Pool *p = run[i];
       cudaStream_t st = sv->side[i % K];
-      p->h_list.clear();
-      for (int slot = 0; slot < p->cap; slot++)
-        if (p->owner[slot] >= 0) p->h_list.push_back(slot);
-      const int nl = (int)p->h_list.size();
-      SCK(cudaMemcpyAsync(p->d_list, p->h_list.data(), sizeof(int32_t) * nl, cudaMemcpyHostToDevice, st));
-      SCK(cudaMemsetAsync(p->d_next, 0, sizeof(int), st));
+      const int nl = (int)(first[i + 1] - first[i]);
       StepParams P{};
       P.t_end = 0;
       P.dt = p->integ == SWARM_HERMITE4 ? sv->cfg.hermite_dt : sv->cfg.mvs_dt;
@@ -541,10 +612,10 @@ extern "C" int swarm_server_step(swarm_server *sv, int32_t *n_completed) {
       P.ce_factor = sv->cfg.ce_hill_factor;
       P.eject2 = sv->cfg.eject_radius > 0 ? sv->cfg.eject_radius * sv->cfg.eject_radius : 0.0;
       P.counters = sv->d_counters;
-      P.work_next = p->d_next;
+      P.work_next = sv->d_next + i;
       P.max_steps = sv->cfg.quantum_steps;
       BinView v = p->view;
-      v.list = p->d_list;
+      v.list = sv->d_lists + first[i];
       v.nlist = nl;
       const int per = 32 / p->n;
       const int nunits = (nl + per - 1) / per;
@@ -563,10 +634,24 @@ extern "C" int swarm_server_step(swarm_server *sv, int32_t *n_completed) {
     ran = true;
   }
   SCK(cudaEventRecord(sv->ev1, sv->stream));
+  for (size_t i0 = 0; i0 < run.size(); i0 += kBatch) {
+    StatusBatch sb;
+    const int k = (int)std::min<size_t>(kBatch, run.size() - i0);
+    int most = 1;
+    for (int i = 0; i < k; i++) {
+      Pool *p = run[i0 + i];
+      sb.from[i] = p->view.status;
+      sb.to[i] = p->h_status;
+      sb.n[i] = p->cap;
+      most = std::max(most, p->cap);
+    }
+    status_kernel<<<dim3((most + 255) / 256, k), 256, 0, sv->stream>>>(sb);
+    SCK(cudaGetLastError());
+  }
+  if (ran) SCK(cudaMemcpyAsync(sv->h_counters, sv->d_counters, sizeof(unsigned long long) * 4, cudaMemcpyDeviceToHost, sv->stream));
   SCK(cudaStreamSynchronize(sv->stream));
   if (ran) {
-    unsigned long long c[4];
-    SCK(cudaMemcpy(c, sv->d_counters, sizeof c, cudaMemcpyDeviceToHost));
+    const unsigned long long *c = sv->h_counters;
     float ms = 0;
     SCK(cudaEventElapsedTime(&ms, sv->ev0, sv->ev1));
     sv->stats.system_steps += (int64_t)c[0];
