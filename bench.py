@@ -107,7 +107,8 @@ def source_hash(patterns):
 
 # the sources of the benchmark's kernel (hermite_uniform_kernel, system per lane)
 HERMITE_SOURCES = ["paper_1208_1157_gb300/csrc/hermite.cuh", "paper_1208_1157_gb300/csrc/hermite_impl.cuh",
-                   "paper_1208_1157_gb300/csrc/hermite_uniform_spl.cu", "paper_1208_1157_gb300/csrc/common.cuh"]
+                   "paper_1208_1157_gb300/csrc/hermite_uniform_spl.cu", "paper_1208_1157_gb300/csrc/common.cuh",
+                   "paper_1208_1157_gb300/csrc/ff.cuh", "paper_1208_1157_gb300/csrc/hermite_ff.cuh"]
 
 
 def traffic_per_launch(kernel, systems):
@@ -368,8 +369,6 @@ def secondary(S, torch, stream, peak):
                                                           ctas=1)
     out["c2_persistent_body_per_lane_1cta_500"] = timed(c2, 500 * DT, S.HERMITE4, DT, mapping=S.MAP_BODY_PER_LANE,
                                                         ctas=1)
-    out["c2_persistent_system_per_lane_3cta_500"] = timed(c2, 500 * DT, S.HERMITE4, DT, mapping=S.MAP_SYSTEM_PER_LANE,
-                                                          ctas=3)
     c3 = ics.ragged(65536, seed=3)
     out["c3_ragged_hermite_per_bin_launches_1e4_steps"] = timed_per_bin(S, stream, c3, 1e4 * DT, DT, peak)
     out["c3_ragged_hermite_single_launch_1e4_steps"] = timed_per_bin(S, stream, c3, 1e4 * DT, DT, peak, single=1)
@@ -710,6 +709,10 @@ def run_ours(args):
                      "implemented_form": "star-relative coordinates with the barycentre's drift: the same map in exact "
                                          "arithmetic with fewer operations (633 at n = 3)",
                      "peak_kind": "measured DFMA-chain peak on this GPU (2 flops per DFMA), of measured",
+                     "note": "the method's flops over the FP64 pipe's peak: the kernel keeps the state and the star's "
+                             "pull in FP64 and forms the rest as pairs of FP32 numbers, so most of these flops do not "
+                             "run on the FP64 pipe and the fraction can exceed 1 (profiles/: that pipe is 57 % busy, "
+                             "the issue slots 58 %)",
                      "peak_clocks": peak_clocks,
                      "avg_launch_ms": launch_ms},
         "e2e": {"value": e2e_steps / e2e_wall, "unit": "system-steps/s", "h2d_bytes_per_step": bytes_io,

@@ -808,12 +808,13 @@ static int run_persistent(swarm_ensemble *e, const StepParams &P0, int integrato
   if (nconc > 1 && (rc = ensure_side(e))) return rc;
   auto enqueue = [&](cudaStream_t cs, const StepParams &Q) -> int {
     const int K = nconc > 1 ? std::min((int)uni.size(), kSideStreams) : 0;
+    // every launch's work counter (the shared launch's, then one per bin)
+    CK(cudaMemsetAsync(e->d_work_next, 0, sizeof(int) * (1 + uni.size()), cs));
     if (K) {
       CK(cudaEventRecord(e->fork_ev, cs));
       for (int j = 0; j < K; j++) CK(cudaStreamWaitEvent(e->side[j], e->fork_ev, 0));
     }
     if (!per_bin) {  // the shared launch stays on the main stream
-      CK(cudaMemsetAsync(e->d_work_next, 0, sizeof(int), cs));
       if (hermite_family(integrator)) CK(launch_hermite_persistent(e->d_bins, e->d_work, e->nwork, Q, grid, cs));
       else CK(launch_mvs_persistent(e->d_bins, e->d_work, e->nwork, Q, grid, cs));
     }
@@ -823,7 +824,6 @@ static int run_persistent(swarm_ensemble *e, const StepParams &P0, int integrato
       cudaStream_t si = K ? e->side[i % K] : cs;
       StepParams Qi = Q;
       Qi.work_next = e->d_work_next + 1 + i;
-      CK(cudaMemsetAsync(Qi.work_next, 0, sizeof(int), si));
       if (compact) CK(live_list(uni[i].view, const_cast<int32_t *>(uni[i].view.list),
                                 const_cast<int *>(uni[i].view.nlist_dev), si));
       CK(launch_uni(uni[i], Qi, uni[i].grid, si, nullptr));
