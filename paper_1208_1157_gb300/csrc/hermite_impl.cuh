@@ -106,9 +106,12 @@ __device__ __forceinline__ void spl_hermite_body(const BinView &B, const StepPar
 // present length, and a longer step is taken in FP64.  A system that comes to level 0 stays
 // in FP64 (eta is about tau / sqrt 2 all along an orbit, and lanes that change back and forth
 // at their own times would make a warp take both kinds of step).  131072 x 3 systems over a
-// quarter of an inner period: 37.4 -> 18 ms; the loop is long enough to miss the instruction
-// cache (lanes are at different points of their systems).
-template <int N, class Take>
+// quarter of an inner period: 37.4 ms wholly in FP64, now 15.
+// CTA: the warps of a CTA take their steps together.  The loop is longer than the instruction
+// cache (4500 instructions), and warps at different places of it would each fetch all of it for
+// themselves: 131072 systems over a quarter period 18.5 -> 15.0 ms, 65536 11.1 -> 10.2, 30011
+// 5.1 either way (the longest system's chain); adaptive Cash-Karp, 131072 systems 20.8 -> 10.6.
+template <int N, bool CTA, class Take>
 __device__ __forceinline__ void spl_hermite_adaptive_run(const BinView &B, const StepParams &P, Take take) {
   const bool printed = P.corr_form != 0;  // warp-uniform
   const unsigned FULL = 0xffffffffu;
@@ -168,7 +171,9 @@ __device__ __forceinline__ void spl_hermite_adaptive_run(const BinView &B, const
         }
       }
     }
-    if (!__any_sync(FULL, has || !exhausted)) break;
+    bool more = __any_sync(FULL, has || !exhausted);
+    if (CTA) more = __syncthreads_or(more);
+    if (!more) break;
     if (!has) continue;
     int code = 0;
     bool reached = false;
@@ -213,13 +218,13 @@ __device__ __forceinline__ void spl_hermite_adaptive_run(const BinView &B, const
 }
 template <int N>
 __device__ __forceinline__ void spl_hermite_adaptive_stream(const BinView &B, const StepParams &P) {
-  spl_hermite_adaptive_run<N>(B, P, [&]() { return stream_system(B, atomicAdd(P.work_next, 1)); });
+  spl_hermite_adaptive_run<N, true>(B, P, [&]() { return stream_system(B, atomicAdd(P.work_next, 1)); });
 }
 // one unit: 32 consecutive entries of the launch's system order
 template <int N>
 __device__ __forceinline__ void spl_hermite_adaptive_body(const BinView &B, const StepParams &P, int unit) {
   bool taken = false;
-  spl_hermite_adaptive_run<N>(B, P, [&]() {
+  spl_hermite_adaptive_run<N, false>(B, P, [&]() {
     const int s = taken ? -1 : stream_system(B, unit * 32 + (threadIdx.x & 31));
     taken = true;
     return s;

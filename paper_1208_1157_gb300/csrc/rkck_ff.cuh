@@ -443,7 +443,9 @@ __device__ __forceinline__ void spl_rkck_stream(const BinView &B, const StepPara
         }
       }
     }
-    if (!__any_sync(FULL, has || !exhausted)) break;
+    bool more = __any_sync(FULL, has || !exhausted);
+    if (ADAPT) more = __syncthreads_or(more);  // see spl_hermite_adaptive_run
+    if (!more) break;
     // the new states' evaluation (also a refill's: one copy)
     float q2[N], d2[N][N];
     if (fresh) {
