@@ -682,10 +682,10 @@ static int run_persistent(swarm_ensemble *e, const StepParams &P0, int integrato
       else if (span >= 5000) bin_ctas[i] = 2;
     }
     // adaptive system per lane: the kernel's full residency (131072 x 3 systems over a
-    // quarter of an inner period: 17.1 ms at two CTAs per SM, 28.9 ms at one, whose single
-    // warp per sub-partition leaves both the FP64 and the FP32 pipe waiting); the printed
-    // corrector's steps are FP64, one warp fills that pipe, and one CTA per SM gives every
-    // lane more systems and the call a smaller tail
+    // quarter of an inner period: 15.0 ms at two CTAs per SM; with one warp per sub-partition
+    // both the FP64 and the FP32 pipe wait, 1.7 times as long); the printed corrector's steps
+    // are FP64, one warp fills that pipe, and one CTA per SM gives every lane more systems
+    // and the call a smaller tail
     if (integrator == SWARM_HERMITE4_ADAPTIVE && m == SWARM_MAP_SYSTEM_PER_LANE && !e->ctas_per_sm)
       bin_ctas[i] = P.corr_form ? 1 : 0;
   }

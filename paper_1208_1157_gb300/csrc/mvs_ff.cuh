@@ -19,7 +19,7 @@
 // so that a system alone and in an ensemble moves bit for bit alike.  The monitor's tests run
 // in FP32 with a margin and, where one of them is met, again in FP64.
 //
-// Bound: the FP64 pipe (72 instructions per warp and step at n = 8 Jacobi, 65 % busy with three
+// Bound: the FP64 pipe (79 instructions per warp and step at n = 8 Jacobi, 68 % busy with three
 // CTAs per SM) and the latency of the drift's chain of 3200 instructions (a step of one system
 // alone: 6.6 us), so 168 registers for three warps per sub-partition (two: 1.31 ms for 40 steps of
 // 16384 systems, three: 1.18).  Before, wholly in FP64, -> now: 16384 Jacobi systems of 8 bodies

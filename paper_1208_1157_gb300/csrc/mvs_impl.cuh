@@ -6,6 +6,8 @@
 // kick half step, Kepler drift, kick half step, Cartesian drift half step (DH); kick,
 // Kepler, kick (Jacobi).  The interaction accelerations computed after the Kepler drift
 // are reused by the next step's first kick (Sec. 4.3.4): one force evaluation per step.
+// Here: the coordinate maps, and the drift and the accelerations in FP64, for the parts of a step
+// that mvs_ff.cuh's pairs do not carry and for 16..32 bodies.
 #pragma once
 #include "hermite.cuh"
 #include "kernels.h"
