@@ -203,6 +203,49 @@ __global__ void __launch_bounds__(kPackThreads) pack_kernel(BinView B, const int
   }
 }
 
+// The same for an ensemble of several bins in one launch, blockIdx.y the bin (13 bins one after
+// the other, a thread per system, its loads in turn: 777 systems of 3..15 bodies 113 us in, 223
+// us out; now 27 and 14; 65536 systems 253 and 227, now 137 and 38).  unpack: a thread per system and every eighth component, so that the SoA rows
+// are written 32 systems at a time; pack: a warp per system, so that the caller's rows are.
+__global__ void __launch_bounds__(256) unpack_bins_kernel(const BinView *__restrict__ bins, const int64_t *__restrict__ offs,
+                                                          const double *__restrict__ pos, const double *__restrict__ vel,
+                                                          const double *__restrict__ mass, const double *__restrict__ time,
+                                                          const int32_t *__restrict__ status) {
+  const BinView B = bins[blockIdx.y];
+  const int s = blockIdx.x * 32 + (threadIdx.x & 31), n = B.n;
+  if (s >= B.S) return;
+  const int g = B.gidx[s];
+  const int64_t o = offs[g];
+  for (int r = threadIdx.x >> 5; r < 3 * n; r += 8) {
+    const int b = r / 3, c = r - 3 * b;
+    const size_t i = (size_t)(c * n + b) * B.S_pad + s;
+    if (pos) B.x[i] = pos[3 * o + r];
+    if (vel) B.v[i] = vel[3 * o + r];
+    if (mass && c == 0) B.m[(size_t)b * B.S_pad + s] = mass[o + b];
+  }
+  if (threadIdx.x >= 32) return;
+  if (time) B.t[s] = time[g];
+  if (status) B.status[s] = status[g];
+}
+__global__ void __launch_bounds__(256) pack_bins_kernel(const BinView *__restrict__ bins, const int64_t *__restrict__ offs,
+                                                        double *__restrict__ pos, double *__restrict__ vel,
+                                                        double *__restrict__ time, int32_t *__restrict__ status) {
+  const BinView B = bins[blockIdx.y];
+  const int s = blockIdx.x * 8 + (threadIdx.x >> 5), lane = threadIdx.x & 31, n = B.n;
+  if (s >= B.S) return;
+  const int g = B.gidx[s];
+  const int64_t o = offs[g];
+  for (int r = lane; r < 3 * n; r += 32) {
+    const int b = r / 3, c = r - 3 * b;
+    const size_t i = (size_t)(c * n + b) * B.S_pad + s;
+    if (pos) pos[3 * o + r] = B.x[i];
+    if (vel) vel[3 * o + r] = B.v[i];
+  }
+  if (lane) return;
+  if (time) time[g] = B.t[s];
+  if (status) status[g] = B.status[s];
+}
+
 // Eq. 6 (each pair once, 1/sqrt in full precision) and L = sum m x cross v, per system.
 __global__ void diag_kernel(BinView B, double *__restrict__ out) {
   const int s = blockIdx.x * blockDim.x + threadIdx.x;
@@ -289,6 +332,21 @@ static int ensure_side(swarm_ensemble *e) {
   return SWARM_OK;
 }
 
+// device arrays in the caller's layout into the bins
+static int unpack_from(const swarm_ensemble *e, const double *pos, const double *vel, const double *mass, const double *time,
+                       const int32_t *status) {
+  int most = 0;
+  for (auto &b : e->bins) most = std::max(most, b.S);
+  if (e->bins.size() > 1) {
+    unpack_bins_kernel<<<dim3((most + 31) / 32, (unsigned)e->bins.size()), 256, 0, e->stream>>>(e->d_bins, e->d_offs, pos, vel,
+                                                                                               mass, time, status);
+  } else {
+    unpack_kernel<<<(most + 127) / 128, 128, 0, e->stream>>>(e->bins[0].view(), e->d_offs, pos, vel, mass, time, status);
+  }
+  CK(cudaGetLastError());
+  return SWARM_OK;
+}
+
 static int upload_state(swarm_ensemble *e, const double *pos, const double *vel, const double *mass,
                         const double *time, const int32_t *status) {
   cudaStream_t st = e->stream;
@@ -297,14 +355,8 @@ static int upload_state(swarm_ensemble *e, const double *pos, const double *vel,
   if (mass) CK(cudaMemcpyAsync(e->stage_mass(), mass, sizeof(double) * e->n_bodies, cudaMemcpyHostToDevice, st));
   if (time) CK(cudaMemcpyAsync(e->stage_time(), time, sizeof(double) * e->n_sys, cudaMemcpyHostToDevice, st));
   if (status) CK(cudaMemcpyAsync(e->d_stage_status, status, sizeof(int32_t) * e->n_sys, cudaMemcpyHostToDevice, st));
-  for (auto &b : e->bins) {
-    unpack_kernel<<<(b.S + 127) / 128, 128, 0, st>>>(b.view(), e->d_offs, pos ? e->stage_pos() : nullptr,
-                                                     vel ? e->stage_vel() : nullptr, mass ? e->stage_mass() : nullptr,
-                                                     time ? e->stage_time() : nullptr,
-                                                     status ? e->d_stage_status : nullptr);
-    CK(cudaGetLastError());
-  }
-  return SWARM_OK;
+  return unpack_from(e, pos ? e->stage_pos() : nullptr, vel ? e->stage_vel() : nullptr, mass ? e->stage_mass() : nullptr,
+                     time ? e->stage_time() : nullptr, status ? e->d_stage_status : nullptr);
 }
 
 // ------------------------------------------------------------------ create / destroy
@@ -682,8 +734,8 @@ static int run_persistent(swarm_ensemble *e, const StepParams &P0, int integrato
       else if (span >= 5000) bin_ctas[i] = 2;
     }
     // adaptive system per lane: the kernel's full residency (131072 x 3 systems over a
-    // quarter of an inner period: 15.0 ms at two CTAs per SM; with one warp per sub-partition
-    // both the FP64 and the FP32 pipe wait, 1.7 times as long); the printed corrector's steps
+    // quarter of an inner period: 15.0 ms at two CTAs per SM, 20.2 at one, whose single warp per
+    // sub-partition leaves both the FP64 and the FP32 pipe waiting); the printed corrector's steps
     // are FP64, one warp fills that pipe, and one CTA per SM gives every lane more systems
     // and the call a smaller tail
     if (integrator == SWARM_HERMITE4_ADAPTIVE && m == SWARM_MAP_SYSTEM_PER_LANE && !e->ctas_per_sm)
@@ -943,11 +995,17 @@ extern "C" int swarm_set_state(swarm_ensemble *e, const double *pos, const doubl
 }
 
 static int pack_to(const swarm_ensemble *e, double *pos, double *vel, double *time, int32_t *status) {
-  for (auto &b : e->bins) {
+  if (e->bins.size() > 1) {
+    int most = 0;
+    for (auto &b : e->bins) most = std::max(most, b.S);
+    pack_bins_kernel<<<dim3((most + 7) / 8, (unsigned)e->bins.size()), 256, 0, e->stream>>>(e->d_bins, e->d_offs, pos, vel,
+                                                                                           time, status);
+  } else {
+    const Bin &b = e->bins[0];
     pack_kernel<<<(b.S + kPackThreads - 1) / kPackThreads, kPackThreads, 0, e->stream>>>(b.view(), e->d_offs, pos, vel,
                                                                                        time, status);
-    CK(cudaGetLastError());
   }
+  CK(cudaGetLastError());
   return SWARM_OK;
 }
 
@@ -964,11 +1022,7 @@ extern "C" int swarm_set_state_dev(swarm_ensemble *e, const double *d_pos, const
     e->t_lo = *std::min_element(h.begin(), h.end());
     e->t_hi = *std::max_element(h.begin(), h.end());
   }
-  for (auto &b : e->bins) {
-    unpack_kernel<<<(b.S + 127) / 128, 128, 0, st>>>(b.view(), e->d_offs, d_pos, d_vel, nullptr, d_time, d_status);
-    CK(cudaGetLastError());
-  }
-  return SWARM_OK;
+  return unpack_from(e, d_pos, d_vel, nullptr, d_time, d_status);
 }
 
 extern "C" int swarm_query_state_dev(const swarm_ensemble *e, double *d_pos, double *d_vel, double *d_time,
