@@ -105,6 +105,16 @@ __device__ __forceinline__ float f_from(double d) {
   return __int_as_float((__funnelshift_l(__double2loint(d), e, 3) & 0x7fffffff) | (hi & 0x80000000));
 }
 
+// Whether every value is below 2^64 in size, and neither NaN nor infinite (exponent bits, integer
+// pipe).  NaN, infinity and what is beyond 2^128 come out of the conversions above as ordinary
+// numbers (the exponent's upper bits are dropped), so a test of those does not see them.
+__device__ __forceinline__ bool ff_tame(const double (&a)[3], const double (&b)[3]) {
+  int e = 0;
+#pragma unroll
+  for (int c = 0; c < 3; c++) e = max(e, max(__double2hiint(a[c]) & 0x7fffffff, __double2hiint(b[c]) & 0x7fffffff));
+  return e < (1023 + 64) << 20;
+}
+
 // Pair -> double times 2^-896, on the integer pipe: the float's exponent field is taken over
 // without its rebias, which the DFMA that adds it supplies (`ff_addto`); the lower part is
 // scaled to the double's last place and added to the bits.  Exact for a normalised pair.

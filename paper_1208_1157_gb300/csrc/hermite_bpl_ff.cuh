@@ -474,7 +474,9 @@ __device__ __forceinline__ void bpl_hermite_run(const BinView &B, const StepPara
   const float ejf = P.eject2 > 0.0 ? 0.998f * (float)P.eject2 : __int_as_float(0x7f800000);
 
   int s = 0, steps = 0, level = 0;
-  bool has = false, exhausted = false, scaled = false;
+  // tame: the state the group began with, or its last FP64 step led to, is one that the pairs can
+  // hold (`spl_ff_state` says why the other steps keep it one)
+  bool has = false, exhausted = false, scaled = false, tame = false;
   // the state's acceleration is a0 + da; j0: FP64, or (level > 0) the bits of a pair
   double x[3] = {0.0, 0.0, 0.0}, v[3] = {0.0, 0.0, 0.0}, m = 1.0, a0[3] = {0.0, 0.0, 0.0}, j0[3] = {0.0, 0.0, 0.0};
   float da[3] = {0.0f, 0.0f, 0.0f};
@@ -563,7 +565,9 @@ __device__ __forceinline__ void bpl_hermite_run(const BinView &B, const StepPara
         g.mf = ff_norm(ff_from(m));
         g.mt = (float)((m - (double)g.mf.h) - (double)g.mf.l);
       }
-      const bool sc2 = scaled;
+      const bool tm = (__ballot_sync(FULL, !ff_tame(x, v)) & gm) == 0;
+      if (got) tame = tm;
+      const bool sc2 = scaled && tame;
       BplEval<N> E;
       double an[3], jn[3];
       ff V[3];
@@ -680,12 +684,15 @@ __device__ __forceinline__ void bpl_hermite_run(const BinView &B, const StepPara
           vn[c] = v[c];
         }
         bpl_fp64_advance<N>(P.fk, hd, P.n_corr, printed, m, g, a0, j0, xn, vn, rd);
-        if (active && kind == 0)
+        const bool tm = (__ballot_sync(FULL, !ff_tame(xn, vn)) & gm) == 0;
+        if (active && kind == 0) {
+          tame = tm;
 #pragma unroll
           for (int c = 0; c < 3; c++) {
             x[c] = xn[c];
             v[c] = vn[c];
           }
+        }
       }
     }
     // Level 2: phase 0 evaluates the prediction and corrects it (spl_hermite_delta_step); then,
@@ -725,7 +732,7 @@ __device__ __forceinline__ void bpl_hermite_run(const BinView &B, const StepPara
         if (mine) hn = hs;
         hf = hs.h;
       }
-      const int lE = bpl_level<N>(g, E, hf, scaled && hf > 0.0f && !printed);
+      const int lE = bpl_level<N>(g, E, hf, scaled && tame && hf > 0.0f && !printed);
       if (mine) {
         lv = lE;
         near = !lE || (b != 0 && (E.near || !(E.q2 < ejf)));

@@ -702,7 +702,12 @@ static __device__ __noinline__ int spl_hermite_fp64_run(const F64k &kk, const do
 }
 constexpr int kFP64Run = 16;  // steps between two looks at the level (a look costs 1/8 of an FP64 step)
 
-// Evaluation at a state (x, v): a0, j0, the monitor's distances; returns the level.
+// Evaluation at a state (x, v): a0, j0, the monitor's distances; returns the level, 0 for a state
+// that is not finite or that the pairs cannot hold.  Every state that comes from outside or from
+// an FP64 step is looked at here.  A step from a state of level 1 or 2 cannot leave that range
+// without the level's own tests seeing it: |x| < 2^20, |v| < 2^40 and h < 2^60 (h^2 mu/r^3 <=
+// 2^-8, mu > 2^-60), so the new |x| is below 2^101 and |x|^2, which `f_from` would take for one
+// within `frange` from 2^216 on, below 2^202.
 template <int N, bool STAR>
 __device__ __forceinline__ int spl_ff_state(const F64k &kk, const FMass<N> &F, float hf, const double (&x)[N][3],
                                             const double (&v)[N][3], double (&a0)[N][3], float (&da)[N][3],
@@ -715,7 +720,10 @@ __device__ __forceinline__ int spl_ff_state(const F64k &kk, const FMass<N> &F, f
   for (int k = 1; k < N; k++)
 #pragma unroll
     for (int c = 0; c < 3; c++) V[k][c] = ff_from(v[k][c]);
-  const int level = spl_eval_full<N, kGuard | (STAR ? kStar : 0)>(kk, F, hf, x, V, R, g);
+  int level = spl_eval_full<N, kGuard | (STAR ? kStar : 0)>(kk, F, hf, x, V, R, g);
+#pragma unroll
+  for (int k = 1; k < N; k++)
+    if (!ff_tame(x[k], v[k])) level = 0;
 #pragma unroll
   for (int k = 1; k < N; k++) {
     q2[k] = R.q2[k];
@@ -756,7 +764,7 @@ static __device__ __noinline__ int spl_hermite_ff_step_call(const F64k &kk, cons
 }
 
 // The monitor (Algorithm 1) after a step in pairs to a state of the given level.  A state of
-// level 1 or 2 is finite, and its tests start from the FP32 distances (kcf = 2 kc, ejf = the
+// level 1 or 2 is finite (`spl_ff_state`), and its tests start from the FP32 distances (kcf = 2 kc, ejf = the
 // squared ejection radius, both moved 2^-9 to the safe side); what comes near a limit, and
 // any state of level 0, is tested in FP64.
 template <int N>

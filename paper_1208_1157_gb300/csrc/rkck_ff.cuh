@@ -144,7 +144,7 @@ __device__ __forceinline__ void spl_acc_full(const F64k &kk, const FMass<N> &F, 
         }
       const float a = f_from(v[k][0]), b = f_from(v[k][1]), c = f_from(v[k][2]);
       const float V2 = __fmaf_rn(c, c, __fmaf_rn(b, b, __fmul_rn(a, a)));
-      R.range = R.range && frange(R.q2[k]) && V2 < 0x1p80f && V2 > 0x1p-80f;
+      R.range = R.range && ff_tame(X[k], v[k]) && frange(R.q2[k]) && V2 < 0x1p80f && V2 > 0x1p-80f;
       R.e1 = fmaxf(R.e1, F.muf[k].h * g.s[0][k]);
       R.sv = fmaxf(R.sv, S * S / V2);
     }
@@ -578,7 +578,7 @@ struct BplAcc {
   double M, dX[3];
   ff P[3];
   float q2, e1, sv;
-  bool range, near;
+  bool tame, range, near;  // tame: this lane's x and v (body 0's too)
 };
 // Acceleration -M dX + P of the lane's body (bpl_eval_ff without the jerks).  FULL: body 0's pull
 // in FP64 from x; else everything from the pairs xf, the acceleration in P.
@@ -612,6 +612,7 @@ __device__ __forceinline__ void bpl_acc_ff(const F64k &k, const BplBody<N> &g, c
   float S = 0.0f;
   if (STATE) {
     R.near = false;
+    R.tame = ff_tame(x, v);
     R.range = frange(R.q2);
   }
 #pragma unroll kRingUnroll<N>
@@ -917,8 +918,8 @@ __device__ __forceinline__ void bpl_rkck_stream(const BinView &B, const StepPara
         }
         e1 = A.e1;
         sv = A.sv;
-        range = scaled && (b == 0 || A.range);
-        near = b != 0 && (!A.range || A.near || !(A.q2 < ejf));
+        range = scaled && A.tame && (b == 0 || A.range);
+        near = !A.tame || (b != 0 && (!A.range || A.near || !(A.q2 < ejf)));
       }
     }
     const bool moved = has && fresh && steps > 0;  // a step led here
@@ -957,7 +958,7 @@ __device__ __forceinline__ void bpl_rkck_stream(const BinView &B, const StepPara
         last = f_from(h) >= 0.999f * f_from(rem) && h >= rem;
         hs = kmul(P.fk, last ? rem : h, dir);
       }
-      const bool mine = b == 0 ? scaled : (range && rk_guard(fabsf(f_from(hs)), e1, sv));
+      const bool mine = b == 0 ? range : (range && rk_guard(fabsf(f_from(hs)), e1, sv));
       bool pairs = (__ballot_sync(FULL, !mine) & gm) == 0 && (!ADAPT || eps_ok);
       double x5[3], v5[3];
       ff err = ff_make(0.0f, 0.0f);  // squared scaled error of the trial
