@@ -609,7 +609,10 @@ __device__ __forceinline__ void bpl_acc_ff(const F64k &k, const BplBody<N> &g, c
     T[c] = ff_mul_raw(rho3, X[c]);
     R.P[c] = ff_make(0.0f, 0.0f);
   }
-  float S = 0.0f;
+  // S begins with body 0's answer to this body, which is in pairs as well (its lane's sum, 2^-46
+  // of it): allowed 1/160 of the relative velocity in a step.  Masses (1e-3, 1), 60 to 130 steps
+  // an orbit, without it: 1.5 to 2.9 times the FP64 steps' error; (1, 1), 470 steps: 0.83.
+  float S = STATE ? 0.625f * g.mf.h * rho2.h : 0.0f;
   if (STATE) {
     R.near = false;
     R.tame = ff_tame(x, v);
@@ -661,7 +664,7 @@ __device__ __forceinline__ void bpl_acc_ff(const F64k &k, const BplBody<N> &g, c
     }
     const float V2 = __fmaf_rn(V[2], V[2], __fmaf_rn(V[1], V[1], __fmul_rn(V[0], V[0])));
     R.range = R.range && V2 < 0x1p80f && V2 > 0x1p-80f;
-    R.e1 = g.m0f.h * rho3.h;
+    R.e1 = (g.m0f.h + g.mf.h) * rho3.h;  // of the relative orbit: body 0 need not be the heavy one
     R.sv = __fmul_rn(S, S) / V2;
   }
 }
