@@ -105,6 +105,22 @@ __device__ __forceinline__ float f_from(double d) {
   return __int_as_float((__funnelshift_l(__double2loint(d), e, 3) & 0x7fffffff) | (hi & 0x80000000));
 }
 
+// a double's 53 bits as three floats
+struct ff3 {
+  float h, l, t;
+};
+__device__ __forceinline__ ff3 ff3_from(double d) {
+  const int hi = __double2hiint(d), lo = __double2loint(d);
+  const int e = max((hi & 0x7fffffff) - (896 << 20), 0);
+  ff3 r;
+  const int top = (__funnelshift_l(lo, e, 3) & 0x7fffffff) | (hi & 0x80000000);
+  const float sc = __int_as_float(top & 0xff800000);
+  r.h = __int_as_float(top);
+  r.l = __fmul_rn(__fmul_rn(__int2float_rn(lo & 0x1fffffe0), 0x1p-52f), sc);
+  r.t = __fmul_rn(__fmul_rn(__int2float_rn(lo & 31), 0x1p-52f), sc);
+  return r;
+}
+
 // Whether every value is below 2^64 in size, and neither NaN nor infinite (exponent bits, integer
 // pipe).  NaN, infinity and what is beyond 2^128 come out of the conversions above as ordinary
 // numbers (the exponent's upper bits are dropped), so a test of those does not see them.

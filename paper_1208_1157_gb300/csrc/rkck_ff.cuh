@@ -26,6 +26,7 @@ __device__ __forceinline__ ff ff_lin(double c, const ff &a, const ff &s) { retur
 struct RkStep {
   double h, hc3, hc4, hc6;
   ff f, h2;
+  float fl;  // what f leaves of h
 };
 __device__ __forceinline__ RkStep rk_step(const F64k &k, double h) {
   RkStep R;
@@ -33,24 +34,33 @@ __device__ __forceinline__ RkStep rk_step(const F64k &k, double h) {
   R.hc3 = kmul(k, CKN::C3, h);
   R.hc4 = kmul(k, CKN::C4, h);
   R.hc6 = kmul(k, CKN::C6, h);
-  R.f = ff_norm(ff_from(h));
+  const ff3 h3 = ff3_from(h);
+  R.f = ff_norm(ff_make(h3.h, h3.l));
+  R.fl = h3.t;
   R.h2 = ff_mul(R.f, R.f);
   return R;
 }
+// h times a pair.  The third part of h (up to 2^-48 of it) is the same at every fixed step, and left
+// out it adds up like a change of the step's length: at 60 steps an orbit, where h is such a number,
+// 200 steps of two bodies ended 6.2e-14 from quadruple precision instead of FP64's 3.2e-14.
+__device__ __forceinline__ ff rk_hmul(const RkStep &R, const ff &a) {
+  const ff p = ff_mul_raw(R.f, a);
+  return ff_norm(ff_make(p.h, __fmaf_rn(R.fl, a.h, p.l)));
+}
 // Per component, from a = a_1 and the D_j: what a stage adds to v in x_i = x + c_i h (v + w_i)
 // and the result in x5 = x + h (v + w): one rounding of x, and v + w's is taken by c_i h.
-__device__ __forceinline__ ff rk_w3(const RkStep &R, const ff &a) { return ff_norm(ff_mul_raw(R.f, ff_lin(0.5 * CKN::C3, a))); }
+__device__ __forceinline__ ff rk_w3(const RkStep &R, const ff &a) { return rk_hmul(R, ff_lin(0.5 * CKN::C3, a)); }
 __device__ __forceinline__ ff rk_w4(const RkStep &R, const ff &a, const ff &d2) {
-  return ff_norm(ff_mul_raw(R.f, ff_lin(CKN::A42 / CKN::C4, d2, ff_lin(0.5 * CKN::C4, a))));
+  return rk_hmul(R, ff_lin(CKN::A42 / CKN::C4, d2, ff_lin(0.5 * CKN::C4, a)));
 }
 __device__ __forceinline__ ff rk_w5(const RkStep &R, const ff &a, const ff &d2, const ff &d3) {
-  return ff_norm(ff_mul_raw(R.f, ff_lin(CKN::A53, d3, ff_lin(CKN::A52, d2, ff_lin(0.5, a)))));
+  return rk_hmul(R, ff_lin(CKN::A53, d3, ff_lin(CKN::A52, d2, ff_lin(0.5, a))));
 }
 __device__ __forceinline__ ff rk_w6(const RkStep &R, const ff &a, const ff &d2, const ff &d3, const ff &d4) {
-  return ff_norm(ff_mul_raw(R.f, ff_lin(CKN::A64 / CKN::C6, d4, ff_lin(CKN::A63 / CKN::C6, d3, ff_lin(CKN::A62 / CKN::C6, d2, ff_lin(0.5 * CKN::C6, a))))));
+  return rk_hmul(R, ff_lin(CKN::A64 / CKN::C6, d4, ff_lin(CKN::A63 / CKN::C6, d3, ff_lin(CKN::A62 / CKN::C6, d2, ff_lin(0.5 * CKN::C6, a)))));
 }
 __device__ __forceinline__ ff rk_wx(const RkStep &R, const ff &a, const ff &d3, const ff &d4, const ff &d5) {
-  return ff_norm(ff_mul_raw(R.f, ff_lin(CKN::B5, d5, ff_lin(CKN::B4, d4, ff_lin(CKN::B3, d3, ff_lin(0.5, a))))));
+  return rk_hmul(R, ff_lin(CKN::B5, d5, ff_lin(CKN::B4, d4, ff_lin(CKN::B3, d3, ff_lin(0.5, a)))));
 }
 // and v5 = v + h (S1 + this)
 __device__ __forceinline__ ff rk_av(const ff &p1, const ff &d3, const ff &d4, const ff &d6) {
