@@ -74,9 +74,9 @@ __device__ __forceinline__ ff rk_ev(const RkStep &R, const ff &d3, const ff &d4,
 }
 
 // e1 = mu/r^3 and sv = (S/v)^2 (see fguard) of a state, largest over its planets; h the step
-__device__ __forceinline__ bool rk_guard(float hf, float e1, float sv) {
-  const float h2 = hf * hf;
-  return h2 * e1 <= 0x1p-6f && h2 * sv <= 0x1p-16f && hf > 0x1p-40f;
+__device__ __forceinline__ bool rk_guard(double h, float e1, float sv) {
+  const float hf = f_from(h), h2 = hf * hf;
+  return h2 * e1 <= 0x1p-6f && h2 * sv <= 0x1p-16f && fscale(h, -40, 60);
 }
 // max of two non-negative pairs
 __device__ __forceinline__ ff ff_max(const ff &a, const ff &b) {
@@ -499,11 +499,11 @@ __device__ __forceinline__ void spl_rkck_stream(const BinView &B, const StepPara
         hs = (last && !plan.exact) ? plan.h_last : P.dt;
       } else {
         const double rem = kmul(P.fk, ksub(P.fk, te, t), dir);
-        last = f_from(h) >= 0.999f * f_from(rem) && h >= rem;
+        last = __double2hiint(h) >= __double2hiint(rem) && h >= rem;  // (FP64 compares are slow)
         hs = kmul(P.fk, last ? rem : h, dir);
       }
       double x5[N][3], v5[N][3];
-      bool accept = true, pairs = range && rk_guard(fabsf(f_from(hs)), e1, sv) && (!ADAPT || eps_ok);
+      bool accept = true, pairs = range && rk_guard(hs, e1, sv) && (!ADAPT || eps_ok);
       ff err = ff_make(0.0f, 0.0f);  // squared scaled error of the trial
       double err64 = 0.0;
       if (pairs) {
@@ -968,10 +968,10 @@ __device__ __forceinline__ void bpl_rkck_stream(const BinView &B, const StepPara
         hs = (last && !plan.exact) ? plan.h_last : P.dt;
       } else {
         const double rem = kmul(P.fk, ksub(P.fk, te, t), dir);
-        last = f_from(h) >= 0.999f * f_from(rem) && h >= rem;
+        last = __double2hiint(h) >= __double2hiint(rem) && h >= rem;  // (FP64 compares are slow)
         hs = kmul(P.fk, last ? rem : h, dir);
       }
-      const bool mine = b == 0 ? range : (range && rk_guard(fabsf(f_from(hs)), e1, sv));
+      const bool mine = b == 0 ? range : (range && rk_guard(hs, e1, sv));
       bool pairs = (__ballot_sync(FULL, !mine) & gm) == 0 && (!ADAPT || eps_ok);
       double x5[3], v5[3];
       ff err = ff_make(0.0f, 0.0f);  // squared scaled error of the trial
