@@ -512,7 +512,7 @@ __device__ __forceinline__ void bpl_hermite_run(const BinView &B, const StepPara
       A[c] = ff_from(an[c]);
       A[c] = ff_norm(ff_make(A[c].h, A[c].l + dn[c]));
     }
-    const ff sum = shfl_ff(grp_sum_ff<N>(g, ff_div(ff_norm2(J), ff_norm2(A))), g.base);
+    const ff sum = shfl_ff(grp_sum_ff<N>(g, ff_eq5_term(A, J)), g.base);
     return ff_mul(tau, ff_rsqrt(sum));
   };
 
@@ -790,7 +790,7 @@ __device__ __forceinline__ void bpl_hermite_run(const BinView &B, const StepPara
           const ff hs = eq5(aE, dA, J);
           if (kind == 2) {
             hn = hs;
-            if (!(hs.h <= hf)) lv = 0;
+            if (!(hs.h > 0.0f && hs.h <= hf)) lv = 0;
           }
         }
       } else if (mine) {

@@ -855,6 +855,23 @@ __device__ __forceinline__ ff ff_rsqrt(const ff &a) {
   const float t = __fsub_rn(__fsub_rn(1.0f, p.h), p.l);
   return fast_two_sum(y, __fmul_rn(__fmul_rn(0.5f, y), __fmaf_rn(0.75f, __fmul_rn(t, t), t)));
 }
+// |j|^2/|a|^2 of a body.  Body 0's vectors have the planets' masses, whose squares (and their lower
+// words first) leave FP32's range: both vectors are taken times the power of two that brings a to
+// 1, which is exact.  NaN, which sends the step to FP64, for a body whose own components are so
+// small that they have lost bits.
+__device__ __forceinline__ ff ff_eq5_term(const ff (&a)[3], const ff (&j)[3]) {
+  const float A = fmaxf(fmaxf(fabsf(a[0].h), fabsf(a[1].h)), fabsf(a[2].h));
+  const float J = fmaxf(fmaxf(fabsf(j[0].h), fabsf(j[1].h)), fabsf(j[2].h));
+  const float s = __int_as_float(0x7f000000 - (__float_as_int(A) & 0x7f800000));
+  ff as[3], js[3];
+#pragma unroll
+  for (int c = 0; c < 3; c++) {
+    as[c] = ff_make(s * a[c].h, s * a[c].l);
+    js[c] = ff_make(s * j[c].h, s * j[c].l);
+  }
+  const ff r = ff_div(ff_norm2(js), ff_norm2(as));
+  return A > 0x1p-100f && J > 0x1p-100f ? r : ff_make(__int_as_float(0x7fffffff), 0.0f);
+}
 // Eq. 5's step tau (sum_i |j_i|^2/|a_i|^2)^(-1/2) over the inertial accelerations and jerks, in
 // pairs (relative error 2^-44: the step's length, not the state, takes it).
 template <int N>
@@ -866,7 +883,7 @@ __device__ __forceinline__ ff spl_ff_eq5(const ff &tau, const double (&a0)[N][3]
     a[c] = ff_norm(sa[c]);
     j[c] = ff_norm(sj[c]);
   }
-  ff sum = ff_div(ff_norm2(j), ff_norm2(a));
+  ff sum = ff_eq5_term(a, j);
 #pragma unroll
   for (int k = 1; k < N; k++) {
 #pragma unroll
@@ -875,7 +892,7 @@ __device__ __forceinline__ ff spl_ff_eq5(const ff &tau, const double (&a0)[N][3]
       a[c] = ff_add(ff_make(A.h, A.l + da[k][c]), sa[c]);
       j[c] = ff_add(j0[k][c], sj[c]);
     }
-    sum = ff_add(sum, ff_div(ff_norm2(j), ff_norm2(a)));
+    sum = ff_add(sum, ff_eq5_term(a, j));
   }
   return ff_mul(tau, ff_rsqrt(sum));
 }
