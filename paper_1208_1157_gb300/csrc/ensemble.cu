@@ -932,8 +932,10 @@ static int integrate_impl(swarm_ensemble *e, double t_end, int integrator, doubl
   if (integrator < SWARM_HERMITE4 || integrator > SWARM_RKCK_ADAPTIVE)
     return fail(SWARM_EINVAL, "unknown integrator %d", integrator);
   if (!(dt != 0.0) || !std::isfinite(dt) || !std::isfinite(t_end)) return fail(SWARM_EINVAL, "dt must be finite and non-zero, t_end finite");
+  // (a call through observation times is planned interval by interval, and its caller has looked
+  // at every one's span)
   double span = std::max(std::fabs(t_end - e->t_lo), std::fabs(t_end - e->t_hi)) / std::fabs(dt);
-  if (!adaptive(integrator) && !(span <= kMaxCallSteps)) return fail(SWARM_EINVAL, "more than 2e9 steps in one call");
+  if (!obs && !adaptive(integrator) && !(span <= kMaxCallSteps)) return fail(SWARM_EINVAL, "more than 2e9 steps in one call");
   if (e->mapping == SWARM_MAP_PLAIN_PER_STEP && (integrator != SWARM_HERMITE4 || e->corr_form))
     return fail(SWARM_EINVAL, "the plain per-step baseline exists for the fixed-step time-symmetric Hermite only");
   StepParams P = make_params(e, t_end, integrator, dt);
