@@ -458,7 +458,7 @@ static int admit(swarm_server *sv) {
     std::vector<double>().swap(r->mass);
     it = sv->queue.erase(it);
   }
-  return flush(false);  // (step() waits for the stream before it writes them again)
+  return flush(false);  // (the round waits for the stream before they are written again)
 }
 
 // Retirement, system by system: the round has left the statuses of every occupied pool in
@@ -553,9 +553,7 @@ static int retire(swarm_server *sv, int32_t *n_completed) {
   return flush();
 }
 
-extern "C" int swarm_server_step(swarm_server *sv, int32_t *n_completed) {
-  if (!sv || !n_completed) return sfail(SWARM_EINVAL, "NULL argument");
-  *n_completed = 0;
+static int scheduling_round(swarm_server *sv, int32_t *n_completed) {
   int rc = admit(sv);
   if (rc) return rc;
   bool ran = false;
@@ -660,6 +658,19 @@ extern "C" int swarm_server_step(swarm_server *sv, int32_t *n_completed) {
     sv->stats.quanta++;
   }
   return retire(sv, n_completed);
+}
+
+extern "C" int swarm_server_step(swarm_server *sv, int32_t *n_completed) {
+  if (!sv || !n_completed) return sfail(SWARM_EINVAL, "NULL argument");
+  *n_completed = 0;
+  const int rc = scheduling_round(sv, n_completed);
+  // A round ends with a wait.  One that failed on the way has not waited for its copies out of the
+  // pinned staging and list buffers, which the next round writes.
+  if (rc) {
+    cudaStreamSynchronize(sv->stream);
+    for (cudaStream_t st : sv->side) cudaStreamSynchronize(st);
+  }
+  return rc;
 }
 
 extern "C" int swarm_server_poll(swarm_server *sv, int64_t id, int32_t *state, double *pos, double *vel,
