@@ -574,24 +574,27 @@ __device__ __forceinline__ void bpl_hermite_run(const BinView &B, const StepPara
       const bool tm = (__ballot_sync(FULL, !ff_tame(x, v)) & gm) == 0;
       if (got) tame = tm;
       const bool sc2 = scaled && tame;
-      BplEval<N> E;
-      double an[3], jn[3];
-      ff V[3];
-#pragma unroll
-      for (int c = 0; c < 3; c++) V[c] = ff_norm(ff_from(v[c]));
-      bpl_eval_ff_call<N>(P.fk, g, x, V, kcf, E);
-#pragma unroll
-      for (int c = 0; c < 3; c++) {
-        an[c] = fma(-E.M, E.dX[c], ff_double(E.P[c]));
-        jn[c] = to_bits(E.J[c]);
-      }
-      float hf = P.fc.hf, zero[3] = {0.0f, 0.0f, 0.0f};
+      double an[3] = {0.0, 0.0, 0.0}, jn[3] = {0.0, 0.0, 0.0};
       ff hn = h;
-      if (ADAPT) {
-        hn = eq5(an, zero, E.J);
-        hf = hn.h;
+      int lv = 0;
+      if (!printed) {
+        BplEval<N> E;
+        ff V[3];
+#pragma unroll
+        for (int c = 0; c < 3; c++) V[c] = ff_norm(ff_from(v[c]));
+        bpl_eval_ff_call<N>(P.fk, g, x, V, kcf, E);
+#pragma unroll
+        for (int c = 0; c < 3; c++) {
+          an[c] = fma(-E.M, E.dX[c], ff_double(E.P[c]));
+          jn[c] = to_bits(E.J[c]);
+        }
+        float hf = P.fc.hf, zero[3] = {0.0f, 0.0f, 0.0f};
+        if (ADAPT) {
+          hn = eq5(an, zero, E.J);
+          hf = hn.h;
+        }
+        lv = bpl_level<N>(g, E, hf, sc2 && hf > 0.0f);
       }
-      const int lv = bpl_level<N>(g, E, hf, sc2 && hf > 0.0f && !printed);
       if (__any_sync(FULL, got && !lv)) {
         double a_[3], j_[3], q_;
         bpl_fp64_eval<N>(P.fk, x, v, m, g, a_, j_, q_, rd);
@@ -703,14 +706,16 @@ __device__ __forceinline__ void bpl_hermite_run(const BinView &B, const StepPara
     }
     // Level 2: phase 0 evaluates the prediction and corrects it (spl_hermite_delta_step); then,
     // for every group or (carry) those of the other kinds, phase 1 evaluates the new state.
-    // One copy of the evaluation serves both phases (instruction cache).
+    // One copy of the evaluation serves both phases (instruction cache).  Not for a warp none of whose
+    // systems the pairs could hold, nor for the printed corrector, whose steps are FP64.
+    const bool look = !printed && __any_sync(FULL, alive && scaled && tame);
     double an[3], jn[3];
     float dn[3] = {0.0f, 0.0f, 0.0f};
     int lv = 0;
     bool near = true;
     ff hn = h;
 #pragma unroll 1
-    for (int phase = any2 ? 0 : 1; phase < (rest || !carry ? 2 : 1); phase++) {
+    for (int phase = any2 ? 0 : 1; phase < (look ? rest || !carry ? 2 : 1 : 0); phase++) {
       BplEval<N> E;
       ff G[3], W[3], V[3];
       double xe[3];
@@ -738,7 +743,7 @@ __device__ __forceinline__ void bpl_hermite_run(const BinView &B, const StepPara
         if (mine) hn = hs;
         hf = hs.h;
       }
-      const int lE = bpl_level<N>(g, E, hf, scaled && tame && hf > 0.0f && !printed);
+      const int lE = bpl_level<N>(g, E, hf, scaled && tame && hf > 0.0f);
       if (mine) {
         lv = lE;
         near = !lE || (b != 0 && (E.near || !(E.q2 < ejf)));
