@@ -241,18 +241,22 @@ __device__ __forceinline__ void bpl_eval_ff(const F64k &k, const BplBody<N> &g, 
 // The group's level (the least of its planets') for steps of length hf.  Body 0's answer to a
 // planet is formed in pairs by its own lane (2^-46 of it: `BplBody::mt` and `star_pull` keep it
 // from the biases that the other sums may have), and may weigh up to 3/64 of the relative velocity
-// in a step.  Only with a body 0 much lighter than its companion does it weigh more, at 130 steps
+// in a step (at level 2 it cannot weigh that much).  Only with a body 0 much lighter than its companion does it weigh more, at 130 steps
 // an orbit and fewer (masses 0.03 and 1, 102 steps an orbit: 1.3 to 1.5 times the FP64 steps'
 // error without this limit; two equal ones 0.8).
 template <int N>
 __device__ __forceinline__ int bpl_level(const BplBody<N> &g, const BplEval<N> &R, float hf, bool ok) {
   int lv = 2;
-  const float w0 = hf * g.mf.h * R.p;
-  if (g.b != 0) lv = R.range && w0 * w0 <= 0x1.2p-9f * R.V2 ? fguard(hf, hf * hf * R.e1, R.S, R.V2) : 0;
+  if (g.b != 0) lv = R.range ? fguard(hf, hf * hf * R.e1, R.S, R.V2) : 0;
   if (!ok) lv = 0;
   const unsigned gm = g.mask();
-  const unsigned n0 = __ballot_sync(0xffffffffu, lv == 0) & gm, n1 = __ballot_sync(0xffffffffu, lv == 1) & gm;
-  return n0 ? 0 : n1 ? 1 : 2;
+  unsigned n0 = __ballot_sync(0xffffffffu, lv == 0);
+  const unsigned n1 = __ballot_sync(0xffffffffu, lv == 1);
+  if (n1) {
+    const float w0 = hf * g.mf.h * R.p;
+    n0 |= __ballot_sync(0xffffffffu, lv == 1 && !(w0 * w0 <= 0x1.2p-9f * R.V2));
+  }
+  return n0 & gm ? 0 : n1 & gm ? 1 : 2;
 }
 
 // change of the evaluation R when the bodies' positions and velocities move by dX, dV, in FP32
@@ -367,24 +371,23 @@ static __device__ __noinline__ void bpl_eval_ff_call(const F64k &k, const BplBod
 // ---------------------------------------------------------------- FP64 steps (guard not met)
 // Out of line; every lane of the warp takes part in the shuffles.  kc, d2: per round of the ring
 // over all n bodies, in registers' place (local memory) or, for N = 0, this lane's column of
-// shared memory.
+// shared memory.  q2: the lane's squared distance to body 0.
 template <int N>
 struct BplRounds {
   static constexpr int RT = Ring<N>::RT > 0 ? Ring<N>::RT : 1;
-  double kc[RT], d2[RT];
+  double kc[RT], d2[RT], q2;
   __device__ __forceinline__ double &kcr(int r) { return kc[r - 1]; }
   __device__ __forceinline__ double &d2r(int r) { return d2[r - 1]; }
 };
 template <>
 struct BplRounds<0> {
-  double *kc, *d2;
+  double *kc, *d2, q2;
   __device__ __forceinline__ double &kcr(int r) { return kc[(r - 1) * 32]; }
   __device__ __forceinline__ double &d2r(int r) { return d2[(r - 1) * 32]; }
 };
 template <int N>
 static __device__ __noinline__ void bpl_fp64_eval(const F64k &k, const double (&x)[3], const double (&v)[3], double m,
-                                                  const BplBody<N> &g, double (&a)[3], double (&j)[3], double &q2,
-                                                  BplRounds<N> &rd) {
+                                                  const BplBody<N> &g, double (&a)[3], double (&j)[3], BplRounds<N> &rd) {
   double a_[3], j_[3], q_;
   if constexpr (N == 0) {
     wring_accjerk<true, 1>(k, x, v, m, g.b, wide_ring(g.nn), a_, j_, q_, rd.d2, 0);
@@ -396,7 +399,7 @@ static __device__ __noinline__ void bpl_fp64_eval(const F64k &k, const double (&
     a[c] = a_[c];
     j[c] = j_[c];
   }
-  q2 = q_;
+  rd.q2 = q_;
 }
 template <int N>
 static __device__ __noinline__ void bpl_fp64_advance(const F64k &k, double h, int n_corr, bool printed, double m,
@@ -404,7 +407,7 @@ static __device__ __noinline__ void bpl_fp64_advance(const F64k &k, double h, in
                                                      const double (&j0)[3], double (&x)[3], double (&v)[3],
                                                      BplRounds<N> &rd) {
   const HCoef C = hcoef(h);
-  double xk[3], vk[3], Xb[3], Vb[3], q2;
+  double xk[3], vk[3], Xb[3], Vb[3];
   // Eq. 3 predictor and the step-invariant parts of the corrector
 #pragma unroll
   for (int c = 0; c < 3; c++) {
@@ -424,7 +427,7 @@ static __device__ __noinline__ void bpl_fp64_advance(const F64k &k, double h, in
 #pragma unroll 1
   for (int ic = 0; ic < n_corr; ic++) {
     double ak[3], jk[3];
-    bpl_fp64_eval<N>(k, xk, vk, m, g, ak, jk, q2, rd);
+    bpl_fp64_eval<N>(k, xk, vk, m, g, ak, jk, rd);
 #pragma unroll
     for (int c = 0; c < 3; c++) vk[c] = fma(-C.h2_12, jk[c], fma(C.hh, ak[c], Vb[c]));
     if (printed) {
@@ -480,9 +483,9 @@ __device__ __forceinline__ void bpl_hermite_run(const BinView &B, const StepPara
   const float ejf = P.eject2 > 0.0 ? 0.998f * (float)P.eject2 : __int_as_float(0x7f800000);
 
   int s = 0, steps = 0, level = 0;
-  // tame: the state the group began with, or its last FP64 step led to, is one that the pairs can
-  // hold (`spl_ff_state` says why the other steps keep it one)
-  bool has = false, exhausted = false, scaled = false, tame = false;
+  // fit: scaled, and the state the group began with, or its last FP64 step led to, is one that the
+  // pairs can hold (`spl_ff_state` says why the other steps keep it one)
+  bool has = false, exhausted = false, scaled = false, fit = false;
   // the state's acceleration is a0 + da; j0: FP64, or (level > 0) the bits of a pair
   double x[3] = {0.0, 0.0, 0.0}, v[3] = {0.0, 0.0, 0.0}, m = 1.0, a0[3] = {0.0, 0.0, 0.0}, j0[3] = {0.0, 0.0, 0.0};
   float da[3] = {0.0f, 0.0f, 0.0f};
@@ -572,8 +575,7 @@ __device__ __forceinline__ void bpl_hermite_run(const BinView &B, const StepPara
         g.mt = (float)((m - (double)g.mf.h) - (double)g.mf.l);
       }
       const bool tm = (__ballot_sync(FULL, !ff_tame(x, v)) & gm) == 0;
-      if (got) tame = tm;
-      const bool sc2 = scaled && tame;
+      if (got) fit = scaled && tm;
       double an[3] = {0.0, 0.0, 0.0}, jn[3] = {0.0, 0.0, 0.0};
       ff hn = h;
       int lv = 0;
@@ -593,11 +595,11 @@ __device__ __forceinline__ void bpl_hermite_run(const BinView &B, const StepPara
           hn = eq5(an, zero, E.J);
           hf = hn.h;
         }
-        lv = bpl_level<N>(g, E, hf, sc2 && hf > 0.0f);
+        lv = bpl_level<N>(g, E, hf, fit && hf > 0.0f);
       }
       if (__any_sync(FULL, got && !lv)) {
-        double a_[3], j_[3], q_;
-        bpl_fp64_eval<N>(P.fk, x, v, m, g, a_, j_, q_, rd);
+        double a_[3], j_[3];
+        bpl_fp64_eval<N>(P.fk, x, v, m, g, a_, j_, rd);
         if (!lv)
 #pragma unroll
           for (int c = 0; c < 3; c++) {
@@ -668,6 +670,9 @@ __device__ __forceinline__ void bpl_hermite_run(const BinView &B, const StepPara
     const FCoef &C = ADAPT ? Cad : P.fc;
     const bool any2 = __any_sync(FULL, active && kind == 2);
     const bool rest = __any_sync(FULL, active && kind != 2);
+    double an[3], jn[3];
+    float dn[3] = {0.0f, 0.0f, 0.0f};
+    bool fp64 = false, clear = false;  // clear: beyond doubt of level 0
     if (rest) {  // groups of level 1, FP64 groups
       double xn[3], vn[3];
       if (__any_sync(FULL, active && kind == 1)) {
@@ -695,27 +700,43 @@ __device__ __forceinline__ void bpl_hermite_run(const BinView &B, const StepPara
         bpl_fp64_advance<N>(P.fk, hd, P.n_corr, printed, m, g, a0, j0, xn, vn, rd);
         const bool tm = (__ballot_sync(FULL, !ff_tame(xn, vn)) & gm) == 0;
         if (active && kind == 0) {
-          tame = tm;
+          fit = scaled && tm;
 #pragma unroll
           for (int c = 0; c < 3; c++) {
             x[c] = xn[c];
             v[c] = vn[c];
           }
         }
+        // The new state in FP64 first: where the step is too long for the pairs by 1 % (their guard's
+        // eta^2 is good to 2^-20) the look at it in pairs is saved.  (ADAPT: the next length is not
+        // known yet.)
+        double a_[3], j_[3];
+        bpl_fp64_eval<N>(P.fk, x, v, m, g, a_, j_, rd);
+        fp64 = true;
+        if (kind == 0)
+#pragma unroll
+          for (int c = 0; c < 3; c++) {
+            an[c] = a_[c];
+            jn[c] = j_[c];
+          }
+        if (!ADAPT) {
+          const float q = f_from(rd.q2), y = rsqrtf(q);
+          const float eta2 = P.fc.hf * P.fc.hf * (g.m0f.h + g.mf.h) * y * y * y;
+          clear = (__ballot_sync(FULL, b != 0 && eta2 > 1.01f * kFFEta2) & gm) != 0 && kind == 0;
+        }
       }
     }
     // Level 2: phase 0 evaluates the prediction and corrects it (spl_hermite_delta_step); then,
     // for every group or (carry) those of the other kinds, phase 1 evaluates the new state.
-    // One copy of the evaluation serves both phases (instruction cache).  Not for a warp none of whose
-    // systems the pairs could hold, nor for the printed corrector, whose steps are FP64.
-    const bool look = !printed && __any_sync(FULL, alive && scaled && tame);
-    double an[3], jn[3];
-    float dn[3] = {0.0f, 0.0f, 0.0f};
+    // One copy of the evaluation serves both phases (instruction cache).  Neither for a warp none of
+    // whose systems the pairs could take or hold, nor for the printed corrector, whose steps are FP64.
     int lv = 0;
     bool near = true;
     ff hn = h;
+    int phase = 0;
+    if (!any2) phase = !printed && __any_sync(FULL, alive && fit && !clear) ? 1 : 2;
 #pragma unroll 1
-    for (int phase = any2 ? 0 : 1; phase < (look ? rest || !carry ? 2 : 1 : 0); phase++) {
+    for (; phase < (rest || !carry ? 2 : 1); phase++) {
       BplEval<N> E;
       ff G[3], W[3], V[3];
       double xe[3];
@@ -743,7 +764,7 @@ __device__ __forceinline__ void bpl_hermite_run(const BinView &B, const StepPara
         if (mine) hn = hs;
         hf = hs.h;
       }
-      const int lE = bpl_level<N>(g, E, hf, scaled && tame && hf > 0.0f);
+      const int lE = bpl_level<N>(g, E, hf, fit && hf > 0.0f);
       if (mine) {
         lv = lE;
         near = !lE || (b != 0 && (E.near || !(E.q2 < ejf)));
@@ -798,7 +819,7 @@ __device__ __forceinline__ void bpl_hermite_run(const BinView &B, const StepPara
             if (!(hs.h > 0.0f && hs.h <= hf)) lv = 0;
           }
         }
-      } else if (mine) {
+      } else if (mine && (lE || kind)) {
 #pragma unroll
         for (int c = 0; c < 3; c++) {
           an[c] = aE[c];
@@ -809,17 +830,20 @@ __device__ __forceinline__ void bpl_hermite_run(const BinView &B, const StepPara
     if (carry && kind == 2 && !lv) near = true;
     int code = 0;
     if (__any_sync(FULL, alive && near)) {  // in FP64: a0, j0 of groups that need them, the exact tests
-      double a_[3], j_[3], q2;
-      bpl_fp64_eval<N>(P.fk, x, v, m, g, a_, j_, q2, rd);
-      if (!lv)
+      if (!fp64 || __any_sync(FULL, alive && near && kind != 0)) {
+        double a_[3], j_[3];
+        bpl_fp64_eval<N>(P.fk, x, v, m, g, a_, j_, rd);
+        if (!lv)
 #pragma unroll
-        for (int c = 0; c < 3; c++) {
-          an[c] = a_[c];
-          jn[c] = j_[c];
-          dn[c] = 0.0f;
-        }
+          for (int c = 0; c < 3; c++) {
+            an[c] = a_[c];
+            jn[c] = j_[c];
+            dn[c] = 0.0f;
+          }
+      }
       const bool nf = nonfinite(x[0]) | nonfinite(x[1]) | nonfinite(x[2]) | nonfinite(v[0]) | nonfinite(v[1]) |
                       nonfinite(v[2]);
+      const double q2 = rd.q2;
       const bool ej = (b != 0) && (P.eject2 > 0.0) && (q2 > P.eject2);
       bool ce = false;
       for (int r = 1; r <= rt; r++) {
