@@ -100,7 +100,17 @@ enum swarm_option {
                                     SWARM_OPT_STEPS_PER_LAUNCH set: from each launch's start) */
   SWARM_OPT_LOG_CAPACITY = 4,   /* records kept per system (ring of this size), 0..65536 */
   SWARM_OPT_STEPS_PER_LAUNCH = 5,/* 0 = whole call in one persistent launch; else launches of
-                                    this many steps, replayed from a captured CUDA graph */
+                                    this many steps, replayed from a captured CUDA graph.  A call
+                                    in launches, or continued by another call from the state that
+                                    the first one left, takes the same steps.  It repeats the
+                                    whole call bit for bit (steps of full length) with the
+                                    Runge-Kutta integrators from four bodies on and with fixed-
+                                    step Hermite, body per lane, in bins of fewer than 512 systems
+                                    of one body count; larger Hermite bins carry an evaluation from
+                                    step to step that the stored state does not hold, and a whole
+                                    system per lane and the mixed-variable integrators map the
+                                    state to other coordinates and back: there it agrees to
+                                    rounding */
   SWARM_OPT_SINGLE_LAUNCH = 6,  /* 0 (default): one single-bin launch per body count (registers
                                     sized for that n, systems handed out per group), the
                                     launches run concurrently on forked streams; 1: the bins
@@ -221,7 +231,8 @@ void swarm_destroy_ensemble(swarm_ensemble *ens);
  *     for the next admission at once; a request is DONE when its last system retires.
  * A system takes the same steps as it would alone (steps of dt, the last one shortened to
  * land on t_end), so results do not depend on the mix or on when each system was
- * admitted.  Stats: `admitted` counts requests with at least one system admitted,
+ * admitted; they agree with an ensemble's to rounding (pools are integrated quantum by
+ * quantum, see SWARM_OPT_STEPS_PER_LAUNCH, and a pool counts as large by its slots).  Stats: `admitted` counts requests with at least one system admitted,
  * `queued` requests with systems still waiting.  Not thread-safe: one thread drives a
  * server. */
 typedef struct swarm_server swarm_server;

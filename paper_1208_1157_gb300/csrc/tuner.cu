@@ -89,9 +89,9 @@ constexpr int kSplMinSystems = 8192;
 // 3x the SM count; a count above the kernel's residency runs at its residency); for the
 // Hermite step with n <= 4 also a whole system per lane at full residency and at 1 CTA
 // per SM, in bins that give every SM sub-partition a warp's worth of lanes to choose from
-// (kSplMinSystems); below that a step's latency decides, and body per lane has the property
-// that its steps follow from the stored state alone: a call in chunks, or resumed from a
-// checkpoint, repeats the uninterrupted one bit for bit.
+// (kSplMinSystems); below that a step's latency decides, and body per lane, below 512 systems
+// (kCarryMinSystems), has the property that its steps follow from the stored state alone: a call
+// in chunks, or resumed from a checkpoint, repeats the uninterrupted one bit for bit.
 void tuner_candidates(int n, int integrator, int S, std::vector<Choice> *out) {
   *out = {{SWARM_MAP_BODY_PER_LANE, 0}, {SWARM_MAP_BODY_PER_LANE, 1}, {SWARM_MAP_BODY_PER_LANE, 2},
           {SWARM_MAP_BODY_PER_LANE, 3}};

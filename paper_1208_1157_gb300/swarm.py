@@ -227,7 +227,10 @@ class Ensemble:
 
 def save_checkpoint(e: "Ensemble", path: str) -> None:
     """Write the ensemble's current state (masses, positions, velocities, times and
-    statuses) to an .npz file; `load_checkpoint` + `Ensemble.resume` continue from it."""
+    statuses) to an .npz file; `load_checkpoint` + `resume` continue from it.  Where a call in
+    several launches repeats the whole one bit for bit (include/swarm.h, SWARM_OPT_STEPS_PER_LAUNCH:
+    for Hermite bins of fewer than 512 systems), so does a resumed one; elsewhere it agrees to
+    rounding."""
     st = e.state()
     np.savez(path, n_body=e.n_body, mass=e._mass, pos=st["pos"], vel=st["vel"], time=st["time"], status=st["status"])
 
@@ -239,7 +242,7 @@ def load_checkpoint(path: str) -> dict:
 
 
 def resume(ckpt: dict, stream=None) -> "Ensemble":
-    """A new ensemble holding a checkpoint's state, times and statuses."""
+    """A new ensemble holding a checkpoint's state, times and statuses (see `save_checkpoint`)."""
     e = Ensemble(ckpt, stream=stream)
     e.set_state(time=ckpt["time"], status=ckpt["status"])
     return e
