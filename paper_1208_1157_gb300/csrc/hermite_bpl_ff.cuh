@@ -710,8 +710,8 @@ __device__ __forceinline__ void bpl_hermite_run(const BinView &B, const StepPara
           }
         }
         // The new state in FP64 first: where the step is too long for the pairs by 1 % (their guard's
-        // eta^2 is good to 2^-20) the look at it in pairs is saved.  (ADAPT: the next length is not
-        // known yet.)
+        // eta^2 is good to 2^-20), or the distance out of their range, the look at it in pairs is
+        // saved.  (ADAPT: the next length is not known yet.)
         double a_[3], j_[3];
         bpl_fp64_eval<N>(P.fk, x, v, m, g, a_, j_, rd);
         fp64 = true;
@@ -721,11 +721,10 @@ __device__ __forceinline__ void bpl_hermite_run(const BinView &B, const StepPara
             an[c] = a_[c];
             jn[c] = j_[c];
           }
-        if (!ADAPT) {
-          const float q = f_from(rd.q2), y = rsqrtf(q);
-          const float eta2 = P.fc.hf * P.fc.hf * (g.m0f.h + g.mf.h) * y * y * y;
-          clear = (__ballot_sync(FULL, b != 0 && eta2 > 1.01f * kFFEta2) & gm) != 0 && kind == 0;
-        }
+        const float q = f_from(rd.q2), y = rsqrtf(q);
+        const float eta2 = ADAPT ? 0.0f : P.fc.hf * P.fc.hf * (g.m0f.h + g.mf.h) * y * y * y;
+        const bool far = eta2 > 1.01f * kFFEta2 || q > 0x1.04p40f || q < 0x1.f8p-41f;
+        clear = (__ballot_sync(FULL, b != 0 && far) & gm) != 0 && kind == 0;
       }
     }
     // Level 2: phase 0 evaluates the prediction and corrects it (spl_hermite_delta_step); then,
