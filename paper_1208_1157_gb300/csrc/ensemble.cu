@@ -316,16 +316,18 @@ static void free_all(swarm_ensemble *e) {
 // One stream for every body count an ensemble can hold (2..32): two bins on one stream run one
 // after the other, and bins of a few hundred systems leave most of the chip to the others
 // (eight streams against one per bin: 777 systems of 3..15 bodies 3.37 -> 2.39 ms, 3001 mixed-
-// variable ones 5.08 -> 3.45, 2048 of 16..32 bodies 4.71 -> 3.69, 65536 18.3 -> 17.7).
+// variable ones 5.08 -> 3.45, 2048 of 16..32 bodies 4.71 -> 3.69, 65536 18.3 -> 17.7).  An
+// ensemble makes as many as its calls come to need.
 constexpr int kSideStreams = 32;
-static int ensure_side(swarm_ensemble *e) {
-  if (!e->side.empty()) return SWARM_OK;
-  CK(cudaEventCreateWithFlags(&e->fork_ev, cudaEventDisableTiming));
-  for (int i = 0; i < kSideStreams; i++) {
-    cudaStream_t st;
+static int ensure_side(swarm_ensemble *e, int count) {
+  if (count > 0 && !e->fork_ev) CK(cudaEventCreateWithFlags(&e->fork_ev, cudaEventDisableTiming));
+  while ((int)e->side_done.size() < count) {  // (a stream whose event failed is kept for the next call)
+    if (e->side.size() == e->side_done.size()) {
+      cudaStream_t st;
+      CK(cudaStreamCreateWithFlags(&st, cudaStreamNonBlocking));
+      e->side.push_back(st);
+    }
     cudaEvent_t ev;
-    CK(cudaStreamCreateWithFlags(&st, cudaStreamNonBlocking));
-    e->side.push_back(st);
     CK(cudaEventCreateWithFlags(&ev, cudaEventDisableTiming));
     e->side_done.push_back(ev);
   }
@@ -857,14 +859,14 @@ static int run_persistent(swarm_ensemble *e, const StepParams &P0, int integrato
   // forked from the main stream (heaviest bin first), so that one launch's tail overlaps
   // the next launch's work; all of them join the main stream before the round ends.
   const int nconc = (int)uni.size() + (per_bin ? 0 : 1);
-  if (nconc > 1 && (rc = ensure_side(e))) return rc;
+  const int nside = nconc > 1 ? std::min((int)uni.size(), kSideStreams) : 0;
+  if ((rc = ensure_side(e, nside))) return rc;
   auto enqueue = [&](cudaStream_t cs, const StepParams &Q) -> int {
-    const int K = nconc > 1 ? std::min((int)uni.size(), kSideStreams) : 0;
     // every launch's work counter (the shared launch's, then one per bin)
     CK(cudaMemsetAsync(e->d_work_next, 0, sizeof(int) * (1 + uni.size()), cs));
-    if (K) {
+    if (nside) {
       CK(cudaEventRecord(e->fork_ev, cs));
-      for (int j = 0; j < K; j++) CK(cudaStreamWaitEvent(e->side[j], e->fork_ev, 0));
+      for (int j = 0; j < nside; j++) CK(cudaStreamWaitEvent(e->side[j], e->fork_ev, 0));
     }
     if (!per_bin) {  // the shared launch stays on the main stream
       if (hermite_family(integrator)) CK(launch_hermite_persistent(e->d_bins, e->d_work, e->nwork, Q, grid, cs));
@@ -873,14 +875,14 @@ static int run_persistent(swarm_ensemble *e, const StepParams &P0, int integrato
     // single-bin launches (every bin, or only the wide bins next to the shared launch),
     // each with its own work counter after the shared launch's
     for (size_t i = 0; i < uni.size(); i++) {
-      cudaStream_t si = K ? e->side[i % K] : cs;
+      cudaStream_t si = nside ? e->side[i % nside] : cs;
       StepParams Qi = Q;
       Qi.work_next = e->d_work_next + 1 + i;
       if (compact) CK(live_list(uni[i].view, const_cast<int32_t *>(uni[i].view.list),
                                 const_cast<int *>(uni[i].view.nlist_dev), si));
       CK(launch_uni(uni[i], Qi, uni[i].grid, si, nullptr));
     }
-    for (int j = 0; j < K; j++) {
+    for (int j = 0; j < nside; j++) {
       CK(cudaEventRecord(e->side_done[j], e->side[j]));
       CK(cudaStreamWaitEvent(cs, e->side_done[j], 0));
     }
