@@ -203,15 +203,25 @@ __global__ void __launch_bounds__(kPackThreads) pack_kernel(BinView B, const int
   }
 }
 
-// The same for an ensemble of several bins in one launch, blockIdx.y the bin (13 bins one after
-// the other, a thread per system, its loads in turn: 777 systems of 3..15 bodies 113 us in, 223
-// us out; now 27 and 14; 65536 systems 253 and 227, now 137 and 38).  unpack: a thread per system and every eighth component, so that the SoA rows
-// are written 32 systems at a time; pack: a warp per system, so that the caller's rows are.
-__global__ void __launch_bounds__(256) unpack_bins_kernel(const BinView *__restrict__ bins, const int64_t *__restrict__ offs,
+// The same for several bins in one launch, blockIdx.y the bin (13 bins one after the other, a thread
+// per system, its loads in turn: 777 systems of 3..15 bodies 113 us in, 223 us out; now 27 and 14;
+// 65536 systems 253 and 227, now 137 and 38).  unpack: a thread per system and every eighth
+// component, so that the SoA rows are written 32 systems at a time; pack: a warp per system, so
+// that the caller's rows are.
+struct BinList {
+  int count = 0;
+  unsigned char at[SWARM_MAX_N];
+};
+// A bin that fills the chip by itself keeps the kernels above, which move more per instruction (two
+// bins of 3 and 4 bodies, us in and out, own launches / one launch: 4096 systems each 12 and 12 / 10
+// and 10, 16384 12 and 12 / 11 and 15, 65536 17 and 16 / 19 and 35, 262144 48 and 45 / 103 and 249;
+// of 8 and 9: 16384 17 and 31 / 14 and 18, 65536 33 and 56 / 42 and 76).
+static bool own_io_launch(const Bin &b) { return b.S >= (b.n <= kPackMaxN ? 16384 : 32768); }
+__global__ void __launch_bounds__(256) unpack_bins_kernel(const BinView *__restrict__ bins, BinList list, const int64_t *__restrict__ offs,
                                                           const double *__restrict__ pos, const double *__restrict__ vel,
                                                           const double *__restrict__ mass, const double *__restrict__ time,
                                                           const int32_t *__restrict__ status) {
-  const BinView B = bins[blockIdx.y];
+  const BinView B = bins[list.at[blockIdx.y]];
   const int s = blockIdx.x * 32 + (threadIdx.x & 31), n = B.n;
   if (s >= B.S) return;
   const int g = B.gidx[s];
@@ -227,10 +237,10 @@ __global__ void __launch_bounds__(256) unpack_bins_kernel(const BinView *__restr
   if (time) B.t[s] = time[g];
   if (status) B.status[s] = status[g];
 }
-__global__ void __launch_bounds__(256) pack_bins_kernel(const BinView *__restrict__ bins, const int64_t *__restrict__ offs,
+__global__ void __launch_bounds__(256) pack_bins_kernel(const BinView *__restrict__ bins, BinList list, const int64_t *__restrict__ offs,
                                                         double *__restrict__ pos, double *__restrict__ vel,
                                                         double *__restrict__ time, int32_t *__restrict__ status) {
-  const BinView B = bins[blockIdx.y];
+  const BinView B = bins[list.at[blockIdx.y]];
   const int s = blockIdx.x * 8 + (threadIdx.x >> 5), lane = threadIdx.x & 31, n = B.n;
   if (s >= B.S) return;
   const int g = B.gidx[s];
@@ -334,19 +344,38 @@ static int ensure_side(swarm_ensemble *e, int count) {
   return SWARM_OK;
 }
 
+// the ensemble's bins one by one (own(bin)) or, the small ones of several, in one launch
+// (shared(list, the most systems of one))
+template <class Own, class Shared>
+static int io_launches(const swarm_ensemble *e, Own own, Shared shared) {
+  BinList list;
+  int most = 0;
+  for (size_t i = 0; i < e->bins.size(); i++) {
+    const Bin &b = e->bins[i];
+    if (e->bins.size() == 1 || own_io_launch(b)) {
+      own(b);
+    } else {
+      list.at[list.count++] = (unsigned char)i;
+      most = std::max(most, b.S);
+    }
+  }
+  if (list.count) shared(list, most);
+  CK(cudaGetLastError());
+  return SWARM_OK;
+}
+
 // device arrays in the caller's layout into the bins
 static int unpack_from(const swarm_ensemble *e, const double *pos, const double *vel, const double *mass, const double *time,
                        const int32_t *status) {
-  int most = 0;
-  for (auto &b : e->bins) most = std::max(most, b.S);
-  if (e->bins.size() > 1) {
-    unpack_bins_kernel<<<dim3((most + 31) / 32, (unsigned)e->bins.size()), 256, 0, e->stream>>>(e->d_bins, e->d_offs, pos, vel,
-                                                                                               mass, time, status);
-  } else {
-    unpack_kernel<<<(most + 127) / 128, 128, 0, e->stream>>>(e->bins[0].view(), e->d_offs, pos, vel, mass, time, status);
-  }
-  CK(cudaGetLastError());
-  return SWARM_OK;
+  return io_launches(
+      e,
+      [&](const Bin &b) {
+        unpack_kernel<<<(b.S + 127) / 128, 128, 0, e->stream>>>(b.view(), e->d_offs, pos, vel, mass, time, status);
+      },
+      [&](const BinList &l, int most) {
+        unpack_bins_kernel<<<dim3((most + 31) / 32, (unsigned)l.count), 256, 0, e->stream>>>(e->d_bins, l, e->d_offs, pos, vel,
+                                                                                            mass, time, status);
+      });
 }
 
 static int upload_state(swarm_ensemble *e, const double *pos, const double *vel, const double *mass,
@@ -999,18 +1028,16 @@ extern "C" int swarm_set_state(swarm_ensemble *e, const double *pos, const doubl
 }
 
 static int pack_to(const swarm_ensemble *e, double *pos, double *vel, double *time, int32_t *status) {
-  if (e->bins.size() > 1) {
-    int most = 0;
-    for (auto &b : e->bins) most = std::max(most, b.S);
-    pack_bins_kernel<<<dim3((most + 7) / 8, (unsigned)e->bins.size()), 256, 0, e->stream>>>(e->d_bins, e->d_offs, pos, vel,
+  return io_launches(
+      e,
+      [&](const Bin &b) {
+        pack_kernel<<<(b.S + kPackThreads - 1) / kPackThreads, kPackThreads, 0, e->stream>>>(b.view(), e->d_offs, pos, vel,
                                                                                            time, status);
-  } else {
-    const Bin &b = e->bins[0];
-    pack_kernel<<<(b.S + kPackThreads - 1) / kPackThreads, kPackThreads, 0, e->stream>>>(b.view(), e->d_offs, pos, vel,
-                                                                                       time, status);
-  }
-  CK(cudaGetLastError());
-  return SWARM_OK;
+      },
+      [&](const BinList &l, int most) {
+        pack_bins_kernel<<<dim3((most + 7) / 8, (unsigned)l.count), 256, 0, e->stream>>>(e->d_bins, l, e->d_offs, pos, vel,
+                                                                                        time, status);
+      });
 }
 
 extern "C" int swarm_set_state_dev(swarm_ensemble *e, const double *d_pos, const double *d_vel, const double *d_time,
