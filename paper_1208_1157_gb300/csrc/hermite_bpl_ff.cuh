@@ -403,48 +403,149 @@ static __device__ __noinline__ void bpl_fp64_eval(const F64k &k, const double (&
   }
   rd.q2 = q_;
 }
+// Eq. 5's length in FP64 from a and j (every lane of the warp)
 template <int N>
-static __device__ __noinline__ void bpl_fp64_advance(const F64k &k, double h, int n_corr, bool printed, double m,
-                                                     const BplBody<N> &g, const double (&a0)[3],
-                                                     const double (&j0)[3], double (&x)[3], double (&v)[3],
-                                                     BplRounds<N> &rd) {
-  const HCoef C = hcoef(h);
-  double xk[3], vk[3], Xb[3], Vb[3];
-  // Eq. 3 predictor and the step-invariant parts of the corrector
+__device__ __forceinline__ double bpl_fp64_eq5(const StepParams &P, const BplBody<N> &g, bool lane_ok, const double (&a)[3],
+                                               const double (&j)[3]) {
+  const double ratio = (j[0] * j[0] + j[1] * j[1] + j[2] * j[2]) / (a[0] * a[0] + a[1] * a[1] + a[2] * a[2]);
+  double ssum;
+  if constexpr (N == 0) ssum = warp_sum(lane_ok ? ratio : 0.0);
+  else ssum = grp_sum<N>(ratio, g.b, g.base);
+  return fabs(P.dt) * rsqrt(ssum);
+}
+// the monitor's tests at a state evaluated into rd (every lane of the warp)
+template <int N>
+__device__ __forceinline__ void bpl_fp64_monitor(const StepParams &P, const BplBody<N> &g, const double (&x)[3],
+                                                 const double (&v)[3], BplRounds<N> &rd, bool &nf, bool &ej, bool &ce) {
+  const double q2 = rd.q2;
+  nf = nonfinite(x[0]) | nonfinite(x[1]) | nonfinite(x[2]) | nonfinite(v[0]) | nonfinite(v[1]) | nonfinite(v[2]);
+  ej = g.b != 0 && P.eject2 > 0.0 && q2 > P.eject2;
+  ce = false;
+  const int n = g.n();
+  for (int r = 1; r <= n / 2; r++) {
+    int p = g.b + r;
+    if (p >= n) p -= n;
+    const double q2p = shfl(q2, g.base + p);
+    const double kc = rd.kcr(r);
+    if (kc > 0.0 && close_encounter(P.fk, rd.d2r(r), kc, q2, q2p)) ce = true;
+  }
+}
+// Up to `count` steps in FP64 for the warp's groups of level 0 (`mine`), each from its state's a and j:
+// steps of hs, or (ADAPT) that one and then Eq. 5's.  Returns the steps taken, the same for every
+// group: before the count is full it ends at a state that a group has to look at, that the
+// monitor stops, or that needs no further step.  x, v, a, j and rd are then that state's, hs, ts and
+// last those of the step that led there, hnext (ADAPT) the next length.  clear: the state is
+// beyond doubt one for FP64, since a step is too long for the pairs by 1 % (their guard's eta^2
+// is good to 2^-20), a distance out of their range, or (free) all of them are.
+// In registers from step to step (200 steps of 0.02 orbits, 300 x 8 bodies: 4.5 ms with the evaluation and
+// the rest of the step out of line each, 4.0 so, 3.8 in a kernel wholly in FP64).
+template <int N, bool ADAPT>
+static __device__ __noinline__ int bpl_fp64_run(const StepParams &P, const BplBody<N> &g, bool lane_ok, double m, bool mine,
+                                                bool free, int count, BplRounds<N> &rd, double (&xs)[3], double (&vs)[3],
+                                                double (&as)[3], double (&js)[3], double &hs, double &ts, double te,
+                                                bool &last, double &hnext, bool &clear) {
+  const F64k &k = P.fk;
+  const unsigned FULL = 0xffffffffu, gm = g.mask();
+  const bool printed = P.corr_form != 0;
+  const double dir = P.dt > 0 ? 1.0 : -1.0;
+  double x[3], v[3], a0[3], j0[3], h = hs, t = ts;
 #pragma unroll
   for (int c = 0; c < 3; c++) {
-    xk[c] = fma(j0[c], C.h3_6, fma(a0[c], C.h2_2, fma(v[c], C.h, x[c])));
-    vk[c] = fma(j0[c], C.h2_2, fma(a0[c], C.h, v[c]));
-    Vb[c] = fma(j0[c], C.h2_12, fma(a0[c], C.hh, v[c]));
+    x[c] = xs[c];
+    v[c] = vs[c];
+    a0[c] = as[c];
+    j0[c] = js[c];
   }
-  PCoef PC;
-  if (printed) {
-    PC = pcoef(h);
+  HCoef C = hcoef(h);
+  int s = 0;
+  bool cl = false, la = last;
+  double hn = 0.0;
+  for (;;) {
+    double xk[3], vk[3], Xb[3], Vb[3], q2 = 0.0;
+    // Eq. 3 predictor and the step-invariant parts of the corrector
 #pragma unroll
-    for (int c = 0; c < 3; c++) Xb[c] = fma(j0[c], PC.pj, fma(a0[c], PC.pa, xk[c]));
-  } else {
-#pragma unroll
-    for (int c = 0; c < 3; c++) Xb[c] = fma(a0[c], C.h2_12, fma(v[c], C.hh, x[c]));
-  }
-#pragma unroll 1
-  for (int ic = 0; ic < n_corr; ic++) {
-    double ak[3], jk[3];
-    bpl_fp64_eval<N>(k, xk, vk, m, g, ak, jk, rd);
-#pragma unroll
-    for (int c = 0; c < 3; c++) vk[c] = fma(-C.h2_12, jk[c], fma(C.hh, ak[c], Vb[c]));
+    for (int c = 0; c < 3; c++) {
+      xk[c] = fma(j0[c], C.h3_6, fma(a0[c], C.h2_2, fma(v[c], C.h, x[c])));
+      vk[c] = fma(j0[c], C.h2_2, fma(a0[c], C.h, v[c]));
+      Vb[c] = fma(j0[c], C.h2_12, fma(a0[c], C.hh, v[c]));
+    }
+    PCoef PC;
     if (printed) {
+      PC = pcoef(h);
 #pragma unroll
-      for (int c = 0; c < 3; c++) xk[c] = fma(PC.cj, jk[c], fma(PC.ca, ak[c], Xb[c]));
+      for (int c = 0; c < 3; c++) Xb[c] = fma(j0[c], PC.pj, fma(a0[c], PC.pa, xk[c]));
     } else {
 #pragma unroll
-      for (int c = 0; c < 3; c++) xk[c] = fma(-C.h2_12, ak[c], fma(C.hh, vk[c], Xb[c]));
+      for (int c = 0; c < 3; c++) Xb[c] = fma(a0[c], C.h2_12, fma(v[c], C.hh, x[c]));
+    }
+#pragma unroll 1
+    for (int ic = 0;; ic++) {
+      if constexpr (N == 0) {
+        wring_accjerk<true, 1>(k, xk, vk, m, g.b, wide_ring(g.nn), a0, j0, q2, rd.d2, 0);
+      } else {
+        ring_accjerk<N, true, (N <= 8 ? Ring<N>::RF : 1)>(k, xk, vk, m, g.b, g.base, a0, j0, q2, rd.d2);
+      }
+      if (ic == P.n_corr) break;
+#pragma unroll
+      for (int c = 0; c < 3; c++) vk[c] = fma(-C.h2_12, j0[c], fma(C.hh, a0[c], Vb[c]));
+      if (printed) {
+#pragma unroll
+        for (int c = 0; c < 3; c++) xk[c] = fma(PC.cj, j0[c], fma(PC.ca, a0[c], Xb[c]));
+      } else {
+#pragma unroll
+        for (int c = 0; c < 3; c++) xk[c] = fma(-C.h2_12, a0[c], fma(C.hh, vk[c], Xb[c]));
+      }
+    }
+#pragma unroll
+    for (int c = 0; c < 3; c++) {
+      x[c] = xk[c];
+      v[c] = vk[c];
+    }
+    rd.q2 = q2;
+    s++;
+    float hf = P.fc.hf;
+    if (ADAPT) {
+      hn = bpl_fp64_eq5<N>(P, g, lane_ok, a0, j0);
+      hf = f_from(hn);
+    }
+    const float q = f_from(q2), y = rsqrtf(q);
+    const bool far = hf * hf * (g.m0f.h + g.mf.h) * y * y * y > 1.01f * kFFEta2 || q > 0x1.04p40f || q < 0x1.f8p-41f;
+    const unsigned fars = __ballot_sync(FULL, g.b != 0 && far);  // (every lane: not behind `free`)
+    cl = free || (fars & gm) != 0;
+    if (s >= count) break;
+    bool nf, ej, ce;
+    bpl_fp64_monitor<N>(P, g, x, v, rd, nf, ej, ce);
+    bool stop = nf || ej || ce || !cl;
+    double tn = t, hx = h;
+    bool ln = la;
+    if (ADAPT) {
+      tn = kadd(k, t, h);
+      const double rem = kmul(k, ksub(k, te, tn), dir);
+      ln = hn >= rem;
+      hx = kmul(k, ln ? rem : hn, dir);
+      stop = stop || la || !(hn > 0.0) || nonfinite(hn);
+    }
+    if (__any_sync(FULL, mine && stop)) break;
+    if (ADAPT) {
+      t = tn;
+      h = hx;
+      la = ln;
+      C = hcoef(h);
     }
   }
 #pragma unroll
   for (int c = 0; c < 3; c++) {
-    x[c] = xk[c];
-    v[c] = vk[c];
+    xs[c] = x[c];
+    vs[c] = v[c];
+    as[c] = a0[c];
+    js[c] = j0[c];
   }
+  hs = h;
+  ts = t;
+  last = la;
+  hnext = hn;
+  clear = cl;
+  return s;
 }
 
 // ---------------------------------------------------------------- the integration loop
@@ -501,6 +602,8 @@ __device__ __forceinline__ void bpl_hermite_run(const BinView &B, const StepPara
   plan.t_end = P.t_end;
   double t = 0.0, t0 = 0.0, te = 0.0;  // fixed steps: t is formed from t0 when needed
   ff h = ff_make(0.0f, 0.0f);          // ADAPT: length of the next step of a group in pairs
+  double h64 = 0.0;                    // and of a group in FP64, where it is known
+  bool known = false;
   g.m0 = 1.0;
   g.m0f = g.mf = ff_make(1.0f, 0.0f);
   g.mt = 0.0f;
@@ -618,6 +721,7 @@ __device__ __forceinline__ void bpl_hermite_run(const BinView &B, const StepPara
         }
         level = lv;
         h = hn;
+        known = false;
         t0 = t = B.t[s];
         steps = 0;
         const bool runnable = B.status[s] <= SWARM_SYS_DONE;
@@ -653,13 +757,10 @@ __device__ __forceinline__ void bpl_hermite_run(const BinView &B, const StepPara
         kind = 0;
       }
     } else {
-      double hs = ff_double(h);
-      if (__any_sync(FULL, alive && !kind)) {
-        const double ratio = (j0[0] * j0[0] + j0[1] * j0[1] + j0[2] * j0[2]) / (a0[0] * a0[0] + a0[1] * a0[1] + a0[2] * a0[2]);
-        double ssum;
-        if constexpr (N == 0) ssum = warp_sum(lane_ok ? ratio : 0.0);
-        else ssum = grp_sum<N>(ratio, b, g.base);
-        if (!kind) hs = fabs(P.dt) * rsqrt(ssum);
+      double hs = kind ? ff_double(h) : h64;
+      if (__any_sync(FULL, alive && !kind && !known)) {
+        const double e = bpl_fp64_eq5<N>(P, g, lane_ok, a0, j0);
+        if (!kind) hs = e;
       }
       const double rem = kmul(P.fk, ksub(P.fk, te, t), dir);
       last = hs >= rem;
@@ -674,10 +775,12 @@ __device__ __forceinline__ void bpl_hermite_run(const BinView &B, const StepPara
     const bool rest = __any_sync(FULL, active && kind != 2);
     double an[3], jn[3];
     float dn[3] = {0.0f, 0.0f, 0.0f};
-    bool fp64 = false, clear = false;  // clear: beyond doubt of level 0
-    if (rest) {  // groups of level 1, FP64 groups
+    int done = 1;
+    bool fp64 = false, clear = false;
+    if (rest) {  // groups of level 1, groups in FP64
       double xn[3], vn[3];
-      if (__any_sync(FULL, active && kind == 1)) {
+      const bool any1 = __any_sync(FULL, active && kind == 1);
+      if (any1) {
         ff jf[3];
 #pragma unroll
         for (int c = 0; c < 3; c++) {
@@ -693,38 +796,50 @@ __device__ __forceinline__ void bpl_hermite_run(const BinView &B, const StepPara
             v[c] = vn[c];
           }
       }
-      if (__any_sync(FULL, active && kind == 0)) {
+      if (__any_sync(FULL, active && kind == 0)) {  // several steps where no group of the warp is in pairs
+        const bool alone = !any1 && !any2;
+        int count = 1;
+        if (alone) {
+          int c = 1 << 30;
+          if (active) {
+            c = ADAPT ? cap - steps : max(1, (plan.exact ? plan.N : plan.N - 1) - steps);
+            if (P.log_interval > 0) c = min(c, P.log_interval - steps % P.log_interval);
+          }
+          count = __reduce_min_sync(FULL, c);
+        }
+        double a_[3], j_[3], hx = hd, tx = t, hn64;
+        bool lx = last, cl;
 #pragma unroll
         for (int c = 0; c < 3; c++) {
           xn[c] = x[c];
           vn[c] = v[c];
+          a_[c] = a0[c];
+          j_[c] = j0[c];
         }
-        bpl_fp64_advance<N>(P.fk, hd, P.n_corr, printed, m, g, a0, j0, xn, vn, rd);
+        done = bpl_fp64_run<N, ADAPT>(P, g, lane_ok, m, active && !kind, printed || !scaled, count, rd, xn, vn, a_, j_, hx, tx, te, lx,
+                                      hn64, cl);
+        fp64 = true;
         const bool tm = (__ballot_sync(FULL, !ff_tame(xn, vn)) & gm) == 0;
-        if (active && kind == 0) {
+        if (active && !kind) {
           fit = scaled && tm;
+          clear = cl;
+          if (ADAPT) {
+            hd = hx;
+            t = tx;
+            last = lx;
+            h64 = hn64;
+            known = true;
+          } else {
+            last = steps + done == plan.N;
+          }
 #pragma unroll
           for (int c = 0; c < 3; c++) {
             x[c] = xn[c];
             v[c] = vn[c];
-          }
-        }
-        // The new state in FP64 first: where the step is too long for the pairs by 1 % (their guard's
-        // eta^2 is good to 2^-20), or the distance out of their range, the look at it in pairs is
-        // saved.  (ADAPT: the next length is not known yet.)
-        double a_[3], j_[3];
-        bpl_fp64_eval<N>(P.fk, x, v, m, g, a_, j_, rd);
-        fp64 = true;
-        if (kind == 0)
-#pragma unroll
-          for (int c = 0; c < 3; c++) {
             an[c] = a_[c];
             jn[c] = j_[c];
           }
-        const float q = f_from(rd.q2), y = rsqrtf(q);
-        const float eta2 = ADAPT ? 0.0f : P.fc.hf * P.fc.hf * (g.m0f.h + g.mf.h) * y * y * y;
-        const bool far = eta2 > 1.01f * kFFEta2 || q > 0x1.04p40f || q < 0x1.f8p-41f;
-        clear = (__ballot_sync(FULL, b != 0 && far) & gm) != 0 && kind == 0;
+        }
       }
     }
     // Level 2: phase 0 evaluates the prediction and corrects it (spl_hermite_delta_step); then,
@@ -842,18 +957,8 @@ __device__ __forceinline__ void bpl_hermite_run(const BinView &B, const StepPara
             dn[c] = 0.0f;
           }
       }
-      const bool nf = nonfinite(x[0]) | nonfinite(x[1]) | nonfinite(x[2]) | nonfinite(v[0]) | nonfinite(v[1]) |
-                      nonfinite(v[2]);
-      const double q2 = rd.q2;
-      const bool ej = (b != 0) && (P.eject2 > 0.0) && (q2 > P.eject2);
-      bool ce = false;
-      for (int r = 1; r <= rt; r++) {
-        int p = b + r;
-        if (p >= n) p -= n;
-        const double q2p = shfl(q2, g.base + p);
-        const double kc = rd.kcr(r);
-        if (kc > 0.0 && close_encounter(P.fk, rd.d2r(r), kc, q2, q2p)) ce = true;
-      }
+      bool nf, ej, ce;
+      bpl_fp64_monitor<N>(P, g, x, v, rd, nf, ej, ce);
       const unsigned bnf = __ballot_sync(FULL, alive && (nf || bad)) & gm;
       const unsigned bej = __ballot_sync(FULL, active && ej) & gm;
       const unsigned bce = __ballot_sync(FULL, active && ce) & gm;
@@ -871,7 +976,8 @@ __device__ __forceinline__ void bpl_hermite_run(const BinView &B, const StepPara
       }
       level = lv;
       h = hn;
-      steps++;
+      if (kind) known = false;
+      steps += done;
       if (ADAPT) t = last ? te : kadd(P.fk, t, hd);
     }
     const bool reached = active && last && !code;

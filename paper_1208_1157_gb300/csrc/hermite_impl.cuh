@@ -253,9 +253,10 @@ __device__ __noinline__ void spl_hermite_adaptive_unit(const BinView &B, const S
 // so registers are allocated for this n alone.  Warps pull unit indices from a counter.
 // Body per lane: three CTAs per SM, or two where the step's latency is all that counts, up to
 // four bodies (a bin that fills the chip runs system per lane) and observations on the way
-// (without the spills 1024 x 3 systems over 400 steps take 1.88 instead of 1.92 ms).
+// (without the spills 1024 x 3 systems over 400 steps take 1.88 instead of 1.92 ms).  P: its address
+// goes to functions out of line, and the loop is to read it from constant memory all the same.
 template <int MAP, int N, bool ADAPT = false, bool OBS = false>
-__global__ void __launch_bounds__(128, MAP == SWARM_MAP_BODY_PER_LANE && N > 4 && !OBS ? 3 : 2) hermite_uniform_kernel(BinView B, int nunits, StepParams P) {
+__global__ void __launch_bounds__(128, MAP == SWARM_MAP_BODY_PER_LANE && N > 4 && !OBS ? 3 : 2) hermite_uniform_kernel(BinView B, int nunits, const __grid_constant__ StepParams P) {
   if (ADAPT && MAP == SWARM_MAP_SYSTEM_PER_LANE) {  // work unit = system (per-lane refill)
     spl_hermite_adaptive_stream<N>(B, P);
     return;

@@ -6,7 +6,7 @@
 namespace swarm {
 
 template <bool ADAPT>
-__global__ void __launch_bounds__(kWideWarps * 32, 3) hermite_wide_kernel(BinView B, StepParams P) {
+__global__ void __launch_bounds__(kWideWarps * 32, 3) hermite_wide_kernel(BinView B, const __grid_constant__ StepParams P) {
   __shared__ double kc_s[kWideWarps][kWideRounds * 32];
   __shared__ double d2_s[kWideWarps][kWideRounds * 32];
   __shared__ float kcf_s[kWideWarps][kWideRounds * 32];
