@@ -700,7 +700,7 @@ static __device__ __noinline__ int spl_hermite_fp64_run(const F64k &kk, const do
     }
   return code;
 }
-constexpr int kFP64Run = 16;  // steps between two looks at the level (a look costs 1/8 of an FP64 step)
+constexpr int kStepRun = 16;  // FP64 steps between two looks at the level (a look costs 1/8 of one)
 
 // Evaluation at a state (x, v): a0, j0, the monitor's distances; returns the level, 0 for a state
 // that is not finite or that the pairs cannot hold.  Every state that comes from outside or from
@@ -761,6 +761,14 @@ static __device__ __noinline__ int spl_hermite_ff_step_call(const F64k &kk, cons
                                                      float (&q2)[N], float (&d2)[N][N], ff (&sa)[3], ff (&sj)[3]) {
   spl_hermite_ff_advance<N>(kk, F, C, n_corr, x, v, a0, da, j0);
   return spl_ff_state<N, STAR>(kk, F, hf, x, v, a0, da, j0, q2, d2, sa, sj);
+}
+
+template <int N>
+static __device__ __noinline__ int spl_hermite_delta_step_call(const F64k &kk, const FMass<N> &F, const FCoef &C, float hf,
+                                                        int n_corr, double (&x)[N][3], double (&v)[N][3],
+                                                        double (&a0)[N][3], float (&da)[N][3], ff (&j0)[N][3],
+                                                        float (&q2)[N], float (&d2)[N][N], ff (&sa)[3], ff (&sj)[3]) {
+  return spl_hermite_delta_step<N, false>(kk, F, C, hf, n_corr, x, v, a0, da, j0, q2, d2, sa, sj);
 }
 
 // The monitor (Algorithm 1) after a step in pairs to a state of the given level.  A state of

@@ -30,7 +30,17 @@ template <int N>
 __device__ __forceinline__ void spl_hermite_body(const BinView &B, const StepParams &P, int unit) {
   const bool printed = P.corr_form != 0;  // warp-uniform
   const int s = unit * 32 + (threadIdx.x & 31);
-  if (s >= B.S) return;
+  double t0 = 0.0;
+  LaunchPlan plan;
+  plan.N = 0;
+  if (s < B.S && B.status[s] <= SWARM_SYS_DONE) {
+    t0 = B.t[s];
+    plan = launch_plan(B, P, s, t0, true);
+    if (plan.N == 0) B.status[s] = SWARM_SYS_DONE;
+  }
+  const int Ns = plan.N;
+  const unsigned lanes = __ballot_sync(0xffffffffu, Ns > 0);  // those with a system to integrate
+  if (Ns == 0) return;
   const int SP = B.S_pad;
   double x[N][3], v[N][3], m[N];
 #pragma unroll
@@ -41,14 +51,6 @@ __device__ __forceinline__ void spl_hermite_body(const BinView &B, const StepPar
       x[i][c] = B.x[(size_t)(c * N + i) * SP + s];
       v[i][c] = B.v[(size_t)(c * N + i) * SP + s];
     }
-  }
-  const double t0 = B.t[s];
-  if (B.status[s] > SWARM_SYS_DONE) return;
-  const LaunchPlan plan = launch_plan(B, P, s, t0, true);
-  const int Ns = plan.N;
-  if (Ns == 0) {
-    B.status[s] = SWARM_SYS_DONE;
-    return;
   }
   const FLimits<N> L = flimits<N>(m, P.ce_factor, P.eject2);
   double Minv, Xc[3], Vc[3];
@@ -61,17 +63,38 @@ __device__ __forceinline__ void spl_hermite_body(const BinView &B, const StepPar
   int level = spl_ff_state_call<N, false>(P.fk, F, P.fc.hf, x, v, a0, da, j0, q2, d2, sa, sj);
   int k = 0, code = 0;  // steps done
   const int whole = plan.exact ? Ns : Ns - 1;
-  while (k < Ns) {
-    if (level == 2 && k < whole) {
-      k++;
-      level = spl_hermite_delta_step<N, false>(P.fk, F, P.fc, P.fc.hf, P.n_corr, x, v, a0, da, j0, q2, d2, sa, sj);
-      code = spl_ff_monitor<N>(P.fk, level, L, q2, d2, x, v, P.eject2);
-    } else if (level && k < whole) {
-      k++;
-      level = spl_hermite_ff_step_call<N, false>(P.fk, F, P.fc, P.fc.hf, P.n_corr, x, v, a0, da, j0, q2, d2, sa, sj);
-      code = spl_ff_monitor<N>(P.fk, level, L, q2, d2, x, v, P.eject2);
+  auto log = [&]() {
+    if (!code && P.log_interval > 0 && (k % P.log_interval) == 0) {
+      const double tk = step_time(plan, k, t0, P.dt);
+      spl_write<N>(B, s, m, x, v, Minv, Xc, Vc, tk - t0, &P, tk);
+    }
+  };
+  // kStepRun steps of the lanes in pairs, then as many of those in FP64: lanes of compact systems
+  // change back and forth, each at its own time, and one run of FP64 steps for all that wait costs
+  // the warp as much as one for a single lane.  131072 compact systems over 300 steps of 0.005 and
+  // 0.01 orbits: n = 3 87 and 103 ms with a run at once for each lane, now 57 and 53 (wholly FP64
+  // 28); n = 4 270 and 254, now 178 and 204 (55).  What is left is fetching three kinds of steps of
+  // 50 KB and more; widely spaced systems, all of one kind: n = 3 11 ms, n = 4 37.
+  while (__any_sync(lanes, k < Ns && !code)) {
+    if (!__any_sync(lanes, level == 1 && k < whole && !code)) {  // the loop that fits the instruction cache
+      for (int c = 0; c < kStepRun && level == 2 && k < whole && !code; c++) {
+        k++;
+        level = spl_hermite_delta_step<N, false>(P.fk, F, P.fc, P.fc.hf, P.n_corr, x, v, a0, da, j0, q2, d2, sa, sj);
+        code = spl_ff_monitor<N>(P.fk, level, L, q2, d2, x, v, P.eject2);
+        log();
+      }
     } else {
-      int count = k < whole ? min(whole - k, kFP64Run) : 1;
+      for (int c = 0; c < kStepRun && level && k < whole && !code; c++) {
+        k++;
+        level = level == 2 ? spl_hermite_delta_step_call<N>(P.fk, F, P.fc, P.fc.hf, P.n_corr, x, v, a0, da, j0, q2, d2, sa, sj)
+                           : spl_hermite_ff_step_call<N, false>(P.fk, F, P.fc, P.fc.hf, P.n_corr, x, v, a0, da, j0, q2, d2, sa, sj);
+        code = spl_ff_monitor<N>(P.fk, level, L, q2, d2, x, v, P.eject2);
+        log();
+      }
+    }
+    __syncwarp(lanes);
+    if ((level == 0 || k >= whole) && k < Ns && !code) {
+      int count = k < whole ? min(whole - k, kStepRun) : 1;
       if (P.log_interval > 0) count = min(count, P.log_interval - k % P.log_interval);
       const double h = k < whole ? P.dt : plan.h_last;
       double t = 0.0;
@@ -79,11 +102,7 @@ __device__ __forceinline__ void spl_hermite_body(const BinView &B, const StepPar
       code = printed ? spl_hermite_fp64_run<N, false, true>(P.fk, m, L.kc, P.eject2, h, P.n_corr, count, true, x, v, a0, j0, k, t, t, reached)
                      : spl_hermite_fp64_run<N, false, false>(P.fk, m, L.kc, P.eject2, h, P.n_corr, count, true, x, v, a0, j0, k, t, t, reached);
       if (!code && k < Ns && !printed) level = spl_ff_state_call<N, false>(P.fk, F, P.fc.hf, x, v, a0, da, j0, q2, d2, sa, sj);
-    }
-    if (code) break;
-    if (P.log_interval > 0 && (k % P.log_interval) == 0) {
-      const double tk = step_time(plan, k, t0, P.dt);
-      spl_write<N>(B, s, m, x, v, Minv, Xc, Vc, tk - t0, &P, tk);
+      log();
     }
   }
   const double tk = step_time(plan, k, t0, P.dt);
