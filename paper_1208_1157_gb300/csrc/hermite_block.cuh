@@ -162,7 +162,6 @@ __device__ __forceinline__ void block_energy(const double (&x)[3], const double 
 
 template <int N>
 __device__ __forceinline__ void bpl_hermite_block_stream(const BinView &B, const StepParams &P, double *sm) {
-  const bool printed = P.corr_form != 0;  // CTA-uniform
   using R = BlockRing<N>;
   constexpr int T = R::T;
   constexpr int G = R::G;
@@ -257,28 +256,17 @@ __device__ __forceinline__ void bpl_hermite_block_stream(const BinView &B, const
       vk[c] = fma(j0[c], C.h2_2, fma(a0[c], C.h, v[c]));
       Vb[c] = fma(j0[c], C.h2_12, fma(a0[c], C.hh, v[c]));
     }
-    PCoef PC;
-    if (printed) {
-      PC = pcoef(C.h);
+    const PCoef PC = pcoef(C.h);
 #pragma unroll
-      for (int c = 0; c < 3; c++) Xb[c] = fma(j0[c], PC.pj, fma(a0[c], PC.pa, xk[c]));
-    } else {
-#pragma unroll
-      for (int c = 0; c < 3; c++) Xb[c] = fma(a0[c], C.h2_12, fma(v[c], C.hh, x[c]));
-    }
+    for (int c = 0; c < 3; c++) Xb[c] = fma(j0[c], PC.pj, fma(a0[c], PC.pa, xk[c]));
     double q2, d2[RT];
     for (int ic = 0; ic < P.n_corr; ic++) {
       double ak[3], jk[3];
       block_accjerk<N, false>(P.fk, xk, vk, m, b, gbase, sm, ak, jk, q2, d2);
 #pragma unroll
       for (int c = 0; c < 3; c++) vk[c] = fma(-C.h2_12, jk[c], fma(C.hh, ak[c], Vb[c]));
-      if (printed) {
 #pragma unroll
-        for (int c = 0; c < 3; c++) xk[c] = fma(PC.cj, jk[c], fma(PC.ca, ak[c], Xb[c]));
-      } else {
-#pragma unroll
-        for (int c = 0; c < 3; c++) xk[c] = fma(-C.h2_12, ak[c], fma(C.hh, vk[c], Xb[c]));
-      }
+      for (int c = 0; c < 3; c++) xk[c] = fma(PC.cj, jk[c], fma(PC.ca, ak[c], Xb[c]));
     }
     double an[3], jn[3];
     block_accjerk<N, true>(P.fk, xk, vk, m, b, gbase, sm, an, jn, q2, d2);
