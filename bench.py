@@ -711,8 +711,8 @@ def run_ours(args):
                      "peak_kind": "measured DFMA-chain peak on this GPU (2 flops per DFMA), of measured",
                      "note": "the method's flops over the FP64 pipe's peak: the kernel keeps the state and the star's "
                              "pull in FP64 and forms the rest as pairs of FP32 numbers, so most of these flops do not "
-                             "run on the FP64 pipe and the fraction can exceed 1 (profiles/: that pipe is 57 % busy, "
-                             "the issue slots 58 %)",
+                             "run on the FP64 pipe and the fraction can exceed 1 (profiles/: that pipe is 60 % busy, "
+                             "the issue slots 65 %)",
                      "peak_clocks": peak_clocks,
                      "avg_launch_ms": launch_ms},
         "e2e": {"value": e2e_steps / e2e_wall, "unit": "system-steps/s", "h2d_bytes_per_step": bytes_io,

@@ -13,10 +13,11 @@
 // Bound: issue slots and the latency of their chains (n = 15: 7200 instructions and 41 FP64
 // ones per step of two systems, 0.52 issued per cycle and sub-partition, the FP64 pipe 18 %
 // busy), so three CTAs per SM (168 registers).  Per step of 5041 systems, wholly in FP64 ->
-// now: n = 3 6.5 -> 4.3 us, 5 20.7 -> 6.7, 8 52.3 -> 9.7, 11 89.4 -> 22.8, 15 120.8 -> 33.0
+// now: n = 3 6.5 -> 4.7 us, 5 20.7 -> 6.5, 8 52.3 -> 9.6, 11 89.4 -> 22.4, 15 120.8 -> 29.8
 // (packed over the CTA for n = 7, 11, 15 before); 65536 systems of 3..15 bodies over 100
-// steps: 69.2 -> 18.3 ms.  A step of 0.02 orbits (level 0), n = 8: 39.9 -> 56 us.
-// 2048 systems of 16..32 bodies (one per warp, n a run-time value) over 50 steps: 13.6 -> 4.7 ms.
+// steps: 69.2 -> 16.7 ms.  Steps of 0.02 orbits (level 0), 200 of them: 38400 x 8 52.3 -> 55.2 ms,
+// 300 x 8 3.82 -> 4.00.  2048 systems of 16..32 bodies (one per warp, n a run-time value) over 50
+// steps: 13.6 -> 2.65 ms.
 #pragma once
 #include "hermite_ff.cuh"
 #include "hermite_wide.cuh"
@@ -556,7 +557,7 @@ static __device__ __noinline__ int bpl_fp64_run(const StepParams &P, const BplBo
 // them (the other groups re-evaluate their unchanged state and keep what they have).
 // OBS (fixed steps): through the observation times P.t_obs in one launch, leaving the radial
 // velocity at each (12 observations 12 steps apart, 257 x 3 systems: 1.14 ms with a launch for
-// each, whose cold start costs as much as three steps, 0.95 in one).
+// each, whose cold start costs as much as three steps, 0.85 in one).
 template <int N, bool ADAPT, bool OBS, class Take>
 __device__ __forceinline__ void bpl_hermite_run(const BinView &B, const StepParams &P, BplRounds<N> &rd, float *kcf,
                                                 Take take) {

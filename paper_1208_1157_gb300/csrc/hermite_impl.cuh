@@ -21,11 +21,11 @@ namespace swarm {
 // X_cm moved by its velocity times the time elapsed.
 //
 // The steps are those of hermite_ff.cuh.  Bound: the FP64 pipe and the issue slots about
-// evenly (57 and 58 % at n = 3, two warps per sub-partition at 255 registers; a 3-warp build
+// evenly (60 and 65 % at n = 3, two warps per sub-partition at 255 registers; a 3-warp build
 // at 168 registers spills and misses the instruction cache: 9 % slower).  131072 x 3 systems
-// over 400 steps: 37.0 ms wholly in FP64 (413 FP64 slots per step, the pipe 97 % busy), 8.0 ms
-// with 50 FP64 and 3250 other instructions per step; 16384 x 4 over 400 steps 10.8 -> 4.1 ms;
-// steps of 0.003 and 0.02 orbits (levels 1 and 0), 100 of them: 9.5 -> 4.1 and 9.6 ms.
+// over 400 steps: 37.0 ms wholly in FP64 (413 FP64 slots per step, the pipe 97 % busy), 7.8 ms
+// with 47 FP64 and 3210 other instructions per step; widely spaced systems, 300 steps of 0.003 and 0.02
+// orbits (levels 1 and 0): 27.8 -> 11.1 and 28.3 -> 28.8 ms.
 template <int N>
 __device__ __forceinline__ void spl_hermite_body(const BinView &B, const StepParams &P, int unit) {
   const bool printed = P.corr_form != 0;  // warp-uniform

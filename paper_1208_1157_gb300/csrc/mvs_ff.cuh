@@ -23,7 +23,7 @@
 // CTAs per SM) and the latency of the drift's chain of 3200 instructions (a step of one system
 // alone: 6.6 us), so 168 registers for three warps per sub-partition (two: 1.31 ms for 40 steps of
 // 16384 systems, three: 1.18).  Before, wholly in FP64, -> now: 16384 Jacobi systems of 8 bodies
-// over 500 steps 24.8 -> 8.5 ms, 3001 DH systems of 3..15 bodies over 300 steps 12.2 -> 5.1 ms,
+// over 500 steps 24.8 -> 8.5 ms, 3001 DH systems of 3..15 bodies over 300 steps 12.2 -> 3.1 ms,
 // one system alone 9.9 -> 6.6 us per step (the former spread over a warp's idle groups).
 // A FP64 form of a part costs its warp as much as before: the drift 5 us, the accelerations 3 us.
 #pragma once
