@@ -15,7 +15,7 @@
 // busy), so three CTAs per SM (168 registers).  Per step of 5041 systems, wholly in FP64 ->
 // now: n = 3 6.5 -> 4.7 us, 5 20.7 -> 6.5, 8 52.3 -> 9.6, 11 89.4 -> 22.4, 15 120.8 -> 29.8
 // (packed over the CTA for n = 7, 11, 15 before); 65536 systems of 3..15 bodies over 100
-// steps: 69.2 -> 16.7 ms.  Steps of 0.02 orbits (level 0), 200 of them: 38400 x 8 52.3 -> 55.2 ms,
+// steps: 69.2 -> 16.6 ms.  Steps of 0.02 orbits (level 0), 200 of them: 38400 x 8 52.3 -> 55.2 ms,
 // 300 x 8 3.82 -> 4.00.  2048 systems of 16..32 bodies (one per warp, n a run-time value) over 50
 // steps: 13.6 -> 2.65 ms.
 #pragma once
@@ -435,7 +435,7 @@ __device__ __forceinline__ void bpl_fp64_monitor(const StepParams &P, const BplB
 // steps of hs, or (ADAPT) that one and then Eq. 5's.  Returns the steps taken, the same for every
 // group: before the count is full it ends at a state that a group has to look at, that the
 // monitor stops, or that needs no further step.  x, v, a, j and rd are then that state's, hs, ts and
-// last those of the step that led there, hnext (ADAPT) the next length.  clear: the state is
+// last those of the step that led there.  clear: the state is
 // beyond doubt one for FP64, since a step is too long for the pairs by 1 % (their guard's eta^2
 // is good to 2^-20), a distance out of their range, or (free) all of them are.
 // In registers from step to step (200 steps of 0.02 orbits, 300 x 8 bodies: 4.5 ms with the evaluation and
@@ -444,7 +444,7 @@ template <int N, bool ADAPT>
 static __device__ __noinline__ int bpl_fp64_run(const StepParams &P, const BplBody<N> &g, bool lane_ok, double m, bool mine,
                                                 bool free, int count, BplRounds<N> &rd, double (&xs)[3], double (&vs)[3],
                                                 double (&as)[3], double (&js)[3], double &hs, double &ts, double te,
-                                                bool &last, double &hnext, bool &clear) {
+                                                bool &last, bool &clear) {
   const F64k &k = P.fk;
   const unsigned FULL = 0xffffffffu, gm = g.mask();
   const bool printed = P.corr_form != 0;
@@ -544,7 +544,6 @@ static __device__ __noinline__ int bpl_fp64_run(const StepParams &P, const BplBo
   hs = h;
   ts = t;
   last = la;
-  hnext = hn;
   clear = cl;
   return s;
 }
@@ -603,8 +602,6 @@ __device__ __forceinline__ void bpl_hermite_run(const BinView &B, const StepPara
   plan.t_end = P.t_end;
   double t = 0.0, t0 = 0.0, te = 0.0;  // fixed steps: t is formed from t0 when needed
   ff h = ff_make(0.0f, 0.0f);          // ADAPT: length of the next step of a group in pairs
-  double h64 = 0.0;                    // and of a group in FP64, where it is known
-  bool known = false;
   g.m0 = 1.0;
   g.m0f = g.mf = ff_make(1.0f, 0.0f);
   g.mt = 0.0f;
@@ -722,7 +719,6 @@ __device__ __forceinline__ void bpl_hermite_run(const BinView &B, const StepPara
         }
         level = lv;
         h = hn;
-        known = false;
         t0 = t = B.t[s];
         steps = 0;
         const bool runnable = B.status[s] <= SWARM_SYS_DONE;
@@ -758,8 +754,8 @@ __device__ __forceinline__ void bpl_hermite_run(const BinView &B, const StepPara
         kind = 0;
       }
     } else {
-      double hs = kind ? ff_double(h) : h64;
-      if (__any_sync(FULL, alive && !kind && !known)) {
+      double hs = ff_double(h);
+      if (__any_sync(FULL, alive && !kind)) {
         const double e = bpl_fp64_eq5<N>(P, g, lane_ok, a0, j0);
         if (!kind) hs = e;
       }
@@ -776,7 +772,6 @@ __device__ __forceinline__ void bpl_hermite_run(const BinView &B, const StepPara
     const bool rest = __any_sync(FULL, active && kind != 2);
     double an[3], jn[3];
     float dn[3] = {0.0f, 0.0f, 0.0f};
-    int done = 1;
     bool fp64 = false, clear = false;
     if (rest) {  // groups of level 1, groups in FP64
       double xn[3], vn[3];
@@ -808,7 +803,7 @@ __device__ __forceinline__ void bpl_hermite_run(const BinView &B, const StepPara
           }
           count = __reduce_min_sync(FULL, c);
         }
-        double a_[3], j_[3], hx = hd, tx = t, hn64;
+        double a_[3], j_[3], hx = hd, tx = t;
         bool lx = last, cl;
 #pragma unroll
         for (int c = 0; c < 3; c++) {
@@ -817,8 +812,8 @@ __device__ __forceinline__ void bpl_hermite_run(const BinView &B, const StepPara
           a_[c] = a0[c];
           j_[c] = j0[c];
         }
-        done = bpl_fp64_run<N, ADAPT>(P, g, lane_ok, m, active && !kind, printed || !scaled, count, rd, xn, vn, a_, j_, hx, tx, te, lx,
-                                      hn64, cl);
+        const int done = bpl_fp64_run<N, ADAPT>(P, g, lane_ok, m, active && !kind, printed || !scaled, count, rd, xn, vn, a_, j_,
+                                                hx, tx, te, lx, cl);
         fp64 = true;
         const bool tm = (__ballot_sync(FULL, !ff_tame(xn, vn)) & gm) == 0;
         if (active && !kind) {
@@ -828,11 +823,10 @@ __device__ __forceinline__ void bpl_hermite_run(const BinView &B, const StepPara
             hd = hx;
             t = tx;
             last = lx;
-            h64 = hn64;
-            known = true;
           } else {
             last = steps + done == plan.N;
           }
+          steps += done - 1;
 #pragma unroll
           for (int c = 0; c < 3; c++) {
             x[c] = xn[c];
@@ -977,8 +971,7 @@ __device__ __forceinline__ void bpl_hermite_run(const BinView &B, const StepPara
       }
       level = lv;
       h = hn;
-      if (kind) known = false;
-      steps += done;
+      steps++;
       if (ADAPT) t = last ? te : kadd(P.fk, t, hd);
     }
     const bool reached = active && last && !code;
