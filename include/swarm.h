@@ -131,7 +131,8 @@ typedef struct swarm_ensemble swarm_ensemble;
 typedef struct {
   int64_t system_steps;       /* steps taken, summed over systems */
   int64_t pair_evaluations;   /* unique-pair force evaluations (Hermite: 3 per pair per step) */
-  int64_t kepler_iterations;  /* Newton iterations of all Kepler drifts (MVS) */
+  int64_t kepler_iterations;  /* Newton iterations of all Kepler drifts (MVS); one for a drift whose
+                                 root is evaluated once and corrected to third order */
   int64_t kernel_launches;    /* kernels launched by the call */
   double kernel_ms;           /* device time of the call's kernels (CUDA events) */
 } swarm_stats;
